@@ -152,12 +152,20 @@ class Plan:
             self._h = None
 
 
+# The current device's current stream and device pointers as plain integers:
+# torch.cuda.current_stream() builds a Stream object (10 us on a Grace core,
+# as much as the rest of a contraction's forward on the host); the raw getter
+# is the same query without the object.
+_raw_stream = torch._C._cuda_getCurrentRawStream
+_cur_device = torch._C._cuda_getDevice
+
+
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(_cur_device())
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _precision(dtype):
@@ -337,11 +345,17 @@ def split_plan(S, leg, parts, precision=BF16X3):
     return _transform_plan(key, make)
 
 
+_sym_contract = L.lib.sym_contract
+_sym_contract_backward = L.lib.sym_contract_backward
+
+
 class _Contract(torch.autograd.Function):
     @staticmethod
     def forward(ctx, plan, a, b):
-        c = torch.empty(plan.c_numel, dtype=a.dtype, device=a.device)
-        L.check(L.lib.sym_contract(plan._h, _ptr(a), _ptr(b), _ptr(c), _stream()))
+        c = a.new_empty(plan.c_numel)
+        rc = _sym_contract(plan._h, a.data_ptr(), b.data_ptr(), c.data_ptr(), _raw_stream(_cur_device()))
+        if rc:
+            L.check(rc)
         ctx.plan = plan
         ctx.save_for_backward(a, b)
         return c
@@ -352,8 +366,10 @@ class _Contract(torch.autograd.Function):
         dc = dc.contiguous()
         da = torch.empty_like(a) if ctx.needs_input_grad[1] else None
         db = torch.empty_like(b) if ctx.needs_input_grad[2] else None
-        L.check(L.lib.sym_contract_backward(ctx.plan._h, _ptr(a), _ptr(b), _ptr(dc), _ptr(da), _ptr(db),
-                                            _stream()))
+        rc = _sym_contract_backward(ctx.plan._h, a.data_ptr(), b.data_ptr(), dc.data_ptr(), _ptr(da), _ptr(db),
+                                    _raw_stream(_cur_device()))
+        if rc:
+            L.check(rc)
         return None, da, db
 
 
