@@ -526,7 +526,7 @@ KERNEL_SOURCES = {
     "gemm_tc": ["gemm_tc.cu", "kernels.h", "pdl.h"],
     "gemm_tile": ["gemm_simt.cu", "kernels.h", "pdl.h"], "gemm_wide": ["gemm_simt.cu", "kernels.h", "pdl.h"],
     "gemm_thin": ["gemm_simt.cu", "kernels.h", "pdl.h"], "gemm_rows": ["gemm_simt.cu", "kernels.h", "pdl.h"],
-    "direct": ["direct.cu", "kernels.h", "pdl.h"],
+    "direct": ["direct.cu", "kernels.h", "pdl.h"], "block": ["block.cu", "kernels.h", "pdl.h"],
     "svd_jacobi": ["svd.cu"],
 }
 

@@ -257,7 +257,8 @@ int sym_plan_profile_read(sym_plan plan, int phase, int* launches,
 #define SYM_KERNEL_GEMM_THIN 5 /* CUDA cores, m, n <= 8, split reduction */
 #define SYM_KERNEL_GEMM_ROWS 6 /* CUDA cores, k, n <= 16 */
 #define SYM_KERNEL_DIRECT 7    /* sectors with a tiny matrix, contracted on the blocks */
-#define SYM_KERNEL_COUNT 8
+#define SYM_KERNEL_BLOCK 8     /* CUDA cores, on the blocks themselves (no matrix form) */
+#define SYM_KERNEL_COUNT 9
 int sym_plan_profile_kernel(sym_plan plan, int kernel, int* launches,
                             double* total_ms, double* bytes, double* flops);
 

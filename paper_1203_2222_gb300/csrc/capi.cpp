@@ -296,33 +296,38 @@ int sym_contract_batch_plan(int nprob, const sym_tensor* A, const sym_tensor* B,
     const std::vector<int> pa(pairsA, pairsA + npairs), pb(pairsB, pairsB + npairs);
     std::vector<sym::Tensor> Ct(nprob);
     std::vector<std::unique_ptr<sym::Plan>> ps(nprob);
+    std::vector<int64_t> oa(nprob + 1, 0), ob(nprob + 1, 0), oc(nprob + 1, 0);
     // the problems are planned independently, on up to 16 host threads
-    std::atomic<int> next{0};
-    std::exception_ptr err;
-    std::mutex emu;
-    auto work = [&] {
-      for (int i = next++; i < nprob; i = next++) {
-        try {
-          Ct[i] = sym::contraction_result(A[i]->t, B[i]->t, pa, pb, nullptr);
-          ps[i] = sym::plan_contract(A[i]->t, B[i]->t, pa, pb, Ct[i], precision, /*device=*/false);
-        } catch (...) {
-          std::lock_guard<std::mutex> lk(emu);
-          if (!err) err = std::current_exception();
+    auto plan_all = [&](bool blocks) {
+      std::atomic<int> next{0};
+      std::exception_ptr err;
+      std::mutex emu;
+      auto work = [&] {
+        for (int i = next++; i < nprob; i = next++) {
+          try {
+            Ct[i] = sym::contraction_result(A[i]->t, B[i]->t, pa, pb, nullptr);
+            ps[i] = sym::plan_contract(A[i]->t, B[i]->t, pa, pb, Ct[i], precision, /*device=*/false, blocks, nprob);
+          } catch (...) {
+            std::lock_guard<std::mutex> lk(emu);
+            if (!err) err = std::current_exception();
+          }
         }
+      };
+      const int nth = std::max(1, std::min({nprob, 16, (int)std::thread::hardware_concurrency()}));
+      std::vector<std::thread> pool;
+      for (int t = 1; t < nth; ++t) pool.emplace_back(work);
+      work();
+      for (auto& t : pool) t.join();
+      if (err) std::rethrow_exception(err);
+      for (int i = 0; i < nprob; ++i) {
+        oa[i + 1] = oa[i] + A[i]->t.numel();
+        ob[i + 1] = ob[i] + B[i]->t.numel();
+        oc[i + 1] = oc[i] + Ct[i].numel();
       }
     };
-    const int nth = std::max(1, std::min({nprob, 16, (int)std::thread::hardware_concurrency()}));
-    std::vector<std::thread> pool;
-    for (int t = 1; t < nth; ++t) pool.emplace_back(work);
-    work();
-    for (auto& t : pool) t.join();
-    if (err) std::rethrow_exception(err);
-    std::vector<int64_t> oa(nprob + 1, 0), ob(nprob + 1, 0), oc(nprob + 1, 0);
-    for (int i = 0; i < nprob; ++i) {
-      oa[i + 1] = oa[i] + A[i]->t.numel();
-      ob[i + 1] = ob[i] + B[i]->t.numel();
-      oc[i + 1] = oc[i] + Ct[i].numel();
-    }
+    plan_all(true);
+    // the block kernel addresses the packed tensors with 32-bit offsets
+    if (std::max({oa[nprob], ob[nprob], oc[nprob]}) >= (int64_t)1 << 31) plan_all(false);
     auto M = sym::merge_contract_plans(ps, oa, ob, oc);
     for (int i = 0; i <= nprob; ++i) {
       offsets[i] = oa[i];
@@ -461,6 +466,7 @@ int sym_plan_gemm_shapes(sym_plan plan, int* nsec, int* mnk) {
     std::vector<std::array<int, 4>> v;
     for (const auto& s : p.secs_tc) v.push_back({s.m, s.n, s.k, 0});
     for (const auto& s : p.secs_simt) v.push_back({s.m, s.n, s.k, 1});
+    for (const auto& s : p.blk_mnk) v.push_back({s[0], s[1], s[2], 1});
     if (mnk)
       for (size_t i = 0; i < v.size(); ++i)
         for (int j = 0; j < 4; ++j) mnk[4 * i + j] = v[i][j];

@@ -178,6 +178,68 @@ struct DirectItem {
 static_assert(sizeof(DirectCol) == 24, "DirectCol layout");
 static_assert(sizeof(DirectItem) == 512, "DirectItem layout");
 
+// Block contraction (block.cu): the product is taken on the tensors' blocks
+// themselves, out(r, c) = sum over segments, sum_k coef * P(r, k) * Q(k, c),
+// with no matrix form of any operand.  An output block is m x n: its legs
+// split into the row legs (shared with P) and the column legs (shared with
+// Q), each side at most kBlkDims dims after merging (last fastest).  A
+// segment is one pair of operand blocks (with its recoupling coefficient or
+// swap sign); its reduction is the box of the contracted legs.  All offsets
+// inside a block stay below 2^31 (host check).
+constexpr int kBlkDims = 3;
+struct BlkSeg {
+  int64_t p_off, q_off;
+  double coef;
+  int32_t k0, kn;               // first position and extent of this segment in the output block's reduction
+  int32_t kd[kBlkDims - 1];     // sizes of the reduction's dims 1 and 2
+  uint32_t kmag[kBlkDims - 1];  // division by them (as in BoxItem)
+  int32_t kshf;                 // the two shifts, one byte each
+  int32_t pk[kBlkDims], qk[kBlkDims];  // strides of the reduction dims in P and Q
+  int32_t pr[kBlkDims], qc[kBlkDims];  // strides of the row dims in P, of the column dims in Q
+  float coef_f;                        // coef rounded to FP32
+};
+static_assert(sizeof(BlkSeg) == 104, "BlkSeg layout");
+struct BlkOut {
+  int64_t off;
+  int32_t m, n, ktot, seg0, nseg;
+  int32_t slots;  // bits 0-1 slot of P, 2-3 slot of Q (0 A, 1 B, 2 dC), 4-6 destination slot
+  int32_t flags;  // kBlkPk: lanes run along the reduction when P is read (else along the rows), kBlkQk: same for Q
+  int32_t rd[kBlkDims - 1], cd[kBlkDims - 1];
+  uint32_t rmag[kBlkDims - 1], cmag[kBlkDims - 1];
+  int32_t shf;    // row shifts in bytes 0-1, column shifts in bytes 2-3
+  int32_t ro[kBlkDims], co[kBlkDims];  // strides of the row and column dims in the output
+};
+static_assert(sizeof(BlkOut) == 96, "BlkOut layout");
+constexpr int kBlkPk = 1, kBlkQk = 2, kBlkCoef = 4;  // kBlkCoef: some segment's coefficient is not 1
+// Tile shapes (rows x columns, reduction steps a slab): the FP32 / FP64 sizes
+// are below; BLK_DOT has no tile in shared memory (a thread per reduction step).
+constexpr int kBlkThreads = 128;
+enum BlkShape { BLK_BIG = 0, BLK_MID = 1, BLK_SMALL = 2, BLK_TALL = 3, BLK_DOT = 4, BLK_SHAPES = 5 };
+SYM_HD constexpr int blk_rows(bool f64, int shape) {
+  return shape == BLK_BIG ? (f64 ? 32 : 64) : shape == BLK_MID ? (f64 ? 24 : 48) : shape == BLK_SMALL ? (f64 ? 16 : 32)
+         : shape == BLK_TALL ? (f64 ? 128 : 256) : 8;
+}
+SYM_HD constexpr int blk_cols(bool f64, int shape) {
+  return shape <= BLK_MID ? (f64 ? 32 : 64) : shape == BLK_SMALL ? (f64 ? 16 : 32) : 8;
+}
+SYM_HD constexpr int blk_slab(bool f64, int shape) {
+  return shape <= BLK_MID ? 16 : shape == BLK_SMALL ? (f64 ? 16 : 32) : shape == BLK_TALL ? 8 : kBlkThreads;
+}
+// One unit of work: a tile of an output block, over slabs [s0, s1) of its
+// reduction.  A tile cut into nparts > 1 parts adds them up in workspace slots
+// ws .. ws + nparts - 1 (kBlkSlot elements each): the part that arrives last
+// (counter cnt) sums them in order, writes the tile and clears the counter.
+constexpr int kBlkSlot = 4096;
+struct BlkTile {
+  BlkOut ob;      // with the segments of [s0, s1) only
+  int32_t r0, c0;
+  int32_t shape;
+  int32_t s0, s1;
+  int32_t part;   // part index in the low half, nparts in the high half
+  int32_t ws, cnt;
+};
+static_assert(sizeof(BlkTile) == 128, "BlkTile layout");
+
 // CUDA-core GEMM tile shapes
 enum SimtShape { SIMT_64x64 = 0, SIMT_256x16 = 1, SIMT_THIN = 2, SIMT_ROWS = 3, SIMT_SHAPES = 4 };
 
@@ -192,6 +254,8 @@ int launch_gemm_simt(bool f64, int shape, const GemmSectorSimt* secs, const Gemm
                      const void* ops, void* outm, void* stream);
 // every item of [items, items + nitems) must have op == `op`
 int launch_direct(bool f64, int op, const DirectItem* items, int nitems, const BoxPtrs& ptrs, void* stream);
+int launch_block(bool f64, const BlkTile* tiles, int ntiles, const BlkSeg* segs, void* ws, int* counters,
+                 const BoxPtrs& ptrs, void* stream);
 int launch_gemm_tc(const TcSector* secs, const GemmTile* tiles, int ntiles, const TensorMap* maps, float* C,
                    int* err_word, void* stream);
 // One bounded mbarrier wait that nothing completes (a test of the expiry

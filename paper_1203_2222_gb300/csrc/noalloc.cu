@@ -126,7 +126,7 @@ extern "C" int sym_contract_noalloc(sym_tensor A, sym_tensor B, int npairs, cons
     auto it = g_plans.find(key);
     if (it == g_plans.end()) {
       Tensor Ct = contraction_result(A->t, B->t, pa, pb, nullptr);
-      auto plan = plan_contract(A->t, B->t, pa, pb, Ct, precision, /*device=*/false);
+      auto plan = plan_contract(A->t, B->t, pa, pb, Ct, precision, /*device=*/false, /*blocks=*/false);
       plan->concurrent = false;  // no side streams or events: launch the GEMM kinds in order
       if (g_plans.size() >= kMaxPlans) {
         g_plans.erase(g_order.front());

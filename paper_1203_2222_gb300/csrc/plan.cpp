@@ -83,16 +83,6 @@ Box simplify(const Box& in) {
   return b;
 }
 
-// Magic numbers for dividing 31-bit dividends by d >= 1 with one multiply-high
-// (Granlund & Montgomery, PLDI 1994, Thm 4.2 with N = 31):
-// s = ceil(log2 d), m = ceil(2^(31+s) / d) < 2^32, floor(a / d) = (2a * m) >> (32 + s).
-void div_magic(int d, uint32_t& m, int8_t& s) {
-  int l = 0;
-  while (((int64_t)1 << l) < d) ++l;
-  m = (uint32_t)((((uint64_t)1 << (31 + l)) + (uint64_t)d - 1) / (uint64_t)d);
-  s = (int8_t)l;
-}
-
 BoxItem make_item(const Box& box, int64_t dst_off, int dst_ld, int sel, int term0,
                   const std::vector<Term>& terms) {
   BoxItem it{};
@@ -759,8 +749,14 @@ void Plan::upload(bool device) {
   d_secs_tc = static_cast<TcSector*>(up(secs_tc.data(), secs_tc.size() * sizeof(TcSector)));
   d_tiles = static_cast<GemmTile*>(up(tiles.data(), tiles.size() * sizeof(GemmTile)));
   d_ditems = static_cast<DirectItem*>(up(ditems.data(), ditems.size() * sizeof(DirectItem)));
+  d_bsegs = static_cast<BlkSeg*>(up(bsegs.data(), bsegs.size() * sizeof(BlkSeg)));
+  d_btiles = static_cast<BlkTile*>(up(btiles.data(), btiles.size() * sizeof(BlkTile)));
   if (kind == CONTRACT) {
     const size_t es = f64() ? sizeof(double) : sizeof(float);
+    if (blk_slots > 0) {
+      blk_ws = arena.alloc((size_t)blk_slots * kBlkSlot * es, false);
+      d_blk_cnt = static_cast<int*>(arena.alloc((size_t)blk_counters * sizeof(int), true));
+    }
     if (img_elems > 0) {  // hi and lo planes; the TMA loads fill past-the-edge boxes with zeros
       img = arena.alloc(img_elems * 2 * 2, false);
       encode_maps(img);
@@ -1311,8 +1307,118 @@ void validate_direct(const Plan& P) {
   }
 }
 
+namespace {
+
+// The kernel-choice parameters as the library ships them: only then does the
+// planner choose between matrix form and the block kernel itself; a caller
+// (the autotuner, a test) that changed one gets the kernels it asked for.
+bool default_kernel_choice(const sym_tune& t) {
+  return t.tc_min_mn == 64 && t.tc_min_k == 48 && t.tc_max_k == 16384 && t.direct_max == kMaxDirect &&
+         t.direct_mixed == 1 && t.tc_all == 0;
+}
+
+// Every product of blocks a contraction sums, with its coefficient (swap
+// signs; SU(2): the recoupling sums on both operands and on the result
+// multiplied out).  False when there are too many for the work lists, or when
+// multiplying the recoupling sums out more than doubles the arithmetic.
+constexpr int64_t kMaxTriples = 200000;
+bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const MatForm& MA, const MatForm& MB, int na,
+                   int nc, const std::vector<TermList>& XA, const std::vector<TermList>& XB,
+                   const std::vector<TermList>& XCt, bool natural, std::vector<BlkTriple>* out) {
+  using Key = std::pair<int, std::vector<int>>;
+  std::map<Key, std::vector<int64_t>> brow;  // (x, contracted labels) -> sectors of B
+  for (int64_t s = 0; s < Bm.nsec(); ++s) brow[{MB.xs[MB.sx[s]], row_key(Bm, s, nc)}].push_back(s);
+  int64_t count = 0;
+  double work = 0.0, useful = 0.0;
+  struct Pair {
+    int64_t a, b;
+  };
+  std::vector<Pair> pairs;
+  for (int64_t s = 0; s < Am.nsec(); ++s) {
+    auto it = brow.find({MA.xs[MA.sx[s]], col_key(Am, s, na)});
+    if (it == brow.end()) continue;
+    for (int64_t b : it->second) {
+      pairs.push_back({s, b});
+      if ((int64_t)pairs.size() > kMaxTriples) return false;
+    }
+  }
+  const bool tree = su2_like(Am.group);
+  std::map<std::array<int64_t, 3>, double> sum;  // SU(2): products met through several intermediate labels
+  std::vector<int> key;
+  for (const Pair& p : pairs) {
+    key.assign(Am.pos.begin() + p.a * Am.rank, Am.pos.begin() + p.a * Am.rank + na);
+    key.insert(key.end(), Bm.pos.begin() + p.b * Bm.rank + nc, Bm.pos.begin() + (p.b + 1) * Bm.rank);
+    if (tree) {  // node spins of the joined tree: A's row nodes, then B's column nodes
+      std::vector<int> ra = row_key(Am, p.a, na), cb = col_key(Bm, p.b, nc);
+      const int nb = Bm.rank - nc, k = Cn.rank;
+      std::vector<int> inner;
+      const int x = su2_top(Am, p.a, na);
+      if (na >= 2) {
+        inner.insert(inner.end(), ra.begin() + na, ra.end());
+        if (nb >= 1) inner.push_back(x);
+      }
+      if (nb >= 2) {
+        inner.insert(inner.end(), cb.begin() + nb, cb.end());
+        if (na >= 1) inner.push_back(x);
+      }
+      if ((int)inner.size() != std::max(k - 2, 0)) return false;
+      key.insert(key.end(), inner.begin(), inner.end());
+    }
+    const int64_t c = Cn.find(key);
+    if (c < 0) return false;
+    double mnk = 1.0;
+    for (int l = 0; l < Am.rank; ++l) mnk *= Am.dim(p.a, l);
+    for (int l = nc; l < Bm.rank; ++l) mnk *= Bm.dim(p.b, l);
+    useful += mnk;
+    for (auto& xa : XA[p.a])
+      for (auto& xb : XB[p.b]) {
+        if (!tree) {
+          out->push_back({xa.first, xb.first, c, xa.second * xb.second});
+        } else if (natural) {
+          sum[{xa.first, xb.first, c}] += xa.second * xb.second;
+        } else {
+          for (auto& xc : XCt[c]) sum[{xa.first, xb.first, xc.first}] += xa.second * xb.second * xc.second;
+        }
+        if (++count > kMaxTriples) return false;
+      }
+    if (tree) work += mnk * (double)XA[p.a].size() * (double)XB[p.b].size() * (natural ? 1.0 : (double)XCt[c].size());
+  }
+  if (tree) {
+    if (work > 4.0 * useful) return false;
+    for (auto& t : sum)
+      if (std::fabs(t.second) > 1e-13) out->push_back({t.first[0], t.first[1], t.first[2], t.second});
+  }
+  return true;
+}
+
+// Modelled time of one phase in matrix form: the moves in and out of matrix
+// form at 3 TB/s, the GEMM kernels, and per phase 40 us for its three to six
+// launches and their side streams (15 us on the device, 25 us more on the host,
+// which is what bounds a chain of small contractions).
+double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, double share) {
+  const double es = f64 ? 8.0 : 4.0;
+  double bytes = 0.0, tc = 0.0, tclat = 0.0, simt = 0.0;
+  for (auto& s : mnk) {
+    const double m = (double)s[0], n = (double)s[1], k = (double)s[2];
+    bytes += 2.0 * es * (m * k + k * n + m * n);
+    if (s[3] == 0) {
+      const double kt = std::ceil(k / 64.0), t = 0.55 * kt + 2.0;
+      tc += std::ceil(m / 128.0) * std::ceil(n / 128.0) * t / 152.0;
+      tclat = std::max(tclat, t);
+    } else if (s[3] >= 3) {
+      bytes += es * (m * k + k * n + m * n);
+    } else {
+      simt += 2.0 * m * n * k;
+    }
+  }
+  return 40.0 * share + bytes / 3.0e6 + std::max(tc, tclat * share) + simt / (f64 ? 0.4e6 : 10e6);
+}
+
+}  // namespace
+
 std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std::vector<int>& pairsA,
-                                    const std::vector<int>& pairsB, const Tensor& C, int precision, bool device) {
+                                    const std::vector<int>& pairsB, const Tensor& C, int precision, bool device,
+                                    bool blocks, int nbatch) {
   auto P = std::make_unique<Plan>();
   P->kind = Plan::CONTRACT;
   P->precision = precision;
@@ -1432,6 +1538,46 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     gs.push_back(g);
   }
 
+  for (auto& g : gs) P->flops_fwd += 2.0 * (double)g.m * (double)g.n * (double)g.k;
+  P->numel_a = A.numel();
+  P->numel_b = B.numel();
+  P->numel_c = C.numel();
+
+  // ---- phases that run on the blocks themselves (block.cu)
+  const bool all_direct = !su2 && C.nsec() == Cn.nsec() &&
+                          std::all_of(gs.begin(), gs.end(), [&](const G& g) {
+                            return g.k <= tp.direct_max && g.n <= tp.direct_max;
+                          });
+  if (blocks && !all_direct && default_kernel_choice(tp)) {
+    std::vector<BlkTriple> triples;
+    if (block_triples(Am, Bm, Cn, MA, MB, na, nc, XA, XB, XCt, natural, &triples)) {
+      // all three phases or none: the matrix form shares its gathers between them
+      const double share = 1.0 / std::max(nbatch, 1);
+      double blk_us = 0.0, mat_us = 0.0;
+      bool ok = true;
+      for (int ph = 0; ph < 3 && ok; ++ph) {
+        std::vector<std::array<int64_t, 4>> mnk;  // the phase's GEMMs in matrix form, with their kernel kinds
+        for (auto& g : gs)
+          mnk.push_back(ph == 0 ? std::array<int64_t, 4>{g.m, g.n, g.k, g.kind[0]}
+                                : ph == 1 ? std::array<int64_t, 4>{g.m, g.k, g.n, g.kind[1]}
+                                          : std::array<int64_t, 4>{g.k, g.n, g.m, g.kind[2]});
+        double us = 0.0;
+        ok = plan_block_phase(*P, ph, A, B, C, triples, freeA, freeB, pairsA, pairsB, share, &us);
+        blk_us += us;
+        mat_us += matrix_form_us(f64, mnk, share);
+        P->blk_flops[ph] = P->flops_fwd;
+        for (size_t i = 0; i < gs.size(); ++i)
+          if (su2 || gs[i].k > tp.direct_max || gs[i].n > tp.direct_max)  // tiny sectors are no GEMMs
+            P->blk_mnk.push_back({(int)mnk[i][0], (int)mnk[i][1], (int)mnk[i][2]});
+      }
+      // in a batch the matrix form's launches run for the other problems anyway:
+      // taking some problems out of them pays only where the blocks win clearly
+      // (128 two-site problems: 2.35 ms in matrix form, 2.47 ms at a factor of 1)
+      P->blocks = ok && blk_us < mat_us * (nbatch > 1 ? 0.5 : 1.0);
+      if (!P->blocks) drop_blocks(*P);
+    }
+  }
+
   // ---- direct sectors (U(1), B_x at most kMaxDirect x kMaxDirect): the
   // product runs on A's and C's blocks (kernels.h, DirectItem).  Such sectors
   // leave gs: no matrix form, GEMM, gather or scatter of their own (the dB
@@ -1439,7 +1585,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   std::set<int> dset;
   std::vector<DirectItem> dfw, dba, dbb;
   int rw[kMaxDim], cw[kMaxDim], st[kMaxDim];
-  if (!su2 && C.nsec() == Cn.nsec()) {
+  if (!su2 && C.nsec() == Cn.nsec() && !P->blocks) {
     const int dmax = tp.direct_max;
     std::map<int, std::map<std::vector<int>, std::vector<int64_t>>> arow, crow;  // x -> row key -> sectors
     std::map<int, std::vector<int64_t>> bsec;                                   // x -> Bm sectors
@@ -1676,7 +1822,6 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     for (auto& g : gs) {
       if (use && g.k <= dmax && g.n <= dmax && plan_direct(g)) {
         dset.insert(g.x);
-        P->flops_fwd += 2.0 * (double)g.m * (double)g.n * (double)g.k;
       } else {
         keep.push_back(g);
       }
@@ -1704,6 +1849,10 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     P->tc_ops.push_back(TcOperand{off, (int)rows, (int)cols, (int)ld64(cols), mn});
     return (int)P->tc_ops.size() - 1;
   };
+  if (P->blocks) {  // nothing in matrix form
+    gs.clear();
+    gofx.clear();
+  }
   for (auto& g : gs) {
     const bool t0 = g.kind[0] == 0, t1 = g.kind[1] == 0, t2 = g.kind[2] == 0;
     if (t0 || t2) g.ta = add_buf(g.m, g.k);
@@ -1744,10 +1893,6 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   P->img_elems = cdiv(ie, 64) * 64;  // the lo plane starts 128-byte aligned
   P->lin_elems = le;
   P->outm_elems = oe;
-  for (auto& g : gs) P->flops_fwd += 2.0 * (double)g.m * (double)g.n * (double)g.k;
-  P->numel_a = A.numel();
-  P->numel_b = B.numel();
-  P->numel_c = C.numel();
 
   // ---- GEMM sectors and tiles: lists per (kind, gemm phase)
   std::vector<std::pair<int64_t, GemmTile>> lists[kGemmKinds][3];
@@ -1877,8 +2022,9 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   // ---- forward gather: A -> A operand, B -> B operand (+ zero fills)
   int begin = (int)P->items.size();
   std::vector<char> doneA;
+  const bool mf = !P->blocks;
   fuse_recoupling(
-      Am.nsec(), XA, 0,
+      mf ? Am.nsec() : 0, XA, 0,
       [&](int64_t s, OffLd& o, int& slot) {
         auto gi = gofx.find(MA.xs[MA.sx[s]]);
         if (gi == gofx.end()) return false;
@@ -1894,7 +2040,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
       },
       [&](int64_t sa) { return OffLd{A.offs[sa], 1}; },
       [&](int64_t s, int64_t sa) { return gather_box(A, pinvA, Am, s, sa, na, false); }, doneA);
-  for (int64_t s = 0; s < Am.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < Am.nsec(); ++s) {
     auto gi = gofx.find(MA.xs[MA.sx[s]]);
     if (gi == gofx.end() || XA[s].empty() || doneA[s]) continue;
     const G& g = gs[gi->second];
@@ -1904,7 +2050,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     else
       put(b, 0, g.a, MA.r0[s], MA.c0[s], g.k, terms_of(XA[s], A));
   }
-  for (int64_t s = 0; s < Bm.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < Bm.nsec(); ++s) {
     auto gi = gofx.find(MB.xs[MB.sx[s]]);
     if (gi == gofx.end() || XB[s].empty()) continue;
     const G& g = gs[gi->second];
@@ -1930,7 +2076,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     t.push_back({g.c + r0 * g.n + c0, g.n, coef});
   };
   begin = (int)P->items.size();
-  for (int64_t s = 0; s < C.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < C.nsec(); ++s) {
     if (natural && dset.count(MC.xs[MC.sx[s]])) continue;  // written by the direct kernel
     std::vector<Term> t;
     if (natural) {
@@ -1968,7 +2114,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     }
   };
   const int b0 = (int)P->items.size();
-  for (int64_t s = 0; s < Bm.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < Bm.nsec(); ++s) {
     auto gi = gofx.find(MB.xs[MB.sx[s]]);
     if (gi == gofx.end() || XB[s].empty()) continue;
     const G& g = gs[gi->second];
@@ -1992,7 +2138,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     if (g.dcl >= 0) put(b, 2, g.dcl, r0, c0, g.n, t);
   });
   const int b2 = (int)P->items.size();
-  for (int64_t s = 0; s < Am.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < Am.nsec(); ++s) {
     auto gi = gofx.find(MA.xs[MA.sx[s]]);
     if (gi == gofx.end() || XA[s].empty()) continue;
     const G& g = gs[gi->second];
@@ -2015,7 +2161,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   begin = (int)P->items.size();
   std::vector<char> doneDA;
   fuse_recoupling(
-      A.nsec(), XAt, 3,
+      mf ? A.nsec() : 0, XAt, 3,
       [&](int64_t s, OffLd& o, int& slot) {
         for (auto& pc : XAt[s])
           if (gofx.find(MA.xs[MA.sx[pc.first]]) == gofx.end()) return false;
@@ -2035,7 +2181,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
         return b;
       },
       doneDA);
-  for (int64_t s = 0; s < A.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < A.nsec(); ++s) {
     if (doneDA[s]) continue;
     bool direct = false;  // dA written by the direct kernel
     for (auto& pc : XAt[s]) direct = direct || dset.count(MA.xs[MA.sx[pc.first]]) > 0;
@@ -2062,7 +2208,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   split_few_recouple_items(*P, begin);
   P->bwd_scatter_a = {begin, (int)P->items.size() - begin};
   begin = (int)P->items.size();
-  for (int64_t s = 0; s < B.nsec(); ++s) {
+  for (int64_t s = 0; mf && s < B.nsec(); ++s) {
     std::vector<Term> t;
     int64_t sm0 = -1;
     for (auto& pc : XBt[s]) {
@@ -2094,6 +2240,7 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
   }
   validate_gemms(*P, f64);
   validate_direct(*P);
+  validate_blocks(*P);
   P->upload(device);
   return P;
 }
@@ -2241,6 +2388,71 @@ std::unique_ptr<Plan> merge_contract_plans(std::vector<std::unique_ptr<Plan>>& p
       *dst[r] = Range{first, (int)M->ditems.size() - first};
     }
   }
+  // block contraction lists, longest tiles first across problems
+  {
+    std::vector<int> seg0(n), out0(n);  // of problem i's lists in the merged ones
+    const int64_t* shifts[3] = {offA.data(), offB.data(), offC.data()};
+    for (int i = 0; i < n; ++i) {
+      const Plan& p = *ps[i];
+      seg0[i] = (int)M->bsegs.size();
+      out0[i] = (int)M->bouts.size();
+      std::vector<int> pslot(p.bsegs.size()), qslot(p.bsegs.size());
+      for (BlkOut b : p.bouts) {
+        const int os = (b.slots >> 4) & 7;
+        for (int j = b.seg0; j < b.seg0 + b.nseg; ++j) {
+          pslot[j] = b.slots & 3;
+          qslot[j] = (b.slots >> 2) & 3;
+        }
+        b.off += os == DST_OUT ? offC[i] : os == DST_DA ? offA[i] : offB[i];
+        b.seg0 += seg0[i];
+        M->bouts.push_back(b);
+      }
+      for (size_t j = 0; j < p.bsegs.size(); ++j) {
+        BlkSeg g = p.bsegs[j];
+        g.p_off += shifts[pslot[j]][i];
+        g.q_off += shifts[qslot[j]][i];
+        M->bsegs.push_back(g);
+      }
+      M->blk_mnk.insert(M->blk_mnk.end(), p.blk_mnk.begin(), p.blk_mnk.end());
+    }
+    std::vector<int> slot0(n), cnt0(n);
+    for (int i = 0; i < n; ++i) {
+      slot0[i] = M->blk_slots;
+      cnt0[i] = M->blk_counters;
+      M->blk_slots += ps[i]->blk_slots;
+      M->blk_counters += ps[i]->blk_counters;
+    }
+    for (int ph = 0; ph < 3; ++ph) {
+      struct Unit {
+        double cost;
+        BlkTile t;
+        int out;
+      };
+      std::vector<Unit> v;
+      for (int i = 0; i < n; ++i) {
+        const Plan& p = *ps[i];
+        M->blk_bytes[ph] += p.blk_bytes[ph];
+        M->blk_flops[ph] += p.blk_flops[ph];
+        for (int t = p.blk_range[ph].first; t < p.blk_range[ph].first + p.blk_range[ph].count; ++t) {
+          const int out = out0[i] + p.btile_out[t];
+          BlkTile b = p.btiles[t];
+          const BlkOut own = b.ob;
+          b.ob = M->bouts[out];
+          b.ob.seg0 = own.seg0 + seg0[i];
+          b.ob.nseg = own.nseg;
+          b.ws += slot0[i];
+          b.cnt += cnt0[i];
+          v.push_back({blk_tile_cost(f64, b), b, out});
+        }
+      }
+      std::stable_sort(v.begin(), v.end(), [](const Unit& a, const Unit& b) { return a.cost > b.cost; });
+      M->blk_range[ph] = Range{(int)M->btiles.size(), (int)v.size()};
+      for (auto& t : v) {
+        M->btiles.push_back(t.t);
+        M->btile_out.push_back(t.out);
+      }
+    }
+  }
   // GEMM tiles per (kind, phase), longest reductions first across problems
   for (int kind = 0; kind < kGemmKinds; ++kind)
     for (int ph = 0; ph < 3; ++ph) {
@@ -2270,6 +2482,7 @@ std::unique_ptr<Plan> merge_contract_plans(std::vector<std::unique_ptr<Plan>>& p
   }
   validate_gemms(*M, f64);
   validate_direct(*M);
+  validate_blocks(*M);
   M->upload(device);
   return M;
 }
@@ -2337,6 +2550,22 @@ int run_direct(Plan& p, int op, Range r, const BoxPtrs& ptrs, void* stream, int 
                p.ditem_flops_prefix[r.first + r.count] - p.ditem_flops_prefix[r.first]);
   return cuda_code(launch_direct(p.f64(), op, p.d_ditems + r.first, r.count, ptrs, stream),
                    "direct kernel");
+}
+
+// block contraction of phases [ph0, ph1] (their tiles are contiguous): one launch
+int run_block(Plan& p, int ph0, int ph1, const BoxPtrs& ptrs, void* stream, int phase) {
+  Range r{p.blk_range[ph0].first, 0};
+  double bytes = 0.0, flops = 0.0;
+  for (int ph = ph0; ph <= ph1; ++ph) {
+    r.count += p.blk_range[ph].count;
+    bytes += p.blk_bytes[ph];
+    flops += p.blk_flops[ph];
+  }
+  if (r.count <= 0) return SYM_OK;
+  p.last_launches++;
+  ProfScope ps(p, phase, SYM_KERNEL_BLOCK, stream, bytes, flops);
+  return cuda_code(launch_block(p.f64(), p.d_btiles + r.first, r.count, p.d_bsegs, p.blk_ws, p.d_blk_cnt, ptrs, stream),
+                   "block kernel");
 }
 
 int run_gemm_kind(Plan& p, int kind, Range r, void* stream, int phase) {
@@ -2474,8 +2703,14 @@ int exec_transform(Plan& p, const void* in, void* out, void* stream) {
 int exec_contract(Plan& p, const void* A, const void* B, void* C, void* stream) {
   if (p.dry) fail(SYM_ERR_UNSUPPORTED, "plan was built with SYM_PLAN_DRYRUN=1 and cannot run");
   p.last_launches = 0;
+  BoxPtrs d{};
+  d.src[0] = A;
+  d.src[1] = B;
+  d.dst[DST_OUT] = C;
+  int rc = run_block(p, 0, 0, d, stream, PH_FWD_GEMM_SIMT);
+  if (rc) return rc;
   BoxPtrs g = gather_ptrs(p, A, B, nullptr);
-  int rc = run_box(p, p.fwd_gather, g, stream, PH_FWD_GATHER);
+  rc = run_box(p, p.fwd_gather, g, stream, PH_FWD_GATHER);
   if (rc) return rc;
   rc = run_gemm(p, 0, 0, stream, PH_FWD_GEMM);
   if (rc) return rc;
@@ -2486,10 +2721,6 @@ int exec_contract(Plan& p, const void* A, const void* B, void* C, void* stream) 
   s.dst[DST_OUT] = C;
   rc = run_box(p, p.fwd_scatter, s, stream, PH_FWD_SCATTER);
   if (rc) return rc;
-  BoxPtrs d{};
-  d.src[0] = A;
-  d.src[1] = B;
-  d.dst[DST_OUT] = C;
   return run_direct(p, kDirectApply, p.fwd_direct, d, stream, PH_FWD_DIRECT);
 }
 
@@ -2498,6 +2729,13 @@ int exec_contract_backward(Plan& p, const void* A, const void* B, const void* dC
   if (p.dry) fail(SYM_ERR_UNSUPPORTED, "plan was built with SYM_PLAN_DRYRUN=1 and cannot run");
   p.last_launches = 0;
   if (!dA && !dB) return SYM_OK;
+  BoxPtrs d{};
+  d.src[0] = A;
+  d.src[1] = B;
+  d.src[2] = dC;
+  d.dst[DST_DA] = dA;
+  d.dst[DST_DB] = dB;
+  if (int rc = run_block(p, dA ? 1 : 2, dB ? 2 : 1, d, stream, PH_BWD_GEMM_SIMT)) return rc;
   BoxPtrs g = gather_ptrs(p, A, B, dC);
   if (p.bwd_reads_fwd_operands && (p.fwd_a != A || p.fwd_b != B)) {
     // the operand buffers hold another forward's inputs: gather A and B again
@@ -2529,12 +2767,6 @@ int exec_contract_backward(Plan& p, const void* A, const void* B, const void* dC
   rc = run_box(p, sr, s, stream, PH_BWD_SCATTER);
   if (rc) return rc;
   // after the scatter, which zero-filled the dB blocks the direct sums add into
-  BoxPtrs d{};
-  d.src[0] = A;
-  d.src[1] = B;
-  d.src[2] = dC;
-  d.dst[DST_DA] = dA;
-  d.dst[DST_DB] = dB;
   if (dA)
     if (int r = run_direct(p, kDirectApply, p.bwd_direct_a, d, stream, PH_BWD_DIRECT)) return r;
   return dB ? run_direct(p, kDirectOuter, p.bwd_direct_b, d, stream, PH_BWD_DIRECT) : SYM_OK;

@@ -1,6 +1,7 @@
 // Execution plans: the precomputed, structure-only part of every operation.
 #pragma once
 
+#include <array>
 #include <memory>
 #include <vector>
 
@@ -64,6 +65,20 @@ struct Plan {
   Range fwd_direct, bwd_direct_a, bwd_direct_b;  // C = A B; dA = dC B^T; dB += A^T dC
   std::vector<double> ditem_bytes_prefix, ditem_flops_prefix;  // launch statistics
 
+  // block contraction work lists (block.cu) of a plan that runs on the blocks
+  // in place of matrix form: phases 0 = forward, 1 = dA, 2 = dB; the tiles of
+  // a phase are contiguous, dA's before dB's
+  bool blocks = false;
+  std::vector<BlkOut> bouts;
+  std::vector<BlkSeg> bsegs;
+  std::vector<BlkTile> btiles;
+  std::vector<int> btile_out;  // output block of every tile (host checks)
+  int blk_slots = 0, blk_counters = 0;  // workspace of the cut tiles
+  Range blk_range[3];
+  double blk_bytes[3] = {0.0, 0.0, 0.0};  // algorithmic bytes of a phase (its two operands and its result once)
+  double blk_flops[3] = {0.0, 0.0, 0.0};  // useful flops of a phase
+  std::vector<std::array<int, 3>> blk_mnk;  // the phases' sectors (statistics)
+
   // GEMM work lists.  Kinds: 0 = tcgen05 split-BF16 x3, 1 = CUDA-core 64x64,
   // 2 = CUDA-core 256x16, 3 = CUDA-core thin (m, n <= 8), 4 = CUDA-core
   // rows (k, n <= 16); GEMM phases:
@@ -103,6 +118,10 @@ struct Plan {
   BoxItem* d_items = nullptr;
   Term* d_terms = nullptr;
   DirectItem* d_ditems = nullptr;
+  BlkSeg* d_bsegs = nullptr;
+  BlkTile* d_btiles = nullptr;
+  void* blk_ws = nullptr;        // parts of the cut tiles
+  int* d_blk_cnt = nullptr;      // their arrival counters (zero between launches)
   GemmSectorSimt* d_secs_simt = nullptr;
   TcSector* d_secs_tc = nullptr;
   GemmTile* d_tiles = nullptr;
@@ -143,14 +162,46 @@ std::unique_ptr<Plan> plan_transform(const Tensor& in, const Tensor& out, const 
 // next one's input); owns two scratch buffers for the intermediates
 std::unique_ptr<Plan> chain_transforms(std::vector<std::unique_ptr<Plan>> steps, int precision);
 // device = false builds and validates the work lists on the host only (no
-// device allocation); such a plan runs only through sym_contract_noalloc.
+// device allocation); such a plan runs only through sym_contract_noalloc or
+// merged into a batch plan.  blocks = false keeps every phase in matrix form.
+// nbatch: how many plans the launches will be shared with.
 std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std::vector<int>& pairsA,
                                     const std::vector<int>& pairsB, const Tensor& C, int precision,
-                                    bool device = true);
+                                    bool device = true, bool blocks = true, int nbatch = 1);
 // many independent contractions as one plan over packed buffers (see plan.cpp)
 std::unique_ptr<Plan> merge_contract_plans(std::vector<std::unique_ptr<Plan>>& ps, const std::vector<int64_t>& offA,
                                            const std::vector<int64_t>& offB, const std::vector<int64_t>& offC,
                                            bool device = true);
+
+// ------------------------------------------------- block contraction (block_plan.cpp) --
+// One product of blocks that a contraction sums: block c of C gains coef
+// times the product of block a of A with block b of B.
+struct BlkTriple {
+  int64_t a, b, c;
+  double coef;
+};
+// Work lists of one phase (0 forward, 1 dA, 2 dB; in this order) from the
+// contraction's products; false when a block has more dims than the kernel
+// takes or an offset leaves 32 bits.  free / pairs: leg numbers as in
+// plan_contract; share: the part of a launch's fixed costs and latency this
+// plan bears (1, or 1/n in a batch of n).  *model_us: the phase's modelled time.
+bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, const Tensor& C,
+                      const std::vector<BlkTriple>& triples, const std::vector<int>& freeA,
+                      const std::vector<int>& freeB, const std::vector<int>& pairsA, const std::vector<int>& pairsB,
+                      double share, double* model_us);
+void drop_blocks(Plan& P);  // takes the lists of every phase out again
+void validate_blocks(const Plan& P);
+double blk_tile_cost(bool f64, const BlkTile& t);  // modelled clocks of a tile (launch order)
+
+// Magic numbers for dividing 31-bit dividends by d >= 1 with one multiply-high
+// (Granlund & Montgomery, PLDI 1994, Thm 4.2 with N = 31):
+// s = ceil(log2 d), m = ceil(2^(31+s) / d) < 2^32, floor(a / d) = (2a * m) >> (32 + s).
+inline void div_magic(int d, uint32_t& m, int8_t& s) {
+  int l = 0;
+  while (((int64_t)1 << l) < d) ++l;
+  m = (uint32_t)((((uint64_t)1 << (31 + l)) + (uint64_t)d - 1) / (uint64_t)d);
+  s = (int8_t)l;
+}
 
 // Execution (asynchronous on `stream`); return SYM_OK or a negative code.
 int exec_transform(Plan& p, const void* in, void* out, void* stream);
