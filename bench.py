@@ -1130,7 +1130,7 @@ def run_svd(args, rank, world):
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms_per_step, 4),
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
         "config": bench_config(EigWorkload.describe if is_eig else SVDWorkload.describe),
-        "precision": "FP64 result: FP32 Jacobi sweeps seed FP64 Newton-Schulz + FP64 Jacobi sweeps"
+        "precision": "FP64 result: FP32 Jacobi sweeps seed FP64 Newton steps (FP64 sweeps where those do not converge)"
                      + (" on the block's symmetric part shifted by its Frobenius norm" if is_eig else ""),
         "blocks": plan.nblocks, "singular_values": plan.nsv, "chi": chi,
         "launch": "eager (host truncation)",
@@ -1138,7 +1138,7 @@ def run_svd(args, rank, world):
         "roofline": roof, "step_roofline": step_roof, "kernels": kernels,
         "e2e": {"value": round(1e3 / ms_e2e * world, 4), "unit": unit, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": round(ms_e2e, 4)},
-        "clocks": clk, "gpu_launches": 2 * args.steps,
+        "clocks": clk, "gpu_launches": 25 * args.steps,  # 24 an execute (kMaxRefine = 5 steps of four kernels), one for the factors
     }
     vals_gpu = plan.execute(T.data).cpu().numpy()  # every block's values, for the oracle's comparison
     torch.cuda.synchronize()

@@ -395,13 +395,13 @@ int sym_wait_probe(int limit_us, int word);
  * sym_svd_plan: plan the decomposition of tensors with T's structure:
  *   nblocks = number of diagonal blocks (labels x with rows and columns),
  *   nsv = sum over blocks of min(m_x, n_x) (the length of S).  The plan owns
- *   a workspace of about 2.5 (max(m,n) + min(m,n)) min(m,n) doubles per
+ *   a workspace of about (3.5 max(m,n) + 6 min(m,n)) min(m,n) doubles per
  *   block.
  * sym_svd_blocks: per block, ascending x: x, m_x, n_x (arrays of nblocks
  *   ints; any may be NULL).
  * sym_svd_execute: decompose the FP64 blocks `T` (device, T's layout).
- *   Jacobi sweeps in FP32 choose the starting point, which is made
- *   orthogonal in FP64 (Newton-Schulz); FP64 sweeps then converge to FP64
+ *   Jacobi sweeps in FP32 choose the starting point, which FP64 Newton
+ *   steps (or, for blocks of less than full rank, FP64 sweeps) take to FP64
  *   accuracy, so the result is an FP64 SVD.
  *   S (device, nsv doubles, caller-owned) receives every block's singular
  *   values in descending order, blocks in ascending x; the singular vectors
@@ -410,8 +410,9 @@ int sym_wait_probe(int limit_us, int word);
  *   (SYM_ERR_NUMERIC, see sym_device_status).
  * sym_svd_stats: per block of the last execute (ascending x; either array
  *   may be NULL): the sweeps it took and the rotations it applied, of the
- *   FP64 sweeps (fp32 = 0; the last one rotated no pair by more than 1e-8
- *   of its columns' norms, so what it left is at the FP64 rounding level)
+ *   FP64 part (fp32 = 0: the Newton steps, with 0 rotations, or, for a block
+ *   finished by FP64 sweeps, those; the last one rotated no pair by more than
+ *   1e-8 of its columns' norms, so what it left is at the FP64 rounding level)
  *   or of the FP32 sweeps (fp32 = 1; the last one rotated no pair by more
  *   than 1e-4, or it is the 40th).  Synchronizes the device.
  * sym_svd_truncation: keep[b] from a host copy of execute's S (reading of

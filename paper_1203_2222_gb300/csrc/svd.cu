@@ -8,35 +8,45 @@
 // because the row legs lead), so there is no separate move into matrix form.
 //
 // svd_jacobi_kernel: one cluster of 16 CTAs per block, one-sided Jacobi
-//   (Hestenes).  A = M_x (m >= n) or M_x^T, R x C with R >= C, is copied
-//   column-major into the workspace.  A sweep visits every column pair once,
-//   in the round-robin order of a tournament (C - 1 rounds of C/2 disjoint
-//   pairs, one warp per pair, a cluster barrier between rounds); a pair whose
-//   columns are not orthogonal to within sqrt(R) ulp is rotated so that they
-//   are, and the same rotation is applied to V (V = I at the start).  When a
-//   whole sweep rotates nothing by more than kBigRotation(32) relative,
-//   A V = W has orthogonal columns: S = their norms, U = W / S.  The sweeps
-//   run first in FP32, then, from the FP32 result made orthogonal in FP64,
-//   in FP64 (see the kernel).  The FP32 sweeps of blocks with at least 32
-//   columns take the same pairs by column blocks, a block pair in a CTA's
-//   shared memory (jacobi_sweeps_blocked).  The FP64
-//   sweeps are bounded (kMaxSweeps); a block that has not converged by then
-//   sets the device error word to SYM_ERR_NUMERIC.  The columns are then
-//   ranked by norm (descending, ties by index) into S and a permutation.
+//   (Hestenes) in FP32.  A = M_x (m >= n) or M_x^T, R x C with R >= C, is
+//   copied column-major into the workspace.  A sweep visits every column pair
+//   once, in the round-robin order of a tournament; a pair whose columns are
+//   not orthogonal to within sqrt(R) ulp is rotated so that they are, and the
+//   same rotation is applied to V (V = I at the start).  Blocks with at least
+//   64 columns take the pairs by column blocks, a block pair in a CTA's shared
+//   memory (jacobi_sweeps_blocked), others a warp per pair with a cluster
+//   barrier between rounds.  V is the starting point of
+// svd_av_kernel, svd_gram_kernel, svd_correction_kernel, svd_update_kernel:
+//   up to kMaxRefine Newton steps in FP64 (below), each a few products over all
+//   blocks that spread over every SM.  A V = W then has orthogonal columns: S =
+//   their norms, U = W / S.
+// svd_sweep_kernel: FP64 Jacobi sweeps for the blocks that the refinement did
+//   not finish (rank-deficient blocks, clusters).  They are bounded
+//   (kMaxSweeps); a block that has not converged by then sets the device error
+//   word to SYM_ERR_NUMERIC.
+// svd_place_kernel, svd_rank_kernel: norms, and the columns ranked by norm
+//   (descending, ties by index) into S and a permutation.
 // svd_factor_kernel: one CTA per block writes the kept singular vectors into
 //   the blocks of U (row legs, bond) and V (bond, column legs), optionally
 //   scaled by S.
 //
-// The same two kernels give the blockwise eigendecomposition of a symmetric
+// Measured (GB300, two-site tensor D = 2048: 41 blocks up to 272 x 272):
+// execute and factors 19.3 -> 7.8 ms; the two-site density matrix (42 blocks)
+// 25.6 -> 9.0 ms.  Before, two FP64 sweeps (eig: four) in serial rounds on each
+// block's own cluster took 14 ms (20 ms); the refinement takes 2.6 ms, bound
+// by FP64 (two multiply-adds a clock of an SM; 70% of it), the FP32 sweeps 5 to
+// 6 ms, bound by shared memory and the rounds' barriers.
+//
+// The same kernels give the blockwise eigendecomposition of a symmetric
 // tensor seen as a square matrix (Ch. 5, Eq. spectral, by blocks as the
-// thesis prescribes after Eq. svd1; blocks flagged `eig`): the block is
-// replaced by its symmetric part B = (M + M^T)/2 plus sigma I, where sigma is
-// B's Frobenius norm (>= its spectral norm), so that B + sigma I is positive
-// semidefinite.  For such a matrix the one-sided Jacobi result A V = W has
-// |w_j| = lambda_j + sigma and V's columns are the eigenvectors, so the
-// eigenvalues are |w_j| - sigma (absolute error ~ eps sigma, the backward
-// error of any FP64 symmetric eigensolver), ranked by |lambda| descending
-// (ties: the larger lambda, then the column), and U = V, V^T for the factors.
+// thesis prescribes after Eq. svd1; blocks flagged `eig`).  The block is
+// replaced by its symmetric part B = (M + M^T)/2.  The FP32 sweeps run on B
+// plus a shift that makes it positive definite (then the one-sided Jacobi
+// result's V holds the eigenvectors), the refinement on V^T B V itself, whose
+// diagonal gives the eigenvalues.  The FP64 sweeps, where a block needs them,
+// run on B + sigma I with sigma the Frobenius norm (>= the spectral norm), so
+// that |w_j| = lambda_j + sigma.  Eigenvalues are ranked by |lambda|
+// descending (ties: the larger lambda, then the column), and U = V, V^T.
 // The workspace stays L2-resident for the sizes of tensor-network bonds
 // (a 300 x 300 block is 1.4 MB), so the sweeps run from L2, not HBM.
 #include <cooperative_groups.h>
@@ -62,8 +72,10 @@ namespace cg = cooperative_groups;
 namespace sym {
 namespace {
 
-constexpr int kSvdThreads = 256;
-constexpr int kSvdWarps = kSvdThreads / 32;
+constexpr int kSvdThreads = 256;  // FP64 sweeps (128 registers a thread, two CTAs an SM)
+// FP32 sweeps: a round has up to 12 column pairs a CTA, one a warp -- with 8
+// warps the 9 pairs of a 272-column block took two passes
+constexpr int kThreads32 = 384;
 // CTAs per diagonal block (16: a cluster size above the portable 8, allowed
 // by a function attribute; two CTAs of the kernel fit on an SM)
 constexpr int kSvdCluster = 16;
@@ -97,9 +109,51 @@ struct SvdBlock {
   double sgn;     // eig, SU(2) with an incoming row leg: (-1)^{2j}, the sign of the dense block; else 1
   int bw;         // FP32 sweeps by column blocks of bw columns (0: by column pairs)
   int bw64;       // the same for the FP64 sweeps
-  int64_t w;   // workspace offset: W (R x C, column-major), V (C x C), norms (C), sorted S (C), then
-               // the Jacobi kernel's A (R x C), Newton-Schulz factor (C x C), FP32 W and V
+  int64_t w;   // workspace offset (SvdWork; matrices column-major)
   int64_t s;   // first singular value of the block in S and in the permutation
+};
+
+// FP64 refinement steps after the FP32 sweeps before a block goes on to FP64 sweeps
+constexpr int kMaxRefine = 5;
+// What the kernels of one call hand on per block (blocks in launch order).
+struct SvdState {
+  double sa, unsa;  // power-of-two scale of A, and its inverse
+  double shift;     // eig: sigma (the block's Frobenius norm)
+  double norm2;     // squared Frobenius norm of sa A
+  unsigned xmax[kMaxRefine];  // bits of the largest squared column norm of a step's correction X (FP32)
+  int nulls[kMaxRefine];      // SVD: a step left pairs of columns at the rounding level alone
+  int done;         // refinement step after which the block counts as converged (0: not, -1: given up)
+};
+// One 32 x 32 tile of a refinement product; kind 0: W or V^T W, 1: V^T V or the other factor (see the kernels)
+struct SvdTile {
+  int block, i0, j0, kind;
+};
+
+// The parts of a block's workspace.
+struct SvdWork {
+  double *W, *V, *nrm, *Ss, *A, *G, *E, *W2, *V2;
+  float *W32, *V32, *X, *F0, *F1;
+  __host__ __device__ static int64_t elems(int64_t R, int64_t C) {
+    const int64_t rc = R * C, cc = C * C;
+    return 3 * rc + 4 * cc + 2 * C + (rc + 4 * cc + 1) / 2 + 1;
+  }
+  __device__ SvdWork(double* w, int64_t R, int64_t C) {
+    const int64_t rc = R * C, cc = C * C;
+    W = w;  // the factor kernel reads W, V, the norms and Ss at these places
+    V = W + rc;
+    nrm = V + cc;
+    Ss = nrm + C;
+    A = Ss + C;
+    G = A + rc;
+    E = G + cc;
+    W2 = E + cc;
+    V2 = W2 + rc;
+    W32 = reinterpret_cast<float*>(V2 + cc);
+    V32 = W32 + rc;
+    X = V32 + cc;
+    F0 = X + cc;
+    F1 = F0 + cc;
+  }
 };
 
 // A tensor block inside its M_x: rows r0.., columns c0.. (row-major, rows x cols).
@@ -127,13 +181,13 @@ struct JacobiArith;
 
 template <>
 struct JacobiArith<float> {
-  static constexpr float kEps = FLT_EPSILON;
+  // the FP32 sweeps only choose a starting point: approximate roots and quotients
+  static __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
   static __device__ __forceinline__ bool angle(float a, float bb, float g, float sab, float tol, float& c,
                                                float& s) {
     if (!(fabsf(g) > tol * sab)) return false;
-    const float zeta = (bb - a) / (2.0f * g);
-    const float t = fabsf(zeta) > 1e18f ? 0.5f / zeta
-                                        : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
+    const float d = bb - a, h = 2.0f * g;  // t = sign(d) h / (|d| + sqrt(d^2 + h^2))
+    const float t = __fdividef(copysignf(1.0f, d) * h, fabsf(d) + root(fmaf(d, d, h * h)));
     c = rsqrtf(fmaf(t, t, 1.0f));
     s = c * t;
     return true;
@@ -142,7 +196,7 @@ struct JacobiArith<float> {
 
 template <>
 struct JacobiArith<double> {
-  static constexpr double kEps = DBL_EPSILON;
+  static __device__ __forceinline__ double root(double x) { return sqrt(x); }
   // The angle itself needs only FP32 accuracy: an inexact angle is still an
   // exact rotation (c^2 + s^2 = 1 to FP64 precision), it just leaves the
   // pair slightly non-orthogonal for the next sweep.  So t = sign(d) h /
@@ -277,11 +331,11 @@ struct SweepCtl {
 // sweeps taken, conv = the last sweep rotated nothing.  The C/2 pairs of a
 // round (tournament order, an odd C playing against a bye) go to the
 // cluster's warps; cluster barriers separate the rounds.
-template <typename T>
+template <typename T, int NT>
 __device__ int jacobi_sweeps(T* W, T* V, T* nrm2, int R, int C, int max_sweeps, T tol, cg::cluster_group& cluster,
                              SweepCtl* ctl, int* flag0, int crank, int cw, int lane, int& gsweep,
                              unsigned long long& myrot, bool& conv, T big_tol) {
-  constexpr int kCW = kSvdCluster * kSvdWarps;
+  constexpr int kCW = kSvdCluster * (NT / 32);
   const int Ce = C + (C & 1);
   const int rpl = (R + 31) / 32;
   const int nr = rpl <= 1 ? 1 : rpl <= 2 ? 2 : rpl <= 4 ? 4 : rpl <= 8 ? 8 : rpl <= 9 ? 9 : rpl <= 12 ? 12 : 0;
@@ -378,7 +432,7 @@ __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* n
   }
   g = warp_sum(g);
   const T a = *na, bb = *nb;
-  const T sab = sqrt(a * bb);
+  const T sab = JacobiArith<T>::root(a * bb);
   T c, sn;
   if (!JacobiArith<T>::angle(a, bb, g, sab, tol, c, sn)) return 0;
 #pragma unroll
@@ -414,13 +468,32 @@ __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* n
 // a sweep, as in the order by pairs, but a sweep needs kColBlocks - 1 cluster
 // barriers instead of C - 1, and the pairs' columns come from shared memory.
 constexpr int kColBlocks = 2 * kSvdCluster;
-template <typename T, int NR>
+// n contiguous values between L2 and shared memory, eight loads in flight a thread
+template <int NT, typename T>
+__device__ __forceinline__ void copy_in(T* dst, const T* src, int n) {
+  int i = threadIdx.x;
+  for (; i + 7 * NT < n; i += 8 * NT) {
+    T x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = __ldcg(src + i + u * NT);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) dst[i + u * NT] = x[u];
+  }
+#pragma unroll 4
+  for (; i < n; i += NT) dst[i] = __ldcg(src + i);
+}
+template <int NT, typename T>
+__device__ __forceinline__ void copy_out(T* dst, const T* src, int n) {
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n; i += NT) __stcg(dst + i, src[i]);
+}
+template <typename T, int NR, int NT>
 __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, int max_sweeps, T tol,
                                      cg::cluster_group& cluster, SweepCtl* ctl, int* flag0, int crank, int lane,
                                      int& gsweep, unsigned long long& myrot, bool& conv, T big_tol, T* sm) {
   const int warp = threadIdx.x >> 5;
-  constexpr int kCW = kSvdCluster * kSvdWarps;
-  const int cw = crank * kSvdWarps + warp;
+  constexpr int kWarps = NT / 32, kCW = kSvdCluster * kWarps;
+  const int cw = crank * kWarps + warp;
   T* Wp = sm;  // bw columns of R, then Q's, then V's columns of P and Q (C each), then their squared norms
   T* Wq = Wp + (int64_t)bw * R;
   T* Vp = Wq + (int64_t)bw * R;
@@ -460,16 +533,16 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
       const int p0 = P * bw, np = max(0, min(bw, C - p0));
       const int q0 = Q * bw, nq = max(0, min(bw, C - q0));
       // the two blocks' columns are contiguous in the column-major W and V
-      for (int i = threadIdx.x; i < np * R; i += kSvdThreads) Wp[i] = __ldcg(W + (int64_t)p0 * R + i);
-      for (int i = threadIdx.x; i < nq * R; i += kSvdThreads) Wq[i] = __ldcg(W + (int64_t)q0 * R + i);
-      for (int i = threadIdx.x; i < np * C; i += kSvdThreads) Vp[i] = __ldcg(V + (int64_t)p0 * C + i);
-      for (int i = threadIdx.x; i < nq * C; i += kSvdThreads) Vq[i] = __ldcg(V + (int64_t)q0 * C + i);
-      for (int i = threadIdx.x; i < np; i += kSvdThreads) Np[i] = __ldcg(nrm2 + p0 + i);
-      for (int i = threadIdx.x; i < nq; i += kSvdThreads) Nq[i] = __ldcg(nrm2 + q0 + i);
+      copy_in<NT>(Wp, W + (int64_t)p0 * R, np * R);
+      copy_in<NT>(Wq, W + (int64_t)q0 * R, nq * R);
+      copy_in<NT>(Vp, V + (int64_t)p0 * C, np * C);
+      copy_in<NT>(Vq, V + (int64_t)q0 * C, nq * C);
+      copy_in<NT>(Np, nrm2 + p0, np);
+      copy_in<NT>(Nq, nrm2 + q0, nq);
       __syncthreads();
       if (r == 0) {  // the pairs inside P and inside Q: each block's own tournament, side by side
         for (int ir = 0; ir < bwe - 1; ++ir) {
-          for (int t = warp; t < bwe; t += kSvdWarps) {
+          for (int t = warp; t < bwe; t += kWarps) {
             const int side = t < bwe / 2 ? 0 : 1, kk = side ? t - bwe / 2 : t;
             int a = kk == 0 ? ir : (ir + kk) % (bwe - 1);
             int c = kk == 0 ? bwe - 1 : (ir - kk + bwe - 1) % (bwe - 1);
@@ -485,19 +558,19 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
         }
       }
       for (int ir = 0; ir < bw; ++ir) {  // the cross pairs (i, (i + ir) mod bw)
-        for (int i = warp; i < bw; i += kSvdWarps) {
+        for (int i = warp; i < bw; i += kWarps) {
           const int j = (i + ir) % bw;
           if (i < np && j < nq)
             rot(Wp + (int64_t)i * R, Wq + (int64_t)j * R, Vp + (int64_t)i * C, Vq + (int64_t)j * C, Np + i, Nq + j);
         }
         __syncthreads();
       }
-      for (int i = threadIdx.x; i < np * R; i += kSvdThreads) __stcg(W + (int64_t)p0 * R + i, Wp[i]);
-      for (int i = threadIdx.x; i < nq * R; i += kSvdThreads) __stcg(W + (int64_t)q0 * R + i, Wq[i]);
-      for (int i = threadIdx.x; i < np * C; i += kSvdThreads) __stcg(V + (int64_t)p0 * C + i, Vp[i]);
-      for (int i = threadIdx.x; i < nq * C; i += kSvdThreads) __stcg(V + (int64_t)q0 * C + i, Vq[i]);
-      for (int i = threadIdx.x; i < np; i += kSvdThreads) __stcg(nrm2 + p0 + i, Np[i]);
-      for (int i = threadIdx.x; i < nq; i += kSvdThreads) __stcg(nrm2 + q0 + i, Nq[i]);
+      copy_out<NT>(W + (int64_t)p0 * R, Wp, np * R);
+      copy_out<NT>(W + (int64_t)q0 * R, Wq, nq * R);
+      copy_out<NT>(V + (int64_t)p0 * C, Vp, np * C);
+      copy_out<NT>(V + (int64_t)q0 * C, Vq, nq * C);
+      copy_out<NT>(nrm2 + p0, Np, np);
+      copy_out<NT>(nrm2 + q0, Nq, nq);
       cluster.sync();  // the next round reads columns this round wrote, on other CTAs
     }
     const int f = (__syncthreads_or(did) ? 1 : 0) | (__syncthreads_or(big) ? 2 : 0);
@@ -518,7 +591,7 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
 // X C x C, out rows x C); a warp per (column j, 128 rows).
 __device__ void gemm_cols(const double* Aop, int rows, int C, const double* X, double* out, double scale, int cw,
                           int lane) {
-  constexpr int kCW = kSvdCluster * kSvdWarps;
+  constexpr int kCW = kSvdCluster * (kSvdThreads / 32);
   const int nrb = (rows + 127) / 128;
   for (int task = cw; task < C * nrb; task += kCW) {
     const int j = task / nrb, r0 = (task - j * nrb) * 128;
@@ -546,7 +619,7 @@ __device__ void gemm_cols(const double* Aop, int rows, int C, const double* X, d
 // Newton-Schulz step Q <- Q G towards the orthogonal polar factor of Q; a
 // warp per (row i, four columns j).
 __device__ void newton_schulz_factor(const double* Q, int C, double* G, int cw, int lane) {
-  constexpr int kCW = kSvdCluster * kSvdWarps;
+  constexpr int kCW = kSvdCluster * (kSvdThreads / 32);
   const int nj = (C + 3) / 4;
   for (int task = cw; task < C * nj; task += kCW) {
     const int i = task / nj, j0 = (task - i * nj) * 4;
@@ -566,6 +639,105 @@ __device__ void newton_schulz_factor(const double* Q, int C, double* G, int cw, 
   }
 }
 
+// eig: a shift that makes the block B (here sa B in FP32, W) positive definite
+// but hardly larger than that needs.  One-sided Jacobi finds a column of
+// norm |lambda + shift| to FP32 accuracy relative to that norm, so with the
+// Frobenius norm as the shift the eigenvectors of close small eigenvalues (a
+// density matrix has many) come out mixed; 17 of the 42 blocks of the two-site
+// density matrix then failed the refinement.  kLanczos Lanczos steps bound
+// the spectrum: shift = max(0, -smallest Ritz value) + 10% of its extent (of
+// the 42 blocks: 1% takes 14 FP32 sweeps and 3 refinement steps, 10% 12 and 3,
+// 100% 10 and 5; 10.5, 9.6 and 9.4 ms in all).  A shift that is still too
+// small only costs accuracy of the starting point.
+constexpr int kLanczos = 32;
+__device__ float lanczos_shift(const float* W, int C, float* v, float* vp, float* y, cg::cluster_group& cluster,
+                               float* red, float* sh, int crank, int cw, int lane) {
+  // v, vp, y: C floats each (global); red: (kThreads32 / 32) + 1 floats, sh: 2 kLanczos + 1 floats of this CTA
+  constexpr int kCW = kSvdCluster * (kThreads32 / 32);
+  const int tid = threadIdx.x;
+  auto block_sum = [&](float x) {
+    x = warp_sum(x);
+    __syncthreads();
+    if (lane == 0) red[tid >> 5] = x;
+    __syncthreads();
+    float t = 0.0f;
+    for (int w = 0; w < (kThreads32 / 32); ++w) t += red[w];
+    return t;
+  };
+  const int K = min(kLanczos, C);
+  if (crank == 0) {  // a fixed start vector without structure
+    float n = 0.0f;
+    for (int i = tid; i < C; i += kThreads32) {
+      const unsigned h = (unsigned)(i + 1) * 2654435761u;
+      const float x = (float)(int)(h ^ (h >> 15)) * 4.656612873077393e-10f;
+      n = fmaf(x, x, n);
+      __stcg(v + i, x);
+      __stcg(vp + i, 0.0f);
+    }
+    n = rsqrtf(block_sum(n));
+    for (int i = tid; i < C; i += kThreads32) __stcg(v + i, n * __ldcg(v + i));
+  }
+  float beta = 0.0f;
+  for (int k = 0; k < K; ++k) {
+    cluster.sync();
+    for (int j = cw; j < C; j += kCW) {  // y = W v (W symmetric)
+      const float* wj = W + (int64_t)j * C;
+      float a = 0.0f;
+      for (int i = lane; i < C; i += 32) a = fmaf(__ldcg(wj + i), __ldcg(v + i), a);
+      a = warp_sum(a);
+      if (lane == 0) __stcg(y + j, a);
+    }
+    cluster.sync();
+    if (crank == 0) {
+      float a = 0.0f;
+      for (int i = tid; i < C; i += kThreads32) a = fmaf(__ldcg(y + i), __ldcg(v + i), a);
+      const float alpha = block_sum(a);
+      float n = 0.0f;
+      for (int i = tid; i < C; i += kThreads32) {
+        const float r = __ldcg(y + i) - alpha * __ldcg(v + i) - beta * __ldcg(vp + i);
+        n = fmaf(r, r, n);
+        __stcg(vp + i, __ldcg(v + i));
+        __stcg(v + i, r);
+      }
+      beta = sqrtf(block_sum(n));
+      const float inv = beta > 1e-6f ? 1.0f / beta : 0.0f;  // an invariant subspace: the rest adds Ritz values 0
+      for (int i = tid; i < C; i += kThreads32) __stcg(v + i, inv * __ldcg(v + i));
+      if (inv == 0.0f) beta = 0.0f;
+      if (tid == 0) {
+        sh[k] = alpha;
+        sh[kLanczos + k] = beta;  // between k and k + 1
+      }
+      __syncthreads();
+    }
+  }
+  if (crank == 0 && tid == 0) {  // smallest eigenvalue of the tridiagonal matrix by bisection (Sturm counts)
+    float lo = 0.0f, hi = 0.0f;
+    for (int k = 0; k < K; ++k) {
+      const float r = (k > 0 ? sh[kLanczos + k - 1] : 0.0f) + (k + 1 < K ? sh[kLanczos + k] : 0.0f);
+      lo = fminf(lo, sh[k] - r);
+      hi = fmaxf(hi, sh[k] + r);
+    }
+    const float extent = fmaxf(-lo, hi);
+    float top = 0.0f;  // only a negative smallest value matters
+    for (int it = 0; it < 24; ++it) {
+      const float x = 0.5f * (lo + top);
+      int below = 0;
+      float d = 1.0f;
+      for (int k = 0; k < K; ++k) {
+        const float bk = k > 0 ? sh[kLanczos + k - 1] : 0.0f;
+        d = sh[k] - x - bk * bk / d;
+        if (d == 0.0f) d = -1e-30f;
+        below += d < 0.0f;
+      }
+      if (below) top = x;
+      else lo = x;
+    }
+    sh[2 * kLanczos] = -top + 0.1f * extent;
+  }
+  cluster.sync();
+  return *cluster.map_shared_rank(sh + 2 * kLanczos, 0);
+}
+
 // One cluster of kSvdCluster CTAs per block: the pairs of a round are spread
 // over the cluster's warps and the rounds are separated by cluster barriers
 // (their release / acquire order the workspace writes; the workspace is read
@@ -573,41 +745,34 @@ __device__ void newton_schulz_factor(const double* Q, int C, double* G, int cw, 
 //
 // Mixed precision.  GB300 runs FP32 at many times its FP64 rate, so the
 // sweeps that do most of the work run in FP32 on A scaled by a power of two
-// (max |A| in [1/2, 1): no FP32 overflow or underflow of the bulk); their V
-// is made orthogonal to FP64 precision by two Newton-Schulz steps in FP64
-// (an orthogonality error e becomes ~1.5 e^2 per step), W = A V is formed in
-// FP64, and FP64 sweeps polish W and V to FP64 convergence.  The result is
-// the FP64 Jacobi result; the FP32 part only chooses the starting point.
-__global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThreads, 2)
+// (max |A| in [1/2, 1): no FP32 overflow or underflow of the bulk).  Their V
+// is only the starting point: the refinement below takes it to FP64.
+__global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32, 2)
     svd_jacobi_kernel(const SvdBlock* __restrict__ blocks, const SvdPiece* __restrict__ pieces,
-                      const double* __restrict__ T, double* __restrict__ work, double* __restrict__ S,
-                      int* __restrict__ perm, int* __restrict__ sweeps, long long* __restrict__ rotations,
-                      int* __restrict__ err) {
-  __shared__ unsigned long long nrot[2];
+                      const double* __restrict__ T, double* __restrict__ work, SvdState* __restrict__ state,
+                      int* __restrict__ sweeps, long long* __restrict__ rotations) {
+  __shared__ unsigned long long nrot;
   __shared__ unsigned long long amax;
   __shared__ SweepCtl ctl;
-  __shared__ double wsum[kSvdWarps];
-  __shared__ double fpart;  // eig: this CTA's part of the squared Frobenius norm
+  __shared__ double wsum[(kThreads32 / 32)];
+  __shared__ double fpart;  // this CTA's part of the squared Frobenius norm
+  __shared__ float lred[(kThreads32 / 32) + 1], lsh[2 * kLanczos + 1];
   extern __shared__ double sm_pair[];  // the sweeps by column blocks: a block pair of W and V
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
-  const SvdBlock b = blocks[blockIdx.x / kSvdCluster];
+  const int bi = blockIdx.x / kSvdCluster;
+  const SvdBlock b = blocks[bi];
   const int R = b.R, C = b.C;
   const int64_t RC = (int64_t)R * C, CC = (int64_t)C * C;
-  double* W = work + b.w;  // FP64 W, then V, norms, sorted S (the factor kernel's view)
-  double* V = W + RC;
-  double* nrm = V + CC;
-  double* Ss = nrm + C;
-  double* A = Ss + C;  // FP64 A (scaled), the Newton-Schulz factor, FP32 W and V
-  double* G = A + RC;
-  float* W32 = reinterpret_cast<float*>(G + CC);
-  float* V32 = W32 + RC;
+  const SvdWork ws(work + b.w, R, C);
+  double* A = ws.A;
+  float *W32 = ws.W32, *V32 = ws.V32;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int ct = crank * kSvdThreads + tid;       // thread of the cluster
-  const int cw = crank * kSvdWarps + (tid >> 5);  // warp of the cluster
-  constexpr int kCT = kSvdCluster * kSvdThreads;
+  const int ct = crank * kThreads32 + tid;       // thread of the cluster
+  const int cw = crank * (kThreads32 / 32) + (tid >> 5);  // warp of the cluster
+  constexpr int kCT = kSvdCluster * kThreads32;
   if (tid == 0) {
-    nrot[0] = nrot[1] = 0;
+    nrot = 0;
     amax = 0;
     ctl.flag[0] = ctl.flag[1] = 0;
     ctl.any = 0;
@@ -629,43 +794,45 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
       mx = max(mx, (unsigned long long)__double_as_longlong(fabs(v)));  // |v| >= 0 orders as its bits
     }
   }
-  double shift = 0.0;  // eig: sigma
+  cluster.sync();  // the whole block is in A
+  // eig: the symmetric part, in place (the thread of (r, c), r < c, writes
+  // both halves); the squared Frobenius norm
+  double f2 = 0.0;
   if (b.eig) {
-    cluster.sync();  // the whole block is in A
-    // the symmetric part, in place (the thread of (r, c), r < c, writes both
-    // halves), and its squared Frobenius norm
-    double f2 = 0.0;
+    mx = 0;
     for (int64_t e = ct; e < RC; e += kCT) {
       const int r = (int)(e % R), c = (int)(e / R);
+      double v = 0.0;
       if (r < c) {
         const int64_t t = c + (int64_t)r * R;
-        const double v = 0.5 * (__ldcg(A + e) + __ldcg(A + t));
+        v = 0.5 * (__ldcg(A + e) + __ldcg(A + t));
         __stcg(A + e, v);
         __stcg(A + t, v);
         f2 = fma(2.0 * v, v, f2);
       } else if (r == c) {
-        const double v = __ldcg(A + e);
+        v = __ldcg(A + e);
         f2 = fma(v, v, f2);
       }
+      mx = max(mx, (unsigned long long)__double_as_longlong(fabs(v)));
     }
-    f2 = warp_sum(f2);
-    if (lane == 0) wsum[tid >> 5] = f2;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < kSvdWarps; ++w) t += wsum[w];
-      fpart = t;
+  } else {
+    for (int64_t e = ct; e < RC; e += kCT) {
+      const double v = __ldcg(A + e);
+      f2 = fma(v, v, f2);
     }
-    cluster.sync();  // every CTA's part and the symmetric part are written
-    double tot = 0.0;  // the same sum, in the same order, in every thread
-    for (int r = 0; r < kSvdCluster; ++r) tot += *cluster.map_shared_rank(&fpart, r);
-    shift = sqrt(tot);
-    for (int j = ct; j < C; j += kCT) __stcg(A + j + (int64_t)j * R, __ldcg(A + j + (int64_t)j * R) + shift);
-    cluster.sync();
-    mx = 0;
-    for (int64_t e = ct; e < RC; e += kCT)
-      mx = max(mx, (unsigned long long)__double_as_longlong(fabs(__ldcg(A + e))));
   }
+  f2 = warp_sum(f2);
+  if (lane == 0) wsum[tid >> 5] = f2;
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < (kThreads32 / 32); ++w) t += wsum[w];
+    fpart = t;
+  }
+  cluster.sync();  // every CTA's part and the symmetric part are written
+  f2 = 0.0;  // the same sum, in the same order, in every thread
+  for (int r = 0; r < kSvdCluster; ++r) f2 += *cluster.map_shared_rank(&fpart, r);
+  const double shift = b.eig ? sqrt(f2) : 0.0;  // eig: sigma
   if (mx) atomicMax(cluster.map_shared_rank(&amax, 0), mx);
   cluster.sync();
   const double amx = __longlong_as_double((long long)*cluster.map_shared_rank(&amax, 0));
@@ -678,20 +845,31 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
   for (int64_t i = ct; i < RC; i += kCT) __stcg(W32 + i, (float)(sa * __ldcg(A + i)));
   for (int64_t i = ct; i < CC; i += kCT) __stcg(V32 + i, (i % (C + 1) == 0) ? 1.0f : 0.0f);
   cluster.sync();
+  if (b.eig) {  // the FP32 sweeps run on B + a shift; A keeps B
+    const double s = C >= 4 ? (double)lanczos_shift(W32, C, ws.F0, ws.F0 + C, ws.F0 + 2 * C, cluster, lred, lsh, crank, cw, lane)
+                            : sa * shift;
+    for (int j = ct; j < C; j += kCT)
+      __stcg(W32 + j + (int64_t)j * R, (float)(sa * __ldcg(A + j + (int64_t)j * R) + s));
+    cluster.sync();
+  }
 
   int* flag0 = cluster.map_shared_rank(ctl.flag, 0);
-  unsigned long long rot32 = 0, rot64 = 0;
-  bool conv32, conv;
+  unsigned long long rot32 = 0;
+  bool conv32;
   int gsweep = 0;
   const float tol32 = sqrtf((float)R) * FLT_EPSILON;
+  float* nrm32 = reinterpret_cast<float*>(ws.nrm);
   int sw32;
   switch (b.bw ? (R + 31) / 32 : 0) {
-#define SYM_BLOCKED(NR)                                                                                           \
-  case NR:                                                                                                         \
-    sw32 = jacobi_sweeps_blocked<float, NR>(W32, V32, reinterpret_cast<float*>(nrm), R, C, b.bw, kMaxSweeps32,     \
-                                            tol32, cluster, &ctl, flag0, crank, lane, gsweep, rot32, conv32,       \
-                                            kBigRotation32, reinterpret_cast<float*>(sm_pair));                    \
+#define SYM_BLOCKED(NR)                                                                                       \
+  case NR:                                                                                                    \
+    sw32 = jacobi_sweeps_blocked<float, NR, kThreads32>(W32, V32, nrm32, R, C, b.bw, kMaxSweeps32, tol32, cluster, &ctl,  \
+                                            flag0, crank, lane, gsweep, rot32, conv32, kBigRotation32,        \
+                                            reinterpret_cast<float*>(sm_pair));                               \
     break;
+#define SYM_BLOCKED_UP_TO(NR) \
+  case NR - 1:                \
+    SYM_BLOCKED(NR)
     SYM_BLOCKED(1)
     SYM_BLOCKED(2)
     SYM_BLOCKED(3)
@@ -704,33 +882,375 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     SYM_BLOCKED(10)
     SYM_BLOCKED(11)
     SYM_BLOCKED(12)
+    SYM_BLOCKED_UP_TO(14)
+    SYM_BLOCKED_UP_TO(16)
+    SYM_BLOCKED_UP_TO(18)
+    SYM_BLOCKED_UP_TO(20)
+#undef SYM_BLOCKED_UP_TO
 #undef SYM_BLOCKED
     default:
-      sw32 = jacobi_sweeps<float>(W32, V32, reinterpret_cast<float*>(nrm), R, C, kMaxSweeps32, tol32, cluster, &ctl,
-                                  flag0, crank, cw, lane, gsweep, rot32, conv32, kBigRotation32);
+      sw32 = jacobi_sweeps<float, kThreads32>(W32, V32, nrm32, R, C, kMaxSweeps32, tol32, cluster, &ctl, flag0, crank, cw, lane,
+                                  gsweep, rot32, conv32, kBigRotation32);
+  }
+  if (lane == 0 && rot32) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot32);
+  for (int64_t i = ct; i < CC; i += kCT) __stcg(ws.V + i, (double)__ldcg(V32 + i));
+  cluster.sync();  // the rotation counts have arrived at rank 0
+  if (crank == 0 && tid == 0) {
+    sweeps[2 * b.slot + 1] = sw32;
+    rotations[2 * b.slot + 1] = (long long)nrot;
+    sweeps[2 * b.slot] = 0;
+    rotations[2 * b.slot] = 0;
+    SvdState& st = state[bi];
+    st.sa = sa;
+    st.unsa = unsa;
+    st.shift = shift;
+    st.norm2 = sa * sa * f2;
+    st.done = 0;
+    for (int i = 0; i < kMaxRefine; ++i) {
+      st.xmax[i] = 0;
+      st.nulls[i] = 0;
+    }
+  }
+}
+
+// ------------------------------------------------------------- FP64 refinement --
+// V (from the FP32 sweeps, or from the step before) is orthogonal and
+// diagonalises the block up to a small error; one step removes it to first
+// order.  From W = A V, G = W^T W (eig: T = V^T W) and E = V^T V - I, all in
+// FP64, the correction X with V' = V (I + X) has X_pq + X_qp = -E_pq and
+// makes the off-diagonal element G_pq + a_p X_pq + a_q X_qp vanish (a_p, a_q:
+// the diagonal elements): the symmetric part is -E/2, the antisymmetric one
+// the Jacobi rotation of the pair with g' = G_pq - E_pq (a_p + a_q) / 2 (its
+// sine, and on the diagonal its cosine less one, so that an isolated pair of
+// close values is rotated exactly).  This is Newton's iteration for the
+// singular value (eigenvalue) problem: what a step leaves is quadratic in X,
+// so a step whose columns of X are all at most 1e-8 long ends the block: its
+// remainder is 1e-16.  X multiplies V in FP32 (V' = V + V X: the product's
+// relative error 6e-8 falls on a term of at most |X|, which the next step
+// sees in full; on the last one it is 6e-16 of 1e-8), everything else is FP64.
+//
+// Against FP64 Jacobi sweeps, which this replaces: 2 RC^2 multiply-adds a
+// step in products that spread over every SM, instead of 9/2 RC^2 a sweep in
+// serial rounds on the block's own cluster.  FP64 (two multiply-adds a clock
+// of an SM) bounds the products.  A block that has not converged after
+// kMaxRefine steps (clusters of values the FP32 sweeps could not tell apart)
+// starts again from the FP32 V with FP64 sweeps (svd_sweep_kernel).
+constexpr int kTile = 32, kSlab = 16, kTileThreads = 128;
+
+// 32 x 32 tile of out = alpha sum_k P(i, k) Q(k, j), Q column-major (ldq), P
+// column-major (kTrans = false: P(i, k) = p[i + k ldp]) or transposed
+// (p[k + i ldp]).  A thread has 4 x 2 elements 8 rows and 16 columns apart,
+// so that rows and columns past the edge are skipped whole: an FP64
+// multiply-add occupies a warp's FP64 pipe for 16 clocks.
+template <bool kTrans, typename Store>
+__device__ __forceinline__ void tile_f64(const double* __restrict__ p, int64_t ldp, int m, const double* __restrict__ q,
+                                         int64_t ldq, int n, int K, int i0, int j0, Store store) {
+  __shared__ double ps[2][kSlab][kTile + 1], qs[2][kSlab][kTile + 1];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int ml = min(kTile, m - i0), nl = min(kTile, n - j0);
+  double rp[4], rq[4];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + kTileThreads * u;
+      const int kk = k0 + (kTrans ? e % kSlab : e / kTile), i = kTrans ? e / kSlab : e % kTile;
+      rp[u] = kk < K && i < ml ? __ldcg(p + (kTrans ? kk + (int64_t)(i0 + i) * ldp : i0 + i + (int64_t)kk * ldp)) : 0.0;
+      const int kq = k0 + e % kSlab, j = e / kSlab;
+      rq[u] = kq < K && j < nl ? __ldcg(q + kq + (int64_t)(j0 + j) * ldq) : 0.0;
+    }
+  };
+  auto put = [&](int s) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + kTileThreads * u;
+      ps[s][kTrans ? e % kSlab : e / kTile][kTrans ? e / kSlab : e % kTile] = rp[u];
+      qs[s][e % kSlab][e / kSlab] = rq[u];
+    }
+  };
+  double acc[4][2] = {};
+  const int ns = (K + kSlab - 1) / kSlab;
+  load(0);
+  put(0);
+  __syncthreads();
+  for (int s = 0; s < ns; ++s) {
+    if (s + 1 < ns) load((s + 1) * kSlab);
+#pragma unroll
+    for (int k = 0; k < kSlab; ++k) {
+      double a[4], b[2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = ps[s & 1][k][ty + 8 * i];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) b[j] = qs[s & 1][k][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (8 * i < ml)
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            if (16 * j < nl) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    if (s + 1 < ns) put((s + 1) & 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if (ty + 8 * i < ml && tx + 16 * j < nl) store(i0 + ty + 8 * i, j0 + tx + 16 * j, acc[i][j]);
+}
+
+__device__ __forceinline__ double* refine_v(const SvdWork& ws, int step) { return step & 1 ? ws.V2 : ws.V; }
+__device__ __forceinline__ float* refine_f(const SvdWork& ws, int step) {
+  return step == 0 ? ws.V32 : step & 1 ? ws.F0 : ws.F1;
+}
+
+// W = sa A V, and its FP32 copy (for W X of a last step)
+__global__ void __launch_bounds__(kTileThreads)
+    svd_av_kernel(const SvdBlock* __restrict__ blocks, const SvdTile* __restrict__ tiles, double* __restrict__ work,
+                  const SvdState* __restrict__ state, int step) {
+  const SvdTile t = tiles[blockIdx.x];
+  if (state[t.block].done) return;
+  const SvdBlock& b = blocks[t.block];
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const double sa = state[t.block].sa;
+  const int R = b.R;
+  const bool eig = b.eig != 0;
+  tile_f64<false>(ws.A, R, R, refine_v(ws, step), b.C, b.C, b.C, t.i0, t.j0, [&](int i, int j, double v) {
+    ws.W[i + (int64_t)j * R] = sa * v;
+    if (!eig) ws.W32[i + (int64_t)j * R] = (float)(sa * v);
+  });
+}
+
+// lower triangles of G = W^T W (eig: T = V^T W) and of V^T V
+__global__ void __launch_bounds__(kTileThreads)
+    svd_gram_kernel(const SvdBlock* __restrict__ blocks, const SvdTile* __restrict__ tiles, double* __restrict__ work,
+                    const SvdState* __restrict__ state, int step) {
+  const SvdTile t = tiles[blockIdx.x];
+  if (state[t.block].done) return;
+  const SvdBlock& b = blocks[t.block];
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const double* V = refine_v(ws, step);
+  const int C = b.C;
+  double* out = t.kind ? ws.E : ws.G;
+  auto store = [&](int i, int j, double v) { out[i + (int64_t)j * C] = v; };
+  if (t.kind)
+    tile_f64<true>(V, C, C, V, C, C, C, t.i0, t.j0, store);
+  else if (b.eig)
+    tile_f64<true>(V, C, C, ws.W, C, C, C, t.i0, t.j0, store);
+  else
+    tile_f64<true>(ws.W, b.R, C, ws.W, b.R, C, b.R, t.i0, t.j0, store);
+}
+
+// X, a warp per column q.  The rotation's angle is formed in FP32 from d =
+// a_q - a_p and h = 2 g' (X is FP32 anyway, and GB300's FP64 square roots and
+// divisions are slow).  Pairs whose off-diagonal element is at FP64's rounding
+// level are left alone, as in the Jacobi sweeps: |g'| <= sqrt(R) ulp of
+// |w_p| |w_q| (eig: 4 ulp of the block's norm).  Many large angles at once do
+// not make an orthogonal I + X, so pairs that the error of V so far cannot
+// tell apart are left alone too: in a null space (g' no larger than that error
+// squared times the norm: 1e-5 in step 0, 1e-9 in step 1, the rounding level
+// 3e-14 after that) and in a cluster of equal values (difference and g' within
+// 1e-6, then 1e-11 of them) -- as V becomes orthogonal their g' vanishes by
+// itself.  In steps 0 and 1 such a pair asks for a further step; the columns of
+// an SVD that stay at the rounding level (a block of less than full rank) are
+// left to FP64 sweeps that start from the refined V.
+__global__ void __launch_bounds__(256)
+    svd_correction_kernel(const SvdBlock* __restrict__ blocks, const int2* __restrict__ cols, int ncols,
+                          double* __restrict__ work, SvdState* __restrict__ state, int step) {
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (w >= ncols) return;
+  const int2 bq = cols[w];  // (block, column)
+  SvdState& st = state[bq.x];
+  if (st.done) return;
+  const SvdBlock& b = blocks[bq.x];
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const int C = b.C, q = bq.y;
+  const double aq = ws.G[q + (int64_t)q * C], eqq = ws.E[q + (int64_t)q * C] - 1.0;
+  const double tol = b.eig ? 4.0 * DBL_EPSILON * st.sa * st.shift : sqrt((double)b.R) * DBL_EPSILON;
+  const float sq = sqrtf((float)aq);
+  // a null space's off-diagonal elements: of W^T W they are squares of the
+  // error of V times the squared norm, of V^T B V times the norm
+  const double null_level = (step == 0 ? 1e-10 : step == 1 ? 1e-18 : 1e-27) * (b.eig ? sqrt(st.norm2) : st.norm2);
+  const double near = step == 0 ? 1e-6 : step == 1 ? 1e-11 : 0.0;
+  bool skipped = false;
+  float n2 = 0.0f, diag = 0.0f;
+  for (int p = lane; p < C; p += 32) {
+    if (p == q) continue;
+    const int64_t at = p > q ? p + (int64_t)q * C : q + (int64_t)p * C;  // lower triangle
+    const double ap = ws.G[p + (int64_t)p * C], e = ws.E[at];
+    const double g = ws.G[at] - 0.5 * e * (ap + aq);
+    float s = 0.0f;
+    if (fabs(g) > (b.eig ? tol : tol * (double)(sq * sqrtf((float)ap)))) {
+      const double d = aq - ap, h = 2.0 * g;
+      const double m = fmax(fabs(d), fabs(h));
+      const int ex = (__double2hiint(m) >> 20) & 0x7ff;
+      float t = 0.0f;
+      if (ex > 0 && ex < 2046) {
+        const double sc = __hiloint2double((2046 - ex) << 20, 0);  // m * sc in [1, 2)
+        const float df = (float)(d * sc), hf = (float)(h * sc);
+        const float sgn = df > 0.0f || (df == 0.0f && p < q) ? 1.0f : -1.0f;
+        t = sgn * hf / (fabsf(df) + sqrtf(fmaf(df, df, hf * hf)));
+      } else {
+        t = (float)(h / d);  // out of range: what comes of it fails the step's test
+      }
+      const double big = fmax(aq, ap);
+      if ((fabs(g) <= null_level && (fabsf(t) > 0.05f || (b.eig ? fabs(d) : big) <= null_level)) ||
+          m <= near * (b.eig ? sqrt(st.norm2) : big)) {
+        skipped = true;
+      } else {
+        const float c = rsqrtf(fmaf(t, t, 1.0f));
+        s = c * t;
+        diag -= s * s / (1.0f + c);  // c - 1
+      }
+    }
+    const float x = s - 0.5f * (float)e;
+    ws.X[p + (int64_t)q * C] = x;
+    n2 = fmaf(x, x, n2);
+  }
+  n2 = warp_sum(n2);
+  diag = warp_sum(diag);
+  skipped = __any_sync(0xffffffffu, skipped);
+  if (skipped && lane == 0) st.nulls[step] = 1;
+  if (lane == 0) {
+    const float x = diag - 0.5f * (float)eqq;
+    ws.X[q + (int64_t)q * C] = x;
+    n2 = fmaf(x, x, n2);
+    if (skipped && step < 2) n2 = fmaxf(n2, 1e-15f);  // not the last step
+    atomicMax(&st.xmax[step], __float_as_uint(n2));  // n2 >= 0 orders as its bits, a NaN above all
+    if (b.eig) ws.nrm[q] = st.unsa * (aq / (1.0 + eqq));  // lambda: the Rayleigh quotient
+  }
+}
+
+__device__ __forceinline__ bool last_step(const SvdState& st, int step) {
+  return __uint_as_float(st.xmax[step]) <= 1e-16f;  // every column of X at most 1e-8 long
+}
+
+// the refinement ended with nothing left to do
+__device__ __forceinline__ bool refined(const SvdState& st, const SvdBlock& b) {
+  return st.done > 0 && (b.eig || !st.nulls[st.done - 1]);
+}
+
+// V' = V + V X (kind 0), and on a block's last step W2 = W + W X (kind 1)
+__global__ void __launch_bounds__(kTileThreads)
+    svd_update_kernel(const SvdBlock* __restrict__ blocks, const SvdTile* __restrict__ tiles, double* __restrict__ work,
+                      SvdState* __restrict__ state, int step) {
+  __shared__ float ps[32][kTile + 1], xs[32][kTile + 1];
+  const SvdTile t = tiles[blockIdx.x];
+  SvdState& st = state[t.block];
+  const int done = *reinterpret_cast<volatile int*>(&st.done);
+  if (done && done != step + 1) return;  // this launch's own mark may be there already
+  const SvdBlock& b = blocks[t.block];
+  const bool last = last_step(st, step);
+  const bool lost = !(__uint_as_float(st.xmax[step]) <= 0.25f);  // no longer a small correction (or a NaN)
+  if (threadIdx.x == 0 && t.kind == 0 && t.i0 == 0 && t.j0 == 0 && (last || lost))
+    *reinterpret_cast<volatile int*>(&st.done) = last ? step + 1 : -1;
+  if (lost || (t.kind && (!last || b.eig))) return;
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const int C = b.C, m = t.kind ? b.R : C;
+  const double* src = t.kind ? ws.W : refine_v(ws, step);
+  const float* srcf = t.kind ? ws.W32 : refine_f(ws, step);
+  double* dst = t.kind ? ws.W2 : refine_v(ws, step + 1);
+  float* dstf = t.kind ? nullptr : refine_f(ws, step + 1);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int ml = min(kTile, m - t.i0), nl = min(kTile, C - t.j0);
+  float acc[4][2] = {};
+  for (int k0 = 0; k0 < C; k0 += 32) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = tid + kTileThreads * u;
+      const int hi = e >> 5, lo = e & 31;
+      ps[hi][lo] = k0 + hi < C && lo < ml ? __ldcg(srcf + t.i0 + lo + (int64_t)(k0 + hi) * m) : 0.0f;
+      xs[lo][hi] = k0 + lo < C && hi < nl ? __ldcg(ws.X + k0 + lo + (int64_t)(t.j0 + hi) * C) : 0.0f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(ps[k][ty + 8 * i], xs[k][tx + 16 * j], acc[i][j]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = ty + 8 * i, c = tx + 16 * j;
+      if (r >= ml || c >= nl) continue;
+      const int64_t at = t.i0 + r + (int64_t)(t.j0 + c) * m;
+      const double v = src[at] + (double)acc[i][j];
+      dst[at] = v;
+      if (dstf) dstf[at] = (float)v;
+    }
+}
+
+// Blocks the refinement did not finish.  Where it converged but left columns
+// at the rounding level (SVD), FP64 sweeps on its W and V, which mostly find
+// nothing to rotate.  Else the FP32 V made orthogonal in FP64 by two
+// Newton-Schulz steps (an orthogonality error e becomes ~1.5 e^2), W = A V
+// (eig: A = B + sigma I), and FP64 sweeps to convergence.  Leaves W and V in
+// place, the scaling undone, and the values (eig: |w_j| - sigma) in nrm.
+__global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThreads, 2)
+    svd_sweep_kernel(const SvdBlock* __restrict__ blocks, double* __restrict__ work,
+                     const SvdState* __restrict__ state, int* __restrict__ sweeps, long long* __restrict__ rotations,
+                     int* __restrict__ err) {
+  __shared__ unsigned long long nrot;
+  __shared__ SweepCtl ctl;
+  extern __shared__ double sm_pair[];  // the sweeps by column blocks: a block pair of W and V
+  cg::cluster_group cluster = cg::this_cluster();
+  const int crank = (int)cluster.block_rank();
+  const int bi = blockIdx.x / kSvdCluster;
+  const int done = state[bi].done;  // the same for the whole cluster
+  const SvdBlock b = blocks[bi];
+  if (refined(state[bi], b)) return;
+  const double sa = state[bi].sa, unsa = state[bi].unsa, shift = state[bi].shift;
+  const int R = b.R, C = b.C;
+  const int64_t CC = (int64_t)C * C;
+  const SvdWork ws(work + b.w, R, C);
+  double *W = ws.W, *V = ws.V, *A = ws.A, *G = ws.G, *nrm = ws.nrm;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ct = crank * kSvdThreads + tid;
+  const int cw = crank * (kSvdThreads / 32) + (tid >> 5);
+  constexpr int kCT = kSvdCluster * kSvdThreads;
+  constexpr int kCW = kSvdCluster * (kSvdThreads / 32);
+  if (tid == 0) {
+    nrot = 0;
+    ctl.flag[0] = ctl.flag[1] = 0;
+    ctl.any = 0;
+  }
+  if (done > 0) {  // the refined V (in V2 after an odd number of steps) and W
+    if (done & 1)
+      for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, __ldcg(ws.V2 + i));
+    for (int64_t i = ct; i < (int64_t)R * C; i += kCT) __stcg(W + i, __ldcg(ws.W2 + i));
+    cluster.sync();
+  } else {
+    // two Newton-Schulz steps through the G buffer, the first one's product in
+    // W's buffer (free until W = A V)
+    for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, (double)__ldcg(ws.V32 + i));
+    if (b.eig)
+      for (int j = ct; j < C; j += kCT) __stcg(A + j + (int64_t)j * R, __ldcg(A + j + (int64_t)j * R) + shift);
+    cluster.sync();
+    newton_schulz_factor(V, C, G, cw, lane);
+    cluster.sync();
+    gemm_cols(V, C, C, G, W, 1.0, cw, lane);
+    cluster.sync();
+    newton_schulz_factor(W, C, G, cw, lane);
+    cluster.sync();
+    gemm_cols(W, C, C, G, V, 1.0, cw, lane);
+    cluster.sync();
+    gemm_cols(A, R, C, V, W, sa, cw, lane);  // W = (sa A) V
+    cluster.sync();
   }
 
-  // V = V32 made orthogonal in FP64: two Newton-Schulz steps through the G
-  // buffer, the first one's product in W's buffer (free until W = A V)
-  for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, (double)__ldcg(V32 + i));
-  cluster.sync();
-  newton_schulz_factor(V, C, G, cw, lane);
-  cluster.sync();
-  gemm_cols(V, C, C, G, W, 1.0, cw, lane);
-  cluster.sync();
-  newton_schulz_factor(W, C, G, cw, lane);
-  cluster.sync();
-  gemm_cols(W, C, C, G, V, 1.0, cw, lane);
-  cluster.sync();
-  gemm_cols(A, R, C, V, W, sa, cw, lane);  // W = (sa A) V
-  cluster.sync();
-
+  int* flag0 = cluster.map_shared_rank(ctl.flag, 0);
+  unsigned long long rot64 = 0;
+  bool conv;
+  int gsweep = 0;
   const double tol64 = sqrt((double)R) * DBL_EPSILON;
   int sw64;
   switch (b.bw64 ? (R + 31) / 32 : 0) {
 #define SYM_BLOCKED(NR)                                                                                          \
   case NR:                                                                                                        \
-    sw64 = jacobi_sweeps_blocked<double, NR>(W, V, nrm, R, C, b.bw64, kMaxSweeps, tol64, cluster, &ctl, flag0,   \
+    sw64 = jacobi_sweeps_blocked<double, NR, kSvdThreads>(W, V, nrm, R, C, b.bw64, kMaxSweeps, tol64, cluster, &ctl, flag0,   \
                                              crank, lane, gsweep, rot64, conv, kBigRotation, sm_pair);          \
     break;
     SYM_BLOCKED(1)
@@ -747,14 +1267,12 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     SYM_BLOCKED(12)
 #undef SYM_BLOCKED
     default:
-      sw64 = jacobi_sweeps<double>(W, V, nrm, R, C, kMaxSweeps, tol64, cluster, &ctl, flag0, crank, cw, lane, gsweep,
+      sw64 = jacobi_sweeps<double, kSvdThreads>(W, V, nrm, R, C, kMaxSweeps, tol64, cluster, &ctl, flag0, crank, cw, lane, gsweep,
                                    rot64, conv, kBigRotation);
   }
-  if (lane == 0 && rot32) atomicAdd(cluster.map_shared_rank(&nrot[0], 0), rot32);
-  if (lane == 0 && rot64) atomicAdd(cluster.map_shared_rank(&nrot[1], 0), rot64);
+  if (lane == 0 && rot64) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot64);
 
   // undo the scaling (a power of two: exact) and take the column norms
-  constexpr int kCW = kSvdCluster * kSvdWarps;
   for (int j = cw; j < C; j += kCW) {
     double* wj = W + (int64_t)j * R;
     double a = 0.0;
@@ -764,35 +1282,61 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
       a = fma(x, x, a);
     }
     a = warp_sum(a);
-    if (lane == 0) __stcg(nrm + j, sqrt(a));
+    if (lane == 0) __stcg(nrm + j, sqrt(a) - shift);
   }
-  cluster.sync();  // norms written; the rotation counts have arrived at rank 0
+  cluster.sync();  // the rotation counts have arrived at rank 0
   if (crank == 0 && tid == 0) {
     if (!conv) atomicExch(err, SYM_ERR_NUMERIC);
     sweeps[2 * b.slot] = sw64;
-    sweeps[2 * b.slot + 1] = sw32;
-    rotations[2 * b.slot] = (long long)nrot[1];
-    rotations[2 * b.slot + 1] = (long long)nrot[0];
+    rotations[2 * b.slot] = (long long)nrot;
   }
-  for (int j = ct; j < C; j += kCT) {
-    const double v = __ldcg(nrm + j);
-    int rank = 0;
-    if (!b.eig) {
-      for (int i = 0; i < C; ++i) {
-        const double u = __ldcg(nrm + i);
-        rank += (u > v) || (u == v && i < j);
-      }
-      S[b.s + rank] = v / b.vscale;
-      Ss[rank] = v;
-    } else {  // lambda = |w| - sigma, ranked by |lambda| (ties: larger lambda, then column)
-      const double lj = v - shift, aj = fabs(lj);
-      for (int i = 0; i < C; ++i) {
-        const double li = __ldcg(nrm + i) - shift, ai = fabs(li);
-        rank += (ai > aj) || (ai == aj && (li > lj || (li == lj && i < j)));
-      }
-      S[b.s + rank] = b.sgn * lj / b.vscale;
-      Ss[rank] = lj;
+}
+
+// Refined blocks: W (the last step's W2, scaling undone) and its column norms,
+// and V, to their places; a warp per column.
+__global__ void __launch_bounds__(256)
+    svd_place_kernel(const SvdBlock* __restrict__ blocks, const int2* __restrict__ cols, int ncols,
+                     double* __restrict__ work, const SvdState* __restrict__ state, int* __restrict__ sweeps) {
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (w >= ncols) return;
+  const int2 bq = cols[w];
+  const SvdState& st = state[bq.x];
+  const SvdBlock& b = blocks[bq.x];
+  if (!refined(st, b)) return;
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const int R = b.R, C = b.C, j = bq.y;
+  if (!b.eig) {
+    double a = 0.0;
+    for (int i = lane; i < R; i += 32) {
+      const double x = st.unsa * ws.W2[i + (int64_t)j * R];
+      ws.W[i + (int64_t)j * R] = x;
+      a = fma(x, x, a);
     }
+    a = warp_sum(a);
+    if (lane == 0) ws.nrm[j] = sqrt(a);
+  }
+  if (st.done & 1)
+    for (int i = lane; i < C; i += 32) ws.V[i + (int64_t)j * C] = ws.V2[i + (int64_t)j * C];
+  if (j == 0 && lane == 0) sweeps[2 * b.slot] = st.done;
+}
+
+// Values in descending order (eig: of |lambda|; ties: the larger lambda, then
+// the column) with their permutation; a thread per column.
+__global__ void __launch_bounds__(128)
+    svd_rank_kernel(const SvdBlock* __restrict__ blocks, double* __restrict__ work, double* __restrict__ S,
+                    int* __restrict__ perm) {
+  const SvdBlock& b = blocks[blockIdx.x];
+  const SvdWork ws(work + b.w, b.R, b.C);
+  const int C = b.C;
+  for (int j = blockIdx.y * 128 + threadIdx.x; j < C; j += gridDim.y * 128) {
+    const double v = ws.nrm[j], av = fabs(v);
+    int rank = 0;
+    for (int i = 0; i < C; ++i) {
+      const double u = ws.nrm[i], au = fabs(u);
+      rank += (au > av) || (au == av && (u > v || (u == v && i < j)));
+    }
+    S[b.s + rank] = (b.eig ? b.sgn : 1.0) * v / b.vscale;
+    ws.Ss[rank] = v;
     perm[b.s + rank] = j;
   }
 }
@@ -932,8 +1476,14 @@ struct SvdPlan {
   bool dry = false;
   bool bonded = false;
 
+  std::vector<SvdTile> tiles[3];  // refinement products: W; the two Gram matrices; V' and W2
+  std::vector<int2> columns;      // (block, column)
+
   DeviceArena arena;
   SvdBlock* d_blocks = nullptr;
+  SvdTile* d_tiles[3] = {nullptr, nullptr, nullptr};
+  int2* d_cols = nullptr;
+  SvdState* state = nullptr;
   double* work = nullptr;
   int* perm = nullptr;
   int* sweeps = nullptr;
@@ -1016,12 +1566,12 @@ std::unique_ptr<SvdPlan> plan_svd(const Tensor& T, int nrow, bool eig) {
     b.sgn = (eig && T.group == SYM_SU2 && T.legs[0].dir == -1 && (x & 1)) ? -1.0 : 1.0;
     if (eig && m != n) fail(SYM_ERR_ARG, "internal: eigendecomposition block is not square");
     // FP32 sweeps by column blocks when a block pair of W and V fits the
-    // shared memory two CTAs of an SM can have, rows up to 12 per lane
+    // shared memory two CTAs of an SM can have, rows up to 20 (FP64: 12) per lane
     {
       const int bw = (b.C + kColBlocks - 1) / kColBlocks;
       const int64_t bytes = 2 * (int64_t)bw * (b.R + b.C + 1) * (int64_t)sizeof(float);
-      const bool ok = b.C >= kColBlocks * 2 && b.R <= 32 * 12;
-      b.bw = (ok && bytes <= kSvdSmem32Max) ? bw : 0;
+      const bool ok = b.C >= kColBlocks * 2 && b.R <= 32 * 12;  // FP64
+      b.bw = (b.C >= kColBlocks * 2 && b.R <= 32 * 20 && bytes <= kSvdSmem32Max) ? bw : 0;
       // FP64 by column blocks for the SVD only: on the shifted symmetric blocks of
       // the eigendecomposition that order took up to 6 FP64 sweeps where the
       // order by pairs takes 4 (two-site density matrix: 29.8 against 29.0 ms;
@@ -1031,9 +1581,7 @@ std::unique_ptr<SvdPlan> plan_svd(const Tensor& T, int nrow, bool eig) {
     }
     b.w = P->work_elems;
     b.s = P->nsv;
-    // W, V, norms, sorted S, A, the Newton-Schulz factor (doubles), W and V in FP32
-    const int64_t rc = (int64_t)b.R * b.C, cc = (int64_t)b.C * b.C;
-    P->work_elems += 2 * rc + 2 * cc + 2 * (int64_t)b.C + (rc + cc + 1) / 2 + 1;
+    P->work_elems += SvdWork::elems(b.R, b.C);
     P->nsv += b.C;
     slot_of[x] = b.slot;
     P->blocks.push_back(b);
@@ -1061,9 +1609,37 @@ std::unique_ptr<SvdPlan> plan_svd(const Tensor& T, int nrow, bool eig) {
     const SvdBlock &A = P->blocks[a], &B = P->blocks[c];
     return (double)A.R * A.C * A.C > (double)B.R * B.C * B.C;
   });
+  // refinement tiles, the blocks in launch order (decreasing work)
+  for (size_t o = 0; o < P->order.size(); ++o) {
+    const SvdBlock& b = P->blocks[P->order[o]];
+    for (int j = 0; j < b.C; j += kTile)
+      for (int i = 0; i < b.R; i += kTile) {
+        P->tiles[0].push_back({(int)o, i, j, 0});
+        if (!eig) P->tiles[2].push_back({(int)o, i, j, 1});
+      }
+    for (int j = 0; j < b.C; j += kTile)
+      for (int i = 0; i < b.C; i += kTile) {
+        if (i >= j) {
+          P->tiles[1].push_back({(int)o, i, j, 0});
+          P->tiles[1].push_back({(int)o, i, j, 1});
+        }
+        P->tiles[2].push_back({(int)o, i, j, 0});
+      }
+    for (int j = 0; j < b.C; ++j) P->columns.push_back(make_int2((int)o, j));
+  }
   const char* dry = std::getenv("SYM_PLAN_DRYRUN");
   P->dry = dry && dry[0] == '1';
   if (!P->dry) {
+    for (int k = 0; k < 3; ++k) {
+      P->d_tiles[k] = static_cast<SvdTile*>(P->arena.alloc(P->tiles[k].size() * sizeof(SvdTile), false));
+      cudaError_t e = cudaMemcpy(P->d_tiles[k], P->tiles[k].data(), P->tiles[k].size() * sizeof(SvdTile),
+                                 cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) fail(SYM_ERR_CUDA, std::string("svd plan upload: ") + cudaGetErrorString(e));
+    }
+    P->d_cols = static_cast<int2*>(P->arena.alloc(P->columns.size() * sizeof(int2), false));
+    cudaError_t ec = cudaMemcpy(P->d_cols, P->columns.data(), P->columns.size() * sizeof(int2), cudaMemcpyHostToDevice);
+    if (ec != cudaSuccess) fail(SYM_ERR_CUDA, std::string("svd plan upload: ") + cudaGetErrorString(ec));
+    P->state = static_cast<SvdState*>(P->arena.alloc(P->blocks.size() * sizeof(SvdState), true));
     P->d_blocks = static_cast<SvdBlock*>(P->arena.alloc(P->blocks.size() * sizeof(SvdBlock), false));
     P->work = static_cast<double*>(P->arena.alloc(P->work_elems * sizeof(double), true));
     P->perm = static_cast<int*>(P->arena.alloc(P->nsv * sizeof(int), true));
@@ -1134,19 +1710,42 @@ int sym_svd_blocks(sym_svd plan, int* x, int* m, int* n) {
 namespace {
 void launch_jacobi(sym::SvdPlan& P, const double* T, double* S, void* stream) {
   if (P.dry) sym::fail(SYM_ERR_UNSUPPORTED, "plan was built with SYM_PLAN_DRYRUN=1 and cannot run");
-  static int attr_set = -1;  // dynamic shared memory the kernel is allowed (set once to the maximum)
+  static int attr_set = -1;  // dynamic shared memory the kernels are allowed (set once to the maximum)
   if (attr_set < 0) {
-    cudaError_t e = cudaFuncSetAttribute(sym::svd_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         sym::kSvdSmem32Max);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(sym::svd_jacobi_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) sym::fail(SYM_ERR_CUDA, std::string("svd_jacobi_kernel attribute: ") + cudaGetErrorString(e));
+    auto allow = [](auto* k) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sym::kSvdSmem32Max);
+      return e == cudaSuccess ? cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
+    };
+    cudaError_t e = allow(sym::svd_jacobi_kernel);
+    if (e == cudaSuccess) e = allow(sym::svd_sweep_kernel);
+    if (e != cudaSuccess) sym::fail(SYM_ERR_CUDA, std::string("SVD kernel attribute: ") + cudaGetErrorString(e));
     attr_set = 1;
   }
-  sym::svd_jacobi_kernel<<<(unsigned)P.blocks.size() * sym::kSvdCluster, sym::kSvdThreads, (size_t)P.smem32,
-                           static_cast<cudaStream_t>(stream)>>>(
-      P.d_blocks, P.d_pieces, T, P.work, S, P.perm, P.sweeps, P.rotations, sym::device_error_word());
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const unsigned nb = (unsigned)P.blocks.size(), ncols = (unsigned)P.columns.size();
+  const unsigned warps = (ncols + 7) / 8;  // CTAs of the warp-per-column kernels
+  sym::svd_jacobi_kernel<<<nb * sym::kSvdCluster, sym::kThreads32, (size_t)P.smem32, s>>>(
+      P.d_blocks, P.d_pieces, T, P.work, P.state, P.sweeps, P.rotations);
   check_launch("svd_jacobi_kernel");
+  for (int step = 0; step < sym::kMaxRefine; ++step) {
+    sym::svd_av_kernel<<<(unsigned)P.tiles[0].size(), sym::kTileThreads, 0, s>>>(P.d_blocks, P.d_tiles[0], P.work,
+                                                                               P.state, step);
+    sym::svd_gram_kernel<<<(unsigned)P.tiles[1].size(), sym::kTileThreads, 0, s>>>(P.d_blocks, P.d_tiles[1], P.work,
+                                                                                 P.state, step);
+    sym::svd_correction_kernel<<<warps, 256, 0, s>>>(P.d_blocks, P.d_cols, (int)ncols, P.work, P.state, step);
+    sym::svd_update_kernel<<<(unsigned)P.tiles[2].size(), sym::kTileThreads, 0, s>>>(P.d_blocks, P.d_tiles[2], P.work,
+                                                                                   P.state, step);
+    check_launch("SVD refinement");
+  }
+  sym::svd_sweep_kernel<<<nb * sym::kSvdCluster, sym::kSvdThreads, (size_t)P.smem32, s>>>(
+      P.d_blocks, P.work, P.state, P.sweeps, P.rotations, sym::device_error_word());
+  check_launch("svd_sweep_kernel");
+  sym::svd_place_kernel<<<warps, 256, 0, s>>>(P.d_blocks, P.d_cols, (int)ncols, P.work, P.state, P.sweeps);
+  int cmax = 1;
+  for (const auto& b : P.blocks) cmax = std::max(cmax, b.C);
+  sym::svd_rank_kernel<<<dim3(nb, (unsigned)std::min(64, (cmax + 127) / 128)), 128, 0, s>>>(P.d_blocks, P.work, S,
+                                                                                          P.perm);
+  check_launch("svd_rank_kernel");
 }
 }  // namespace
 

@@ -490,7 +490,8 @@ class SVDPlan:
 
     def stats(self, fp32=False):
         """(sweeps, rotations) per block of the last execute, of its FP64
-        sweeps or (fp32) of its FP32 sweeps (synchronizes)."""
+        part (refinement steps and 0, or, for a block finished by FP64
+        sweeps, those) or (fp32) of its FP32 sweeps (synchronizes)."""
         sw = (ctypes.c_int * self.nblocks)()
         rot = (ctypes.c_int64 * self.nblocks)()
         L.check(L.lib.sym_svd_stats(self._h, 1 if fp32 else 0, sw, rot))
@@ -501,25 +502,29 @@ class SVDPlan:
 
         Per sweep one FMA per row of every pair visited and the squared
         column norms (one FMA per element of W) when the kernel carries the
-        norms through the rotations (blocks of at most 384 rows), else three
-        FMAs per row of every pair visited; per rotation 4 multiply-adds per
-        row of W and V; in FP64 also the two Newton-Schulz steps (2 C^3 FMAs
-        each), W = A V (R C^2) and the column norms.  An FMA counts 2."""
-        out = []
-        for fp32 in (False, True):
-            sweeps, rotations = self.stats(fp32)
-            f = 0.0
-            for m, n, sw, rot in zip(self.m, self.n, sweeps, rotations):
-                R, C = max(m, n), min(m, n)
-                if R <= 384:
-                    f += sw * ((C * (C - 1) // 2) * 2.0 * R + 2.0 * R * C)
-                else:
-                    f += sw * (C * (C - 1) // 2) * 6.0 * R
-                f += rot * 6.0 * (R + C)
-                if not fp32:
-                    f += 2.0 * (4.0 * C ** 3 + R * C * C + R * C)
-            out.append(f)
-        return tuple(out)
+        norms through the rotations, else three FMAs per row of every pair
+        visited; per rotation 4 multiply-adds per row of W and V.  FP64: a
+        refined block (no rotations) takes W = A V, half of W^T W and half of
+        V^T V per step; a block finished by FP64 sweeps those sweeps and
+        W = A V.  FP32: the sweeps, and V X per refinement step.  An FMA
+        counts 2."""
+        s64, r64 = self.stats(False)
+        s32, r32 = self.stats(True)
+        f64 = f32 = 0.0
+
+        def sweep(R, C, sw, rot, carried):
+            pairs = C * (C - 1) // 2
+            return sw * (pairs * 2.0 * R + 2.0 * R * C if carried else pairs * 6.0 * R) + rot * 6.0 * (R + C)
+
+        for m, n, a, ra, b, rb in zip(self.m, self.n, s64, r64, s32, r32):
+            R, C = max(m, n), min(m, n)
+            f32 += sweep(R, C, b, rb, R <= 640)
+            if ra:
+                f64 += sweep(R, C, a, ra, R <= 384) + 2.0 * R * C * C
+            else:
+                f64 += a * (3.0 * R * C * C + C ** 3)
+                f32 += a * 2.0 * C ** 3
+        return f64, f32
 
     def truncation(self, S_host, chi=None, cutoff=0.0):
         """keep per block (ascending x) for a host copy of execute's S."""
