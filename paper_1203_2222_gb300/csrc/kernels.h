@@ -246,8 +246,9 @@ enum SimtShape { SIMT_64x64 = 0, SIMT_256x16 = 1, SIMT_THIN = 2, SIMT_ROWS = 3, 
 // Launchers (return cudaError_t as int).
 // mode: the items the launch holds, which picks the kernel variant.
 // kBoxGeneral: any item; kBoxFlat: only flat linear items (kSelFlat without
-// kSelTile); kBoxRecouple: only flat linear and fused recoupling items.
-constexpr int kBoxGeneral = 0, kBoxFlat = 1, kBoxRecouple = 2;
+// kSelTile); kBoxRecouple: only flat linear and fused recoupling items;
+// kBoxTile: only flat items, linear or tiles.
+constexpr int kBoxGeneral = 0, kBoxFlat = 1, kBoxRecouple = 2, kBoxTile = 3;
 int launch_box(bool src_f64, bool dst_f64, int mode, const BoxItem* items, int nitems, const Term* terms,
                const BoxPtrs& ptrs, void* stream);
 int launch_gemm_simt(bool f64, int shape, const GemmSectorSimt* secs, const GemmTile* tiles, int ntiles,

@@ -683,9 +683,12 @@ void Plan::upload(bool device) {
   if (item_bytes_prefix.size() != items.size() + 1) item_bytes_prefix.assign(items.size() + 1, 0.0);
   for (size_t i = 0; i < items.size(); ++i) item_bytes_prefix[i + 1] += item_bytes_prefix[i];
   flat_prefix.assign(items.size() + 1, 0);
+  tile_prefix.assign(items.size() + 1, 0);
   recouple_prefix.assign(items.size() + 1, 0);
   for (size_t i = 0; i < items.size(); ++i) {
     flat_prefix[i + 1] = flat_prefix[i] + ((items[i].sel & (kSelFlat | kSelTile)) == kSelFlat ? 1 : 0);
+    tile_prefix[i + 1] =
+        tile_prefix[i] + ((items[i].sel & (kSelFlat | kSelTile)) == (kSelFlat | kSelTile) ? 1 : 0);
     recouple_prefix[i + 1] = recouple_prefix[i] + ((items[i].sel & kSelRecouple) ? 1 : 0);
   }
   tile_flops_prefix.assign(tiles.size() + 1, 0.0);
@@ -2534,7 +2537,11 @@ int run_box(Plan& p, Range r, const BoxPtrs& ptrs, void* stream, int phase) {
   p.last_launches++;
   const int flat = p.flat_prefix[r.first + r.count] - p.flat_prefix[r.first];
   const int rec = p.recouple_prefix[r.first + r.count] - p.recouple_prefix[r.first];
-  const int mode = flat == r.count ? kBoxFlat : flat + rec == r.count ? kBoxRecouple : kBoxGeneral;
+  const int tile = p.tile_prefix[r.first + r.count] - p.tile_prefix[r.first];
+  const int mode = flat == r.count         ? kBoxFlat
+                   : flat + rec == r.count ? kBoxRecouple
+                   : flat + tile == r.count ? kBoxTile
+                                            : kBoxGeneral;
   ProfScope ps(p, phase, mode == kBoxFlat ? SYM_KERNEL_BOX_FLAT : SYM_KERNEL_BOX, stream,
                p.item_bytes_prefix[r.first + r.count] - p.item_bytes_prefix[r.first], 0.0);
   return cuda_code(launch_box(p.f64(), p.f64(), mode, p.d_items + r.first, r.count, p.d_terms, ptrs, stream),
