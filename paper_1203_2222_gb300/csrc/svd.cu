@@ -31,11 +31,11 @@
 //   scaled by S.
 //
 // Measured (GB300, two-site tensor D = 2048: 41 blocks up to 272 x 272):
-// execute and factors 19.3 -> 7.8 ms; the two-site density matrix (42 blocks)
-// 25.6 -> 9.0 ms.  Before, two FP64 sweeps (eig: four) in serial rounds on each
+// execute and factors 19.3 -> 6.6 ms; the two-site density matrix (42 blocks)
+// 25.6 -> 8.0 ms.  Before, two FP64 sweeps (eig: four) in serial rounds on each
 // block's own cluster took 14 ms (20 ms); the refinement takes 2.6 ms, bound
-// by FP64 (two multiply-adds a clock of an SM; 70% of it), the FP32 sweeps 5 to
-// 6 ms, bound by shared memory and the rounds' barriers.
+// by FP64 (two multiply-adds a clock of an SM; 70% of it), the FP32 sweeps 3.8
+// to 4.7 ms, bound by the latencies of a round.
 //
 // The same kernels give the blockwise eigendecomposition of a symmetric
 // tensor seen as a square matrix (Ch. 5, Eq. spectral, by blocks as the
@@ -72,6 +72,7 @@ namespace cg = cooperative_groups;
 namespace sym {
 namespace {
 
+constexpr int kMaxGram = 14;  // columns of a block the FP32 sweeps through Gram matrices take (C <= 448)
 constexpr int kSvdThreads = 256;  // FP64 sweeps (128 registers a thread, two CTAs an SM)
 // FP32 sweeps: a round has up to 12 column pairs a CTA, one a warp -- with 8
 // warps the 9 pairs of a 272-column block took two passes
@@ -79,9 +80,11 @@ constexpr int kThreads32 = 384;
 // CTAs per diagonal block (16: a cluster size above the portable 8, allowed
 // by a function attribute; two CTAs of the kernel fit on an SM)
 constexpr int kSvdCluster = 16;
-// dynamic shared memory a Jacobi CTA may take for the FP32 sweeps by column
-// blocks (two CTAs of 256 threads and 128 registers share an SM)
-constexpr int kSvdSmem32Max = 100 * 1024;
+// dynamic shared memory a CTA may take for the FP32 and the FP64 sweeps by
+// column blocks, so that two share an SM (with one, 41 blocks take waves of
+// clusters: 6.7 against 3.8 ms)
+constexpr int kSvdSmem32Max = 112 * 1024;
+constexpr int kSvdSmem64Max = 100 * 1024;
 constexpr int kMaxSweeps = 64;    // FP64 sweeps before a block counts as not converged
 constexpr int kMaxSweeps32 = 40;  // FP32 sweeps (their result only seeds the FP64 ones)
 // An FP64 sweep whose rotations all had |w_p.w_q| <= kBigRotation |w_p| |w_q|
@@ -457,7 +460,7 @@ __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* n
   return fabs(g) > big * sab ? 2 : 1;
 }
 
-// FP32 sweeps by column blocks: the C columns form kColBlocks blocks of bw
+// FP64 sweeps by column blocks: the C columns form kColBlocks blocks of bw
 // (the last ones ragged or empty), and a sweep is the tournament over the
 // blocks (kColBlocks - 1 rounds of kSvdCluster disjoint block pairs).  In a
 // round, CTA k of the cluster takes block pair k -- the columns of W and V
@@ -577,6 +580,225 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
     if (f && threadIdx.x == 0) atomicOr(flag0 + (gs & 1), f);
     cluster.sync();
     if (threadIdx.x == 0) {
+      ctl->any = flag0[gs & 1];
+      if (crank == 0) ctl->flag[(gs + 1) & 1] = 0;
+    }
+    __syncthreads();
+    conv = !(ctl->any & 2);
+    __syncthreads();
+  }
+  return sweeps;
+}
+
+// FP32 sweeps by column blocks through Gram matrices.  The order of the pairs
+// is that of jacobi_sweeps_blocked (a CTA takes a block pair, N = 2 BW columns
+// or fewer, a round), but the rotations of a round act on the N x N Gram
+// matrix of the block pair's W columns and are collected in Q, which then
+// multiplies the columns of W and V once: a pair costs a few operations on
+// shared values instead of a pass over its columns in shared memory, and a
+// set of disjoint pairs one barrier.  The starting point needs no more than
+// that: rotated Gram entries carry FP32's rounding relative to their columns'
+// norms, and every round forms them afresh.  The FP32 kernel on the blocks of
+// a U(1) two-site tensor of D = 2048 took 4.98 ms with the columns rotated a pair a warp
+// (a pass over both columns in shared memory a pair) and takes 3.78 ms; on the
+// density matrix of the eigendecomposition 5.82 and 4.69 ms.  A round is bound
+// by latencies: 1.2-2.4 us for the columns from L2, 1.6 the Gram matrix, 3 the
+// nine sets of rotations, 2-4 the product, 1.2 the cluster's barrier.
+template <int BW>
+struct GramSmem {
+  static constexpr int N = 2 * BW, GP = N + 1, QP = (N + 3) / 4 * 4;
+};
+// W columns are gram_pitch apart: eight rows of four column pairs, what a warp
+// reads for the Gram matrix, fall on different banks
+__host__ __device__ inline int gram_pitch(int R) { return (R + 3) / 8 * 8 + 4; }
+__host__ __device__ inline int64_t gram_floats(int R, int C, int bw) {
+  const int64_t n = 2 * bw, qp = (n + 3) / 4 * 4;
+  return n * gram_pitch(R) + n * qp + 2 * n * (n + 1) + n * C;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {  // of x >= 0, no branch
+  return x * rsqrtf(fmaxf(x, FLT_MIN));
+}
+template <int BW>
+__device__ int jacobi_sweeps_gram(float* W, float* V, int R, int C, int bw, int max_sweeps, float tol,
+                                  cg::cluster_group& cluster, SweepCtl* ctl, int* flag0, int crank, int lane,
+                                  int& gsweep, unsigned long long& myrot, bool& conv, float big_tol, float* sm) {
+  using GS = GramSmem<BW>;
+  constexpr int N = GS::N, GP = GS::GP, QP = GS::QP, NT = kThreads32, NW = NT / 32;
+  const int RP = gram_pitch(R);
+  float* Ws = sm;
+  float* Qt = Ws + (size_t)N * RP;  // Q transposed: row j holds column j's coefficients (RP, N QP multiples of 4)
+  float* G0 = Qt + N * QP;
+  float* Vs = G0 + 2 * N * GP;
+  // warps 0 .. GW-1 rotate the Gram matrix, GW .. GW+QW-1 Q
+  constexpr int GW = (BW * BW + 31) / 32, QW = (BW * QP / 4 + 31) / 32;
+  static_assert(GW + QW <= NW, "threads of a set");
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int gx = tid / BW, gy = tid % BW;
+  const int qx = tid < 32 * GW ? BW : (tid - 32 * GW) / (QP / 4), qy = tid < 32 * GW ? 0 : (tid - 32 * GW) % (QP / 4);
+  int sweeps = 0;
+  conv = C < 2;
+  while (!conv && sweeps < max_sweeps) {
+    ++sweeps;
+    const int gs = ++gsweep;
+    int did = 0, big = 0;
+    for (int r = 0; r < kColBlocks - 1; ++r) {
+      const int k = crank;
+      const int P = k == 0 ? r : (r + k) % (kColBlocks - 1);
+      const int Q = k == 0 ? kColBlocks - 1 : (r - k + kColBlocks - 1) % (kColBlocks - 1);
+      const int p0 = P * bw, np = max(0, min(bw, C - p0));
+      const int q0 = Q * bw, nq = max(0, min(bw, C - q0));
+      if (np + nq >= 2) {
+        // columns of W and V (absent ones: zeros, which nothing rotates)
+        for (int c = warp; c < N; c += NW) {
+          const int n = c < BW ? np : nq, d = c < BW ? c : c - BW;
+          const int64_t col = (c < BW ? p0 : q0) + d;
+          const float *w = W + col * R, *v = V + col * C;
+          if (d < n) {
+            float x[12], y[12];
+            for (int i = lane; i < max(R, C); i += 384) {
+#pragma unroll
+              for (int u = 0; u < 12; ++u) {
+                x[u] = i + 32 * u < R ? __ldcg(w + i + 32 * u) : 0.0f;
+                y[u] = i + 32 * u < C ? __ldcg(v + i + 32 * u) : 0.0f;
+              }
+#pragma unroll
+              for (int u = 0; u < 12; ++u) {
+                if (i + 32 * u < R) Ws[c * RP + i + 32 * u] = x[u];
+                if (i + 32 * u < C) Vs[c * C + i + 32 * u] = y[u];
+              }
+            }
+          } else {
+            for (int i = lane; i < R; i += 32) Ws[c * RP + i] = 0.0f;
+            for (int i = lane; i < C; i += 32) Vs[c * C + i] = 0.0f;
+          }
+        }
+        for (int i = tid; i < N * QP; i += NT) Qt[i] = i / QP == i % QP ? 1.0f : 0.0f;
+        __syncthreads();
+        // Gram matrix: eight lanes per 2 x 2 tile of its upper triangle
+        for (int t = tid >> 3; t < (BW * (BW + 1) / 2 + 3) / 4 * 4; t += NT / 8) {
+          int ti = 0, rest = min(t, BW * (BW + 1) / 2 - 1);
+          while (rest >= BW - ti) rest -= BW - ti, ++ti;
+          const int i0 = 2 * ti, j0 = 2 * (ti + rest);
+          const float *a = Ws + i0 * RP, *b = Ws + j0 * RP;
+          float g[4] = {};
+#pragma unroll 4
+          for (int row = lane & 7; row < R; row += 8) {
+            const float a0 = a[row], a1 = a[row + RP], b0 = b[row], b1 = b[row + RP];
+            g[0] = fmaf(a0, b0, g[0]);
+            g[1] = fmaf(a0, b1, g[1]);
+            g[2] = fmaf(a1, b0, g[2]);
+            g[3] = fmaf(a1, b1, g[3]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) g[u] += __shfl_xor_sync(0xffffffffu, g[u], o);
+          }
+          if ((lane & 7) < 4) {
+            const int u = lane & 7, x = i0 + (u >> 1), y = j0 + (u & 1);
+            const float v = u == 0 ? g[0] : u == 1 ? g[1] : u == 2 ? g[2] : g[3];
+            G0[x * GP + y] = v;
+            G0[y * GP + x] = v;
+          }
+        }
+        __syncthreads();
+        // Round 0: every pair of the N columns (a tournament); later rounds:
+        // the cross pairs.  Every thread forms the angles it needs from the
+        // old Gram matrix and writes the new one: one barrier a set.
+        const int inner = r == 0 ? N - 1 : BW;
+        int rotated = 0;
+        for (int ir = 0; ir < inner && tid < 32 * (GW + QW); ++ir) {
+          const float* G = G0 + (ir & 1) * N * GP;
+          float* H = G0 + (~ir & 1) * N * GP;
+          auto pair = [&](int t, int& p, int& q) {
+            if (r == 0) {
+              p = t == 0 ? ir : ir + t >= N - 1 ? ir + t - (N - 1) : ir + t;
+              q = t == 0 ? N - 1 : ir - t < 0 ? ir - t + N - 1 : ir - t;
+            } else {
+              p = t;
+              q = BW + (t + ir >= BW ? t + ir - BW : t + ir);
+            }
+          };
+          // no branches: a warp's threads look at different pairs, a thread at two
+          auto angle = [&](int p, int q, float& c, float& s) {  // 0: no rotation, 1, or 2: a large one
+            const float a = G[p * GP + p], b = G[q * GP + q], g = G[p * GP + q];
+            const float sab = sqrt_approx(a * b), d = b - a, h = 2.0f * g;
+            const float t = __fdividef(copysignf(1.0f, d) * h, fabsf(d) + sqrt_approx(fmaf(d, d, h * h)));
+            const bool on = fabsf(g) > tol * sab;
+            c = on ? rsqrtf(fmaf(t, t, 1.0f)) : 1.0f;
+            s = on ? c * t : 0.0f;
+            return on ? (fabsf(g) > big_tol * sab ? 2 : 1) : 0;
+          };
+          int p, q;
+          float c, s;
+          if (gx < BW) {  // a 2 x 2 block of the Gram matrix: both sides' rotations
+            int u, v;
+            float d, t;
+            pair(gx, p, q);
+            pair(gy, u, v);
+            const int did_pair = angle(p, q, c, s);
+            angle(u, v, d, t);
+            const float gpu = G[p * GP + u], gpv = G[p * GP + v], gqu = G[q * GP + u], gqv = G[q * GP + v];
+            const float pu = c * gpu - s * gqu, pv = c * gpv - s * gqv;
+            const float qu = s * gpu + c * gqu, qv = s * gpv + c * gqv;
+            H[p * GP + u] = d * pu - t * pv;
+            H[p * GP + v] = t * pu + d * pv;
+            H[q * GP + u] = d * qu - t * qv;
+            H[q * GP + v] = t * qu + d * qv;
+            if (gx == gy) {
+              rotated += did_pair != 0;
+              big |= did_pair == 2;
+            }
+          } else if (qx < BW) {  // four rows of a pair's columns of Q
+            pair(qx, p, q);
+            angle(p, q, c, s);
+            float4 *qp = reinterpret_cast<float4*>(Qt + p * QP) + qy, *qq = reinterpret_cast<float4*>(Qt + q * QP) + qy;
+            const float4 a = *qp, b = *qq;
+            *qp = make_float4(c * a.x - s * b.x, c * a.y - s * b.y, c * a.z - s * b.z, c * a.w - s * b.w);
+            *qq = make_float4(s * a.x + c * b.x, s * a.y + c * b.y, s * a.z + c * b.z, s * a.w + c * b.w);
+          }
+          // only the warps at work wait for one another
+          asm volatile("bar.sync 1, %0;" ::"n"(32 * (GW + QW)) : "memory");
+        }
+        myrot += rotated;
+        if (__syncthreads_or(rotated)) {
+          // columns of W and V times Q: a warp per 32 rows and half of the columns
+          did = 1;
+          const int gw = (R + 31) / 32, gv = (C + 31) / 32;
+          for (int t = warp; t < 2 * (gw + gv); t += NW) {
+            const int h = t & 1, gr = t >> 1;
+            const bool w = gr < gw;
+            const int ld = w ? R : C, pitch = w ? RP : C, i = 32 * (w ? gr : gr - gw) + lane;
+            if (i >= ld) continue;
+            const float* src = (w ? Ws : Vs) + i;
+            float* dst = (w ? W : V) + (int64_t)(h ? q0 : p0) * ld + i;
+            const int n = h ? nq : np;
+            float x[QP];
+#pragma unroll
+            for (int c = 0; c < QP; ++c) x[c] = c < N ? src[c * pitch] : 0.0f;
+#pragma unroll 3
+            for (int j = 0; j < n; ++j) {
+              const float* y = Qt + (h * BW + j) * QP;
+              float acc[2] = {};
+#pragma unroll
+              for (int c = 0; c < QP; c += 4) {
+                const float4 z = *reinterpret_cast<const float4*>(y + c);
+                acc[0] = fmaf(z.x, x[c], acc[0]);
+                acc[1] = fmaf(z.y, x[c + 1], acc[1]);
+                acc[0] = fmaf(z.z, x[c + 2], acc[0]);
+                acc[1] = fmaf(z.w, x[c + 3], acc[1]);
+              }
+              __stcg(dst + (int64_t)j * ld, acc[0] + acc[1]);
+            }
+          }
+        }
+      }
+      cluster.sync();  // the next round reads columns this round wrote, on other CTAs
+    }
+    const int f = (__syncthreads_or(did) ? 1 : 0) | (__syncthreads_or(big) ? 2 : 0);
+    if (f && tid == 0) atomicOr(flag0 + (gs & 1), f);
+    cluster.sync();
+    if (tid == 0) {
       ctl->any = flag0[gs & 1];
       if (crank == 0) ctl->flag[(gs + 1) & 1] = 0;
     }
@@ -860,39 +1082,31 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   const float tol32 = sqrtf((float)R) * FLT_EPSILON;
   float* nrm32 = reinterpret_cast<float*>(ws.nrm);
   int sw32;
-  switch (b.bw ? (R + 31) / 32 : 0) {
-#define SYM_BLOCKED(NR)                                                                                       \
-  case NR:                                                                                                    \
-    sw32 = jacobi_sweeps_blocked<float, NR, kThreads32>(W32, V32, nrm32, R, C, b.bw, kMaxSweeps32, tol32, cluster, &ctl,  \
-                                            flag0, crank, lane, gsweep, rot32, conv32, kBigRotation32,        \
-                                            reinterpret_cast<float*>(sm_pair));                               \
+  switch (b.bw) {  // the columns of a block, up to the bound of an instance
+#define SYM_GRAM(BW)                                                                                              \
+  case BW:                                                                                                        \
+    sw32 = jacobi_sweeps_gram<BW>(W32, V32, R, C, b.bw, kMaxSweeps32, tol32, cluster, &ctl, flag0, crank, lane,   \
+                                  gsweep, rot32, conv32, kBigRotation32, reinterpret_cast<float*>(sm_pair));      \
     break;
-#define SYM_BLOCKED_UP_TO(NR) \
-  case NR - 1:                \
-    SYM_BLOCKED(NR)
-    SYM_BLOCKED(1)
-    SYM_BLOCKED(2)
-    SYM_BLOCKED(3)
-    SYM_BLOCKED(4)
-    SYM_BLOCKED(5)
-    SYM_BLOCKED(6)
-    SYM_BLOCKED(7)
-    SYM_BLOCKED(8)
-    SYM_BLOCKED(9)
-    SYM_BLOCKED(10)
-    SYM_BLOCKED(11)
-    SYM_BLOCKED(12)
-    SYM_BLOCKED_UP_TO(14)
-    SYM_BLOCKED_UP_TO(16)
-    SYM_BLOCKED_UP_TO(18)
-    SYM_BLOCKED_UP_TO(20)
-#undef SYM_BLOCKED_UP_TO
-#undef SYM_BLOCKED
+    SYM_GRAM(2)
+    SYM_GRAM(3)
+    SYM_GRAM(4)
+    SYM_GRAM(5)
+    SYM_GRAM(6)
+    SYM_GRAM(7)
+    SYM_GRAM(8)
+    SYM_GRAM(9)
+    SYM_GRAM(10)
+    SYM_GRAM(11)
+    SYM_GRAM(12)
+    SYM_GRAM(13)
+    SYM_GRAM(14)
+#undef SYM_GRAM
     default:
       sw32 = jacobi_sweeps<float, kThreads32>(W32, V32, nrm32, R, C, kMaxSweeps32, tol32, cluster, &ctl, flag0, crank, cw, lane,
                                   gsweep, rot32, conv32, kBigRotation32);
   }
-  if (lane == 0 && rot32) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot32);
+  if (b.bw ? rot32 != 0 : lane == 0 && rot32) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot32);
   for (int64_t i = ct; i < CC; i += kCT) __stcg(ws.V + i, (double)__ldcg(V32 + i));
   cluster.sync();  // the rotation counts have arrived at rank 0
   if (crank == 0 && tid == 0) {
@@ -1565,19 +1779,20 @@ std::unique_ptr<SvdPlan> plan_svd(const Tensor& T, int nrow, bool eig) {
     // SU(2) with an incoming row leg: the dense block is (-1)^{2j} M_x / sqrt(2j+1) (x) 1
     b.sgn = (eig && T.group == SYM_SU2 && T.legs[0].dir == -1 && (x & 1)) ? -1.0 : 1.0;
     if (eig && m != n) fail(SYM_ERR_ARG, "internal: eigendecomposition block is not square");
-    // FP32 sweeps by column blocks when a block pair of W and V fits the
-    // shared memory two CTAs of an SM can have, rows up to 20 (FP64: 12) per lane
+    // sweeps by column blocks when a block pair of W and V (FP64: rows up to 12
+    // per lane) fits the shared memory two CTAs of an SM can have
     {
       const int bw = (b.C + kColBlocks - 1) / kColBlocks;
       const int64_t bytes = 2 * (int64_t)bw * (b.R + b.C + 1) * (int64_t)sizeof(float);
+      const int64_t gram = gram_floats(b.R, b.C, bw) * (int64_t)sizeof(float);
       const bool ok = b.C >= kColBlocks * 2 && b.R <= 32 * 12;  // FP64
-      b.bw = (b.C >= kColBlocks * 2 && b.R <= 32 * 20 && bytes <= kSvdSmem32Max) ? bw : 0;
+      b.bw = (b.C >= kColBlocks * 2 && bw <= kMaxGram && gram <= kSvdSmem32Max) ? bw : 0;
       // FP64 by column blocks for the SVD only: on the shifted symmetric blocks of
       // the eigendecomposition that order took up to 6 FP64 sweeps where the
       // order by pairs takes 4 (two-site density matrix: 29.8 against 29.0 ms;
       // two-site SVD: 20.4 against 22.3 ms)
-      b.bw64 = (ok && !eig && 2 * bytes <= kSvdSmem32Max) ? bw : 0;
-      if (b.bw) P->smem32 = std::max<int64_t>(P->smem32, b.bw64 ? 2 * bytes : bytes);
+      b.bw64 = (ok && !eig && 2 * bytes <= kSvdSmem64Max) ? bw : 0;
+      P->smem32 = std::max<int64_t>(P->smem32, std::max<int64_t>(b.bw ? gram : 0, b.bw64 ? 2 * bytes : 0));
     }
     b.w = P->work_elems;
     b.s = P->nsv;

@@ -506,8 +506,9 @@ class SVDPlan:
         visited; per rotation 4 multiply-adds per row of W and V.  FP64: a
         refined block (no rotations) takes W = A V, half of W^T W and half of
         V^T V per step; a block finished by FP64 sweeps those sweeps and
-        W = A V.  FP32: the sweeps, and V X per refinement step.  An FMA
-        counts 2."""
+        W = A V.  FP32: the sweeps (64 to 448 columns: the Gram matrices of
+        the block pairs and the products with the collected rotations), and
+        V X per refinement step.  An FMA counts 2."""
         s64, r64 = self.stats(False)
         s32, r32 = self.stats(True)
         f64 = f32 = 0.0
@@ -518,7 +519,12 @@ class SVDPlan:
 
         for m, n, a, ra, b, rb in zip(self.m, self.n, s64, r64, s32, r32):
             R, C = max(m, n), min(m, n)
-            f32 += sweep(R, C, b, rb, R <= 640)
+            w = 2 * -(-C // 32)
+            smem = 4 * w * ((R + 3) // 8 * 8 + 4 + (w + 3) // 4 * 4 + 2 * (w + 1) + C)
+            if 64 <= C <= 448 and smem <= 112 << 10:  # by column blocks: 496 block pairs' Gram matrices and products
+                f32 += b * 496 * (w * (w + 1.0) * R + 2.0 * w * w * (R + C))
+            else:
+                f32 += sweep(R, C, b, rb, R <= 384)
             if ra:
                 f64 += sweep(R, C, a, ra, R <= 384) + 2.0 * R * C * C
             else:

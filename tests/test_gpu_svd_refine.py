@@ -44,6 +44,14 @@ SVD = {
 }
 
 
+# FP32 sweeps through Gram matrices: each width of a column block (2 .. 14), the
+# last blocks ragged or absent, and rows that are no multiple of a warp's
+SVD.update({f"blocks of {b}": lambda b=b: _mat(32 * b - 31 + 3 * b, 32 * b - 31, 30 + b) for b in range(3, 15)})
+SVD["blocks of 2"] = lambda: _mat(64, 64, 31)
+SVD["blocks of 14, full"] = lambda: _mat(448, 448, 32)
+SVD["blocks of 5, rows past their shared memory"] = lambda: _mat(2600, 160, 33)
+
+
 @pytest.mark.parametrize("name", sorted(SVD))
 def test_svd(name):
     M = SVD[name]()
