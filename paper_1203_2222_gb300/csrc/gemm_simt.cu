@@ -7,10 +7,10 @@
 // bandwidth- or latency-bound and are computed here in FP32.
 //
 // Three kernels, chosen per sector by the planner:
-//   tile  TM x TN output tile per 256-thread CTA, 32-deep k slices staged in
-//         shared memory, the next slice prefetched into registers while the
-//         current one is multiplied; a tile may cover a slice [k0, k1) of the
-//         reduction (split-K: slices add into a zero-filled C with atomics).
+//   tile  TM x TN output tile per CTA, k slices staged in shared memory, the
+//         next ones in flight while the current one is multiplied (FP32: of
+//         its own, gemm_tile_f32_kernel); a tile may cover a slice [k0, k1) of
+//         the reduction (split-K: slices add into a zero-filled C with atomics).
 //   rows  k, n <= 16: a persistent streaming kernel -- each warp stages runs
 //         of whole rows of A in shared memory and writes whole rows of C.
 //   thin  m, n <= 8 and a long reduction: each thread streams k and keeps
@@ -106,6 +106,141 @@ __global__ void __launch_bounds__(256) gemm_tile_kernel(const GemmSectorSimt* __
         atomicAdd(&c[(int64_t)r * s.ldc + cc], alpha * acc[i][j]);
       else
         c[(int64_t)r * s.ldc + cc] = alpha * acc[i][j];
+    }
+  }
+}
+
+// The tile kernel in FP32.  Bound by the issue of its multiply-adds, so few
+// other instructions go with them: a warp takes a WM x WN part of the tile, a
+// thread 32 of its elements (groups of 4 x 4) from 3 16-byte loads of shared
+// memory per reduction step, and slices come by cp.async straight to their
+// transposed place (rows TM + 4 apart: the four rows of eight reduction steps
+// that a warp copies at once fall on 32 banks).  Rows, columns and reduction
+// steps past the sector are neither copied nor (by whole warps) multiplied:
+// garbage in shared memory reaches only elements that are not stored.  Every
+// element is one chain of fused multiply-adds in the order of k, as in the
+// FP64 kernel; two columns' go in one instruction (fma.rn.f32x2), which leaves
+// issue slots to the rest.  The 128 two-site problems of 64 <= D <= 1024, both
+// directions (18 GFLOP in sectors below the tensor-core tile): 64 x 64 tiles 640
+// -> 419 us, 256 x 16 tiles 135 -> 60 us against 256 threads with 4 x 4 (16 x 1)
+// elements and one 4-byte load per operand value (438 us without the packed
+// form).  What bounds it now is shared memory (72-78% of its throughput).
+__device__ __forceinline__ void cp_async4(float* smem, const float* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
+}
+constexpr int kTileThreads32 = 128;
+template <int TM, int TN, int WM, int WN, int KS>
+__global__ void __launch_bounds__(kTileThreads32, 5)
+    gemm_tile_f32_kernel(const GemmSectorSimt* __restrict__ secs, const GemmTile* __restrict__ tiles,
+                         const float* __restrict__ ops, float* __restrict__ outm) {
+  constexpr int kStages = 3, GM = WM / 32, GN = WN / 16, TP = TM + 4;
+  static_assert((TM / WM) * (TN / WN) == kTileThreads32 / 32 && GM * GN == 2 && (KS == 8 || KS == 16), "tile split");
+  __shared__ __align__(16) float As[kStages][KS][TP];
+  __shared__ __align__(16) float Bs[kStages][KS][TN];
+  const GemmTile tl = tiles[blockIdx.x];
+  const GemmSectorSimt s = secs[tl.sector];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m0 = tl.mt * TM, n0 = tl.nt * TN;
+  const int rows = min(TM, s.m - m0), cols = min(TN, s.n - n0);
+  // copies: this thread's reduction step and first row of A, its column and first step of B
+  constexpr int kOct = KS / 8, kRowStep = 16 / kOct, kColStep = kTileThreads32 / TN;
+  const int ac = warp % kOct * 8 + (lane & 7), ar = warp / kOct * 4 + (lane >> 3);
+  const int bc = tid % TN, br = tid / TN;
+  const float* __restrict__ a = ops + s.a_off + (int64_t)(m0 + ar) * s.lda + ac;
+  const float* __restrict__ b = ops + s.b_off + (int64_t)br * s.ldb + n0 + bc;
+  auto issue = [&](int kb, int st) {
+    if (kb < tl.k1) {
+      const int kn = tl.k1 - kb;
+      if (ac < kn) {
+        const float* src = a + kb;
+#pragma unroll
+        for (int u = 0; u < TM / kRowStep; ++u, src += (int64_t)kRowStep * s.lda)
+          if (ar + kRowStep * u < rows) cp_async4(&As[st][ac][ar + kRowStep * u], src);
+      }
+      if (bc < cols) {
+        const float* src = b + (int64_t)kb * s.ldb;
+#pragma unroll
+        for (int u = 0; u < KS / kColStep; ++u, src += (int64_t)kColStep * s.ldb)
+          if (br + kColStep * u < kn) cp_async4(&Bs[st][br + kColStep * u][bc], src);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  const int wm = warp % (TM / WM) * WM, wn = warp / (TM / WM) * WN;
+  const int r0 = wm + (lane >> 2) * 4, c0 = wn + (lane & 3) * 4;  // groups at r0 + 32 i, c0 + 16 j
+  const bool active = wm < rows && wn < cols;
+  unsigned long long acc2[4 * GM][2 * GN];
+#pragma unroll
+  for (int i = 0; i < 4 * GM; ++i)
+#pragma unroll
+    for (int j = 0; j < 2 * GN; ++j) acc2[i][j] = 0ull;
+  issue(tl.k0, 0);
+  issue(tl.k0 + KS, 1);
+  int st = 0;
+  for (int kb = tl.k0; kb < tl.k1; kb += KS) {
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();  // this slice is here, and every warp is done with the one before
+    issue(kb + 2 * KS, st >= 1 ? st - 1 : kStages - 1);
+    if (active) {
+      auto step = [&](int kk) {
+        float av[4 * GM];
+        unsigned long long bv[2 * GN];
+#pragma unroll
+        for (int i = 0; i < GM; ++i)
+          *reinterpret_cast<float4*>(av + 4 * i) = *reinterpret_cast<const float4*>(&As[st][kk][r0 + 32 * i]);
+#pragma unroll
+        for (int j = 0; j < GN; ++j)
+          { const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&Bs[st][kk][c0 + 16 * j]); bv[2*j]=q.x; bv[2*j+1]=q.y; }
+#pragma unroll
+        for (int i = 0; i < 4 * GM; ++i) {
+          unsigned long long aa;
+          asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(av[i]));
+#pragma unroll
+          for (int j = 0; j < 2 * GN; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[i][j]) : "l"(aa), "l"(bv[j]));
+        }
+      };
+      if (kb + KS <= tl.k1) {
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) step(kk);
+      } else {
+        for (int kk = 0; kk < tl.k1 - kb; ++kk) step(kk);
+      }
+    }
+    st = st + 1 == kStages ? 0 : st + 1;
+  }
+  if (!active) return;
+  float acc[4 * GM][4 * GN];
+#pragma unroll
+  for (int i = 0; i < 4 * GM; ++i)
+#pragma unroll
+    for (int j = 0; j < 2 * GN; ++j) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][2*j]), "=f"(acc[i][2*j+1]) : "l"(acc2[i][j]));
+  float* c = outm + s.c_off;
+  const float alpha = (float)s.alpha;
+  const bool vec = (s.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(c) & 15) == 0 && !tl.atomic;
+#pragma unroll
+  for (int i = 0; i < 4 * GM; ++i) {
+    const int r = r0 + 32 * (i / 4) + i % 4;
+    if (r >= rows) continue;
+#pragma unroll
+    for (int j = 0; j < GN; ++j) {
+      const int cc = c0 + 16 * j;
+      float* out = c + (int64_t)(m0 + r) * s.ldc + n0 + cc;
+      const float* x = acc[i] + 4 * j;
+      if (vec && cc + 4 <= cols) {
+        *reinterpret_cast<float4*>(out) = make_float4(alpha * x[0], alpha * x[1], alpha * x[2], alpha * x[3]);
+        continue;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (cc + u >= cols) break;
+        if (tl.atomic)
+          atomicAdd(out + u, alpha * x[u]);
+        else
+          out[u] = alpha * x[u];
+      }
     }
   }
 }
@@ -262,8 +397,16 @@ int launch_t(int shape, const GemmSectorSimt* secs, const GemmTile* tiles, int n
   T* c = static_cast<T*>(outm);
   const dim3 g(ntiles), b(256);
   switch (shape) {
-    case SIMT_64x64: return (int)launch_pdl(gemm_tile_kernel<T, 64, 64>, g, b, 0, s, secs, tiles, o, c);
-    case SIMT_256x16: return (int)launch_pdl(gemm_tile_kernel<T, 256, 16>, g, b, 0, s, secs, tiles, o, c);
+    case SIMT_64x64:
+      if constexpr (sizeof(T) == 4)
+        return (int)launch_pdl(gemm_tile_f32_kernel<64, 64, 32, 32, 16>, g, dim3(kTileThreads32), 0, s, secs, tiles, o, c);
+      else
+        return (int)launch_pdl(gemm_tile_kernel<T, 64, 64>, g, b, 0, s, secs, tiles, o, c);
+    case SIMT_256x16:
+      if constexpr (sizeof(T) == 4)
+        return (int)launch_pdl(gemm_tile_f32_kernel<256, 16, 64, 16, 8>, g, dim3(kTileThreads32), 0, s, secs, tiles, o, c);
+      else
+        return (int)launch_pdl(gemm_tile_kernel<T, 256, 16>, g, b, 0, s, secs, tiles, o, c);
     case SIMT_THIN: return (int)launch_pdl(gemm_thin_kernel<T>, g, b, 0, s, secs, tiles, o, c);
     default: {
       const int ctas = std::min((ntiles + 7) / 8, tc_num_sms() * rows_ctas_per_sm<T>());
