@@ -14,13 +14,23 @@
 //   outer  dN(s, d) += sum_t A_s[t] dC_d[t] (dB = A^T dC), reduced across the
 //          warp with butterfly shuffles and added into the zero-filled
 //          gradient blocks with atomics
+//   both   dA and dB of an outer item from one read of dC (and of A)
 //
 // Persistent and warp-independent: a warp copies one 512-byte descriptor
 // (columns inline) into its shared-memory slot while the previous item runs,
-// stages the item's coefficients and column pointers in registers, and
-// streams the box with coalesced loads along its last dim.
-// Apply and outer items run as separate launches of their own kernels (every
-// item of a launch has the same kind).
+// and streams the box with coalesced loads along its last dim, 64 bytes of
+// them a lane and step in flight, in registers.  What bounds it is the
+// instructions and round trips around short streams, so: columns are read
+// from the descriptor as they are used (few registers, 24 to 32 warps an SM),
+// a position's index is formed once for loads and stores, and an item shorter
+// than a step takes smaller ones.  Every item form is a function of its own
+// (inlined into one another they spilled 1 KB a thread).  Items come longest
+// first (plan.cpp) and go to the CTAs in turn.  128 two-site problems of 64 <=
+// D <= 1024, 154 MB in and out per step: apply 107 -> 86 us (3.6 TB/s), both
+// gradients 255 -> 115 us (4.0 TB/s) against apply and outer launches with two
+// cp.async stages in shared memory (with items in the order of the sectors 92
+// and 186 us); one FP64 problem of D = 512, latency-bound: 33 -> 28 us.
+// Items of one kind run as launches of their own.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,28 +43,12 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
-// Loads are staged by cp.async into a per-lane slice of shared memory, two
-// stages deep, so that a lane keeps 2 * kH(T) positions x kMaxDirect columns
-// in flight (2 * 8 KB per warp) without holding them in registers; each lane
-// reads back only what it copied itself, so no barrier is needed.
-template <typename T>
-constexpr int kH = 32 / (int)sizeof(T);  // apply: positions per lane per stage (8 fp32, 4 fp64)
-template <typename T>
-constexpr int kHo = kH<T> / 2;           // outer: (twice the columns per position)
-constexpr int kStageBytes = 32 * 32 * kMaxDirect;  // one stage of one warp: 32 lanes x 8 fp32 x 4 columns
-
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem, int bytes) {
-  const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
-  if (bytes == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
+// positions of a step: COLS values each, 64 bytes of them a lane, at most 8
+template <typename T, int COLS>
+constexpr int kSteps = 64 / (int)sizeof(T) / COLS >= 8   ? 8
+                       : 64 / (int)sizeof(T) / COLS >= 4 ? 4
+                       : 64 / (int)sizeof(T) / COLS >= 2 ? 2
+                                                         : 1;
 
 template <typename T>
 __device__ __forceinline__ const T* src_ptr(const BoxPtrs& p, int slot) {
@@ -92,151 +86,140 @@ struct DirectShape {
   }
 };
 
-// Columns of one side of an item: column c at box index t is base[c][<t, str[c]>]
-// (the relative offset stays below 2^31 -- host check -- so it is formed in 32 bits).
-template <typename P, int NC, int ND>
-struct Cols {
-  P base[NC];
-  int str[NC][ND];
-  __device__ __forceinline__ void load(P slot, const DirectCol* cols, int n) {
+// One step of an item: the H positions p0 + lane + 32 h.  Columns are walked
+// one by one, each one's offset and strides read from the descriptor in shared
+// memory (the barrier keeps the compiler from holding all of them, which
+// spilled): column c at box index t is base[off + <t, str>], the relative
+// offset below 2^31 (host check).
+template <int ND, int H>
+struct Positions {
+  int t[H][ND];
+  __device__ __forceinline__ Positions(const DirectShape<ND>& sh, int p, int last) {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const bool on = c < n;
-      base[c] = slot + cols[on ? c : 0].off;
-#pragma unroll
-      for (int d = 0; d < ND; ++d) str[c][d] = on ? cols[c].str[d] : 0;
-    }
+    for (int h = 0; h < H; ++h) sh.index(min(p + 32 * h, last), t[h]);
+    asm volatile("" ::: "memory");
   }
-  __device__ __forceinline__ int off(int c, const int (&t)[ND]) const {
+  __device__ __forceinline__ int off(const int (&str)[ND], int h) const {
     int o = 0;
 #pragma unroll
-    for (int d = 0; d < ND; ++d) o += t[d] * str[c][d];
+    for (int d = 0; d < ND; ++d) o += t[h][d] * str[d];
     return o;
   }
-};
-
-// apply: NS source and NQ destination columns (exact counts when the item has
-// them, else upper bounds with the actual counts ns <= NS, nq <= NQ); the
-// coefficient values are in this warp's cf[d * kMaxDirect + s]
-template <typename T, int ND, int NS, int NQ>
-__device__ __forceinline__ void apply_item(const DirectItem& it, const T* __restrict__ cfv, const BoxPtrs& ptrs,
-                                           int lane, T* __restrict__ stage) {
-  const int ns = it.ns, nq = it.nd;
-  Cols<const T*, NS, ND> S;
-  Cols<T*, NQ, ND> Q;
-  S.load(src_ptr<T>(ptrs, it.slots & 3), it.src, ns);
-  Q.load(dst_ptr<T>(ptrs, (it.slots >> 4) & 7), it.dst, nq);
-  T cf[NQ][NS];
+  template <typename T, int NC>
+  __device__ __forceinline__ void load(T (&x)[H][NC], const T* __restrict__ p, const DirectCol* cols, int n) const {
 #pragma unroll
-  for (int d = 0; d < NQ; ++d)
+    for (int c = 0; c < NC; ++c) {
+      if (c < n) {
+        const T* __restrict__ b = p + cols[c].off;
+        int str[ND];
 #pragma unroll
-    for (int c = 0; c < NS; ++c) cf[d][c] = (d < nq && c < ns) ? cfv[d * kMaxDirect + c] : T(0);
-  const DirectShape<ND> sh(it);
-  const int last = it.start + it.count - 1;
-  constexpr int H = kH<T>;
-  constexpr int SLOT = H * NS * 32;  // one stage: [H][NS][32], this lane's values at [..][..][lane]
-  auto issue = [&](int u, T* buf) {
+        for (int d = 0; d < ND; ++d) str[d] = cols[c].str[d];
 #pragma unroll
-    for (int h = 0; h < H; ++h) {
-      int t[ND];
-      sh.index(min(u + 32 * h, last), t);
+        for (int h = 0; h < H; ++h) x[h][c] = __ldg(b + off(str, h));
+      } else {
 #pragma unroll
-      for (int c = 0; c < NS; ++c)
-        if (c < ns) cp_async(buf + (h * NS + c) * 32 + lane, S.base[c] + S.off(c, t), sizeof(T));
-    }
-    cp_commit();
-  };
-  const int step = 32 * H;
-  int u = it.start + lane;
-  if (u <= last) issue(u, stage);
-  for (int k = 0; u <= last; u += step, ++k) {
-    T* cur = stage + (k & 1) * SLOT;
-    if (u + step <= last) {
-      issue(u + step, stage + ((k + 1) & 1) * SLOT);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-      if (u + 32 * h > last) break;
-      int t[ND];
-      sh.index(u + 32 * h, t);
-      T v[NS];
-#pragma unroll
-      for (int c = 0; c < NS; ++c) v[c] = c < ns ? cur[(h * NS + c) * 32 + lane] : T(0);
-#pragma unroll
-      for (int d = 0; d < NQ; ++d) {
-        if (d >= nq) break;
-        T acc = T(0);
-#pragma unroll
-        for (int c = 0; c < NS; ++c) acc = fma(cf[d][c], v[c], acc);
-        Q.base[d][Q.off(d, t)] = acc;
+        for (int h = 0; h < H; ++h) x[h][c] = T(0);
       }
     }
   }
+  // column c of `cols` at the positions: sum_s cf[c * cs + s * ss] x[.][s], in the order of s
+  template <typename T, int NX, int NC>
+  __device__ __forceinline__ void store(T* __restrict__ p, const DirectCol* cols, int n, const T (&x)[H][NX],
+                                        const T* cf, int cs, int ss, int left) const {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (c >= n) break;
+      T* __restrict__ b = p + cols[c].off;
+      int str[ND];
+      T k[NX];
+#pragma unroll
+      for (int d = 0; d < ND; ++d) str[d] = cols[c].str[d];
+#pragma unroll
+      for (int i = 0; i < NX; ++i) k[i] = cf[c * cs + i * ss];
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        T v = T(0);
+#pragma unroll
+        for (int i = 0; i < NX; ++i) v = fma(k[i], x[h][i], v);
+        if (32 * h <= left) b[off(str, h)] = v;
+      }
+    }
+  }
+};
+
+// Steps of H positions a lane as long as they are whole, then of fewer: a small
+// item does not pay for the positions it does not have.  step(Positions, u, left).
+template <int ND, int H, typename Step>
+__device__ __forceinline__ void steps(const DirectShape<ND>& sh, int p, int lane, int last, const Step& step) {
+  for (; p + 32 * (H - 1) <= last; p += 32 * H) step(Positions<ND, H>(sh, p + lane, last), last - p - lane);
+  if constexpr (H > 1) {
+    if (p <= last) steps<ND, H / 2>(sh, p, lane, last, step);
+  }
+}
+
+// apply: NS source and NQ destination columns (exact counts when the item has
+// them, else upper bounds with the actual counts ns <= NS, nq <= NQ)
+template <typename T, int ND, int NS, int NQ>
+struct ApplyStep {
+  const DirectItem& it;
+  const T* slot;
+  const T* src;
+  T* dst;
+  int ns, nq;
+  template <int H>
+  __device__ __forceinline__ void operator()(const Positions<ND, H>& t, int left) const {
+    T x[H][NS];
+    t.load(x, src, it.src, ns);
+    t.template store<T, NS, NQ>(dst, it.dst, nq, x, slot, kMaxDirect, 1, left);
+  }
+};
+template <typename T, int ND, int NS, int NQ>
+__device__ __noinline__ void apply_item(const DirectItem& it, const T* __restrict__ slot, const T* __restrict__ src,
+                                        T* __restrict__ dst, int lane) {
+  const ApplyStep<T, ND, NS, NQ> step{it, slot, src, dst, it.ns, it.nd};
+  steps<ND, kSteps<T, NS>>(DirectShape<ND>(it), it.start, lane, it.start + it.count - 1, step);
 }
 
 // outer: out(s, d) = sum_t A_s[t] dC_d[t] over the item's positions, scaled
-// by kc and added into the destination at koff
-template <typename T, int ND, int NS, int NQ>
-__device__ __forceinline__ void outer_item(const DirectItem& it, const BoxPtrs& ptrs, int lane,
-                                           T* __restrict__ stage) {
+// by kc and added into the destination at koff.  kBoth: also dA_s[t] = sum_d
+// N(s, d) dC_d[t], at A's columns in dA, in the order of an apply item of dA.
+template <typename T, int ND, int NS, int NQ, bool kBoth>
+struct OuterStep {
+  const DirectItem& it;
+  const T* slot;
+  const T* src;
+  const T* qsrc;
+  T* da;
+  int ns, nq;
+  T (&acc)[NS][NQ];
+  template <int H>
+  __device__ __forceinline__ void operator()(const Positions<ND, H>& t, int left) const {
+    T a[H][NS], q[H][NQ];
+    t.load(a, src, it.src, ns);
+    t.load(q, qsrc, it.dst, nq);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      if (32 * h > left) continue;  // positions past the last one repeat it: they add nothing
+#pragma unroll
+      for (int c = 0; c < NS; ++c)
+#pragma unroll
+        for (int d = 0; d < NQ; ++d) acc[c][d] = fma(a[h][c], q[h][d], acc[c][d]);
+    }
+    if (kBoth) t.template store<T, NQ, NS>(da, it.src, ns, q, slot, 1, kMaxDirect, left);
+  }
+};
+template <typename T, int ND, int NS, int NQ, bool kBoth>
+__device__ __noinline__ void outer_item(const DirectItem& it, const T* __restrict__ slot, const T* __restrict__ src,
+                                        const T* __restrict__ qsrc, T* __restrict__ dst, T* __restrict__ da,
+                                        int lane) {
   const int ns = it.ns, nq = it.nd;
-  T* __restrict__ dst = dst_ptr<T>(ptrs, (it.slots >> 4) & 7);
-  Cols<const T*, NS, ND> S;
-  Cols<const T*, NQ, ND> Q;
-  S.load(src_ptr<T>(ptrs, it.slots & 3), it.src, ns);
-  Q.load(src_ptr<T>(ptrs, (it.slots >> 2) & 3), it.dst, nq);
   T acc[NS][NQ];
 #pragma unroll
   for (int c = 0; c < NS; ++c)
 #pragma unroll
     for (int d = 0; d < NQ; ++d) acc[c][d] = T(0);
-  const DirectShape<ND> sh(it);
-  const int last = it.start + it.count - 1;
-  constexpr int H = kHo<T>;
-  constexpr int W = NS + NQ;          // values per position
-  constexpr int SLOT = H * W * 32;    // one stage: [H][W][32]
-  auto issue = [&](int u, T* buf) {
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-      int t[ND];
-      sh.index(min(u + 32 * h, last), t);
-#pragma unroll
-      for (int c = 0; c < NS; ++c)
-        if (c < ns) cp_async(buf + (h * W + c) * 32 + lane, S.base[c] + S.off(c, t), sizeof(T));
-#pragma unroll
-      for (int d = 0; d < NQ; ++d)
-        if (d < nq) cp_async(buf + (h * W + NS + d) * 32 + lane, Q.base[d] + Q.off(d, t), sizeof(T));
-    }
-    cp_commit();
-  };
-  const int step = 32 * H;
-  int u = it.start + lane;
-  if (u <= last) issue(u, stage);
-  for (int k = 0; u <= last; u += step, ++k) {
-    T* cur = stage + (k & 1) * SLOT;
-    if (u + step <= last) {
-      issue(u + step, stage + ((k + 1) & 1) * SLOT);
-      cp_wait<1>();
-    } else {
-      cp_wait<0>();
-    }
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-      if (u + 32 * h > last) break;
-      T va[NS], vq[NQ];
-#pragma unroll
-      for (int c = 0; c < NS; ++c) va[c] = c < ns ? cur[(h * W + c) * 32 + lane] : T(0);
-#pragma unroll
-      for (int d = 0; d < NQ; ++d) vq[d] = d < nq ? cur[(h * W + NS + d) * 32 + lane] : T(0);
-#pragma unroll
-      for (int c = 0; c < NS; ++c)
-#pragma unroll
-        for (int d = 0; d < NQ; ++d) acc[c][d] = fma(va[c], vq[d], acc[c][d]);
-    }
-  }
+  const OuterStep<T, ND, NS, NQ, kBoth> step{it, slot, src, qsrc, da, ns, nq, acc};
+  steps<ND, kSteps<T, NS + NQ>>(DirectShape<ND>(it), it.start, lane, it.start + it.count - 1, step);
   // butterfly: every lane ends with the warp's sums
 #pragma unroll
   for (int c = 0; c < NS; ++c)
@@ -261,23 +244,26 @@ __device__ __forceinline__ void outer_item(const DirectItem& it, const BoxPtrs& 
 
 // the item's column counts pick an exact variant (the MPO and physical legs
 // of a tensor network give 1 or 4 columns per side), else the bounded one
+template <typename T, int kOp, int ND, int NS, int NQ>
+__device__ __forceinline__ void run_cols(const DirectItem& it, const T* __restrict__ slot, const BoxPtrs& ptrs,
+                                         int lane) {
+  if constexpr (kOp == kDirectApply)
+    apply_item<T, ND, NS, NQ>(it, slot, src_ptr<T>(ptrs, it.slots & 3), dst_ptr<T>(ptrs, (it.slots >> 4) & 7), lane);
+  else
+    outer_item<T, ND, NS, NQ, kOp == kDirectBoth>(it, slot, src_ptr<T>(ptrs, it.slots & 3),
+                                                  src_ptr<T>(ptrs, (it.slots >> 2) & 3),
+                                                  dst_ptr<T>(ptrs, (it.slots >> 4) & 7), dst_ptr<T>(ptrs, DST_DA), lane);
+}
+
 template <typename T, int kOp, int ND>
-__device__ __forceinline__ void run_item(const DirectItem& it, const T* __restrict__ cfv, const BoxPtrs& ptrs,
-                                         int lane, T* __restrict__ stage) {
+__device__ __forceinline__ void run_item(const DirectItem& it, const T* __restrict__ slot, const BoxPtrs& ptrs,
+                                         int lane) {
   const int key = ND == 3 ? 0 : it.ns * 8 + it.nd;  // three-dim boxes take the bounded variant only
-  if (kOp == kDirectApply) {
-    if (key == 4 * 8 + 4) apply_item<T, ND, 4, 4>(it, cfv, ptrs, lane, stage);
-    else if (key == 1 * 8 + 1) apply_item<T, ND, 1, 1>(it, cfv, ptrs, lane, stage);
-    else if (key == 1 * 8 + 4) apply_item<T, ND, 1, 4>(it, cfv, ptrs, lane, stage);
-    else if (key == 4 * 8 + 1) apply_item<T, ND, 4, 1>(it, cfv, ptrs, lane, stage);
-    else apply_item<T, ND, kMaxDirect, kMaxDirect>(it, cfv, ptrs, lane, stage);
-  } else {
-    if (key == 4 * 8 + 4) outer_item<T, ND, 4, 4>(it, ptrs, lane, stage);
-    else if (key == 1 * 8 + 1) outer_item<T, ND, 1, 1>(it, ptrs, lane, stage);
-    else if (key == 1 * 8 + 4) outer_item<T, ND, 1, 4>(it, ptrs, lane, stage);
-    else if (key == 4 * 8 + 1) outer_item<T, ND, 4, 1>(it, ptrs, lane, stage);
-    else outer_item<T, ND, kMaxDirect, kMaxDirect>(it, ptrs, lane, stage);
-  }
+  if (key == 4 * 8 + 4) run_cols<T, kOp, ND, 4, 4>(it, slot, ptrs, lane);
+  else if (key == 1 * 8 + 1) run_cols<T, kOp, ND, 1, 1>(it, slot, ptrs, lane);
+  else if (key == 1 * 8 + 4) run_cols<T, kOp, ND, 1, 4>(it, slot, ptrs, lane);
+  else if (key == 4 * 8 + 1) run_cols<T, kOp, ND, 4, 1>(it, slot, ptrs, lane);
+  else run_cols<T, kOp, ND, kMaxDirect, kMaxDirect>(it, slot, ptrs, lane);
 }
 
 // One kernel per item kind, so that each gets the registers of its own loop.
@@ -285,16 +271,14 @@ __device__ __forceinline__ void run_item(const DirectItem& it, const T* __restri
 // lane) while it runs the current one, so an item's set-up costs one round
 // trip: the apply coefficients, loaded by one lane each.
 template <typename T, int kOp>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(kThreads, kOp == kDirectApply ? (sizeof(T) == 4 ? 4 : 3) : 3)
     direct_kernel(const DirectItem* __restrict__ items, int nitems, BoxPtrs ptrs) {
   static_assert(sizeof(DirectItem) == 32 * sizeof(int4), "one 16-byte descriptor word per lane");
   __shared__ __align__(16) DirectItem desc[kWarps];
   __shared__ T cfs[kWarps][kMaxDirect * kMaxDirect];
-  extern __shared__ __align__(16) unsigned char dyn[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* stage = reinterpret_cast<T*>(dyn + (size_t)warp * 2 * kStageBytes);
   const int stride = gridDim.x * kWarps;
-  int w = blockIdx.x * kWarps + warp;
+  int w = warp * gridDim.x + blockIdx.x;  // the longest items, which come first, spread over the CTAs
   int4 next = make_int4(0, 0, 0, 0);
   if (w < nitems) next = __ldg(reinterpret_cast<const int4*>(items + w) + lane);
   pdl_wait();
@@ -305,32 +289,25 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
     __syncwarp();
     if (w + stride < nitems) next = __ldg(reinterpret_cast<const int4*>(items + w + stride) + lane);
     const DirectItem& it = desc[warp];
-    if (kOp == kDirectApply) {  // coefficient values, one lane each
-      const T* __restrict__ ksrc = src_ptr<T>(ptrs, (it.slots >> 2) & 3);
-      if (lane < kMaxDirect * kMaxDirect) {
-        const double k = it.kc[lane];
-        cfs[warp][lane] = k != 0.0 ? T(k) * __ldg(ksrc + it.koff[lane]) : T(0);
-      }
-      __syncwarp();
+    if (kOp != kDirectOuter && lane < kMaxDirect * kMaxDirect) {  // N(s, d), one lane each
+      const double k = it.kc[lane];
+      cfs[warp][lane] = k != 0.0 ? T(k) * __ldg(src_ptr<T>(ptrs, 1) + it.koff[lane]) : T(0);
     }
+    __syncwarp();
     if (it.ndim == 1)
-      run_item<T, kOp, 1>(it, cfs[warp], ptrs, lane, stage);
+      run_item<T, kOp, 1>(it, cfs[warp], ptrs, lane);
     else if (it.ndim == 2)
-      run_item<T, kOp, 2>(it, cfs[warp], ptrs, lane, stage);
+      run_item<T, kOp, 2>(it, cfs[warp], ptrs, lane);
     else
-      run_item<T, kOp, 3>(it, cfs[warp], ptrs, lane, stage);
+      run_item<T, kOp, 3>(it, cfs[warp], ptrs, lane);
   }
 }
-
-constexpr int kDynSmem = kWarps * 2 * kStageBytes;  // 64 KB: two stages per warp
 
 template <typename T, int kOp>
 int ctas_per_sm() {
   static const int n = [] {
     int v = 0;
-    cudaFuncSetAttribute(direct_kernel<T, kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, direct_kernel<T, kOp>, kThreads, kDynSmem) != cudaSuccess ||
-        v < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, direct_kernel<T, kOp>, kThreads, 0) != cudaSuccess || v < 1)
       v = 1;
     return v;
   }();
@@ -341,18 +318,21 @@ template <typename T, int kOp>
 int launch_op(const DirectItem* items, int nitems, const BoxPtrs& ptrs, cudaStream_t s) {
   if (nitems <= 0) return 0;
   const int ctas = std::min((nitems + kWarps - 1) / kWarps, tc_num_sms() * ctas_per_sm<T, kOp>());
-  return (int)launch_pdl(direct_kernel<T, kOp>, dim3(ctas), dim3(kThreads), kDynSmem, s, items, nitems, ptrs);
+  return (int)launch_pdl(direct_kernel<T, kOp>, dim3(ctas), dim3(kThreads), 0, s, items, nitems, ptrs);
+}
+
+template <typename T>
+int launch_t(int op, const DirectItem* items, int nitems, const BoxPtrs& ptrs, cudaStream_t s) {
+  return op == kDirectApply   ? launch_op<T, kDirectApply>(items, nitems, ptrs, s)
+         : op == kDirectOuter ? launch_op<T, kDirectOuter>(items, nitems, ptrs, s)
+                              : launch_op<T, kDirectBoth>(items, nitems, ptrs, s);
 }
 
 }  // namespace
 
 int launch_direct(bool f64, int op, const DirectItem* items, int nitems, const BoxPtrs& ptrs, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (op == kDirectApply)
-    return f64 ? launch_op<double, kDirectApply>(items, nitems, ptrs, s)
-               : launch_op<float, kDirectApply>(items, nitems, ptrs, s);
-  return f64 ? launch_op<double, kDirectOuter>(items, nitems, ptrs, s)
-             : launch_op<float, kDirectOuter>(items, nitems, ptrs, s);
+  return f64 ? launch_t<double>(op, items, nitems, ptrs, s) : launch_t<float>(op, items, nitems, ptrs, s);
 }
 
 }  // namespace sym

@@ -157,7 +157,7 @@ struct TcOperand {
 constexpr int kMaxDirect = 4;
 constexpr int kDirectDims = 3;
 constexpr int kDirectApplyChunk = 1024;  // default positions per apply item
-enum DirectOp { kDirectApply = 0, kDirectOuter = 1 };
+enum DirectOp { kDirectApply = 0, kDirectOuter = 1, kDirectBoth = 2 };  // both: a launch of outer items, dA and dB
 struct DirectCol {
   int64_t off;
   int32_t str[kDirectDims];

@@ -63,7 +63,7 @@ struct Plan {
   // see kernels.h), their columns inline
   std::vector<DirectItem> ditems;
   Range fwd_direct, bwd_direct_a, bwd_direct_b;  // C = A B; dA = dC B^T; dB += A^T dC
-  std::vector<double> ditem_bytes_prefix, ditem_flops_prefix;  // launch statistics
+  std::vector<double> ditem_bytes_prefix, ditem_abytes_prefix, ditem_flops_prefix;  // launch statistics
 
   // block contraction work lists (block.cu) of a plan that runs on the blocks
   // in place of matrix form: phases 0 = forward, 1 = dA, 2 = dB; the tiles of
