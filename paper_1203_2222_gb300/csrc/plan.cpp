@@ -678,9 +678,39 @@ void Plan::encode_maps(const void* img_base) {
   maps_base = img_base;
 }
 
+// Box items of a launch by falling size class (powers of two; order kept
+// within a class, where neighbours share cache lines): a warp takes every W-th
+// item, W warps resident, so this order evens out the warps' shares.  Gathers,
+// scatters and transposes of 128 two-site problems 640 -> 540 us, a U(1) permute,
+// fuse and split of 470 MB 246 -> 237 us.  Only launches of flat items: with
+// recoupling sums (SU(2), FP64: 237 -> 263 us) the order of the sectors is the
+// better one, where items that share their sources are neighbours.
+void Plan::sort_items() {
+  std::vector<int> cut = {0, (int)items.size()};  // items between two cuts are in the same launches
+  for (const Range* r : {&xform, &fwd_gather, &fwd_scatter, &bwd_gather_a, &bwd_gather_b, &bwd_scatter_a, &bwd_scatter_b})
+    if (r->count > 0) cut.insert(cut.end(), {r->first, r->first + r->count});
+  std::sort(cut.begin(), cut.end());
+  std::vector<int> ord(items.size()), cls(items.size());
+  for (size_t i = 0; i < items.size(); ++i) {
+    ord[i] = (int)i;
+    cls[i] = std::ilogb((double)items[i].count * std::max(1, items[i].nterm));
+  }
+  for (size_t k = 0; k + 1 < cut.size(); ++k)
+    if (std::all_of(items.begin() + cut[k], items.begin() + cut[k + 1], [](const BoxItem& i) { return i.sel & kSelFlat; }))
+      std::stable_sort(ord.begin() + cut[k], ord.begin() + cut[k + 1], [&](int a, int b) { return cls[a] > cls[b]; });
+  std::vector<BoxItem> sorted(items.size());
+  std::vector<double> bytes(item_bytes_prefix);
+  for (size_t i = 0; i < items.size(); ++i) {
+    sorted[i] = items[ord[i]];
+    item_bytes_prefix[i + 1] = bytes[ord[i] + 1];
+  }
+  items.swap(sorted);
+}
+
 void Plan::upload(bool device) {
   // finish the statistics tables (prefix sums)
   if (item_bytes_prefix.size() != items.size() + 1) item_bytes_prefix.assign(items.size() + 1, 0.0);
+  sort_items();
   for (size_t i = 0; i < items.size(); ++i) item_bytes_prefix[i + 1] += item_bytes_prefix[i];
   flat_prefix.assign(items.size() + 1, 0);
   tile_prefix.assign(items.size() + 1, 0);

@@ -109,6 +109,7 @@ struct Plan {
   std::vector<int> tile_prefix;      // flat tile items among the first i
   std::vector<int> recouple_prefix;  // fused recoupling items among the first i
   void set_item_bytes(Range r, int es_src, int es_dst);
+  void sort_items();
   bool profiling = false;
   PhaseProfile prof[PH_COUNT];
   void clear_profile();
