@@ -29,7 +29,7 @@
 // D <= 1024, 154 MB in and out per step: apply 107 -> 86 us (3.6 TB/s), both
 // gradients 255 -> 115 us (4.0 TB/s) against apply and outer launches with two
 // cp.async stages in shared memory (with items in the order of the sectors 92
-// and 186 us); one FP64 problem of D = 512, latency-bound: 33 -> 28 us.
+// and 186 us); one FP64 problem of D = 768, latency-bound: 33 -> 28 us.
 // Items of one kind run as launches of their own.
 #include <cuda_runtime.h>
 
