@@ -155,9 +155,10 @@ class Plan:
 # The current device's current stream and device pointers as plain integers:
 # torch.cuda.current_stream() builds a Stream object (10 us on a Grace core,
 # as much as the rest of a contraction's forward on the host); the raw getter
-# is the same query without the object.
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_cur_device = torch._C._cuda_getDevice
+# is the same query without the object.  A torch built without CUDA has neither
+# getter; structures and host-side planning work there all the same.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_cur_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream():
