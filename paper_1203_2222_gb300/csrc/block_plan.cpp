@@ -91,6 +91,12 @@ Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k) {
 
 }  // namespace
 
+// The best rates tile_cost knows: 76.8 multiply-adds a clock of an SM in FP32
+// (BLK_BIG), below 2 in FP64; whole tiles and latencies only add to that.
+double block_floor_us(bool f64, double fma) {
+  return kModelScale * fma / (f64 ? 2.0 : 76.8) / 152.0 / 1900.0;
+}
+
 double blk_tile_cost(bool f64, const BlkTile& t) {
   const int64_t ks = blk_slab(f64, t.shape);
   return tile_cost(f64, t.shape, t.ob.m - t.r0, t.ob.n - t.c0, std::min<int64_t>(t.ob.ktot, t.s1 * ks) - t.s0 * ks).lat;

@@ -684,27 +684,41 @@ void Plan::encode_maps(const void* img_base) {
 // scatters and transposes of 128 two-site problems 640 -> 540 us, a U(1) permute,
 // fuse and split of 470 MB 246 -> 237 us.  Only launches of flat items: with
 // recoupling sums (SU(2), FP64: 237 -> 263 us) the order of the sectors is the
-// better one, where items that share their sources are neighbours.
+// better one, where items that share their sources are neighbours.  And only
+// stretches of at most kMaxSorted items: beyond 200 items a warp the shares are
+// even anyway (the full-size SU(2) recoupling contraction with gradients, 21.5
+// million items: 90.0 ms in the order of the sectors, 90.6 sorted), and sorting
+// them took 2.0 of 9.8 s of planning.
+constexpr int kMaxSorted = 1 << 20;
 void Plan::sort_items() {
   std::vector<int> cut = {0, (int)items.size()};  // items between two cuts are in the same launches
   for (const Range* r : {&xform, &fwd_gather, &fwd_scatter, &bwd_gather_a, &bwd_gather_b, &bwd_scatter_a, &bwd_scatter_b})
     if (r->count > 0) cut.insert(cut.end(), {r->first, r->first + r->count});
   std::sort(cut.begin(), cut.end());
-  std::vector<int> ord(items.size()), cls(items.size());
-  for (size_t i = 0; i < items.size(); ++i) {
-    ord[i] = (int)i;
-    cls[i] = std::ilogb((double)items[i].count * std::max(1, items[i].nterm));
+  std::vector<std::pair<int, int>> ord;  // (class, item) of one stretch
+  std::vector<BoxItem> sorted;
+  std::vector<double> bytes;
+  for (size_t k = 0; k + 1 < cut.size(); ++k) {
+    const int i0 = cut[k], i1 = cut[k + 1];
+    if (i1 - i0 > kMaxSorted) continue;
+    if (!std::all_of(items.begin() + i0, items.begin() + i1, [](const BoxItem& i) { return i.sel & kSelFlat; })) continue;
+    ord.clear();
+    ord.reserve(i1 - i0);
+    for (int i = i0; i < i1; ++i) ord.push_back({std::ilogb((double)items[i].count * std::max(1, items[i].nterm)), i});
+    auto larger = [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first > y.first; };
+    if (std::is_sorted(ord.begin(), ord.end(), larger)) continue;
+    std::stable_sort(ord.begin(), ord.end(), larger);
+    sorted.clear();
+    bytes.clear();
+    sorted.reserve(ord.size());
+    bytes.reserve(ord.size());
+    for (auto& o : ord) {
+      sorted.push_back(items[o.second]);
+      bytes.push_back(item_bytes_prefix[o.second + 1]);
+    }
+    std::copy(sorted.begin(), sorted.end(), items.begin() + i0);
+    std::copy(bytes.begin(), bytes.end(), item_bytes_prefix.begin() + i0 + 1);
   }
-  for (size_t k = 0; k + 1 < cut.size(); ++k)
-    if (std::all_of(items.begin() + cut[k], items.begin() + cut[k + 1], [](const BoxItem& i) { return i.sel & kSelFlat; }))
-      std::stable_sort(ord.begin() + cut[k], ord.begin() + cut[k + 1], [&](int a, int b) { return cls[a] > cls[b]; });
-  std::vector<BoxItem> sorted(items.size());
-  std::vector<double> bytes(item_bytes_prefix);
-  for (size_t i = 0; i < items.size(); ++i) {
-    sorted[i] = items[ord[i]];
-    item_bytes_prefix[i + 1] = bytes[ord[i] + 1];
-  }
-  items.swap(sorted);
 }
 
 void Plan::upload(bool device) {
@@ -1388,7 +1402,6 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
     }
   }
   const bool tree = su2_like(Am.group);
-  std::map<std::array<int64_t, 3>, double> sum;  // SU(2): products met through several intermediate labels
   std::vector<int> key;
   for (const Pair& p : pairs) {
     key.assign(Am.pos.begin() + p.a * Am.rank, Am.pos.begin() + p.a * Am.rank + na);
@@ -1417,12 +1430,10 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
     useful += mnk;
     for (auto& xa : XA[p.a])
       for (auto& xb : XB[p.b]) {
-        if (!tree) {
+        if (!tree || natural) {
           out->push_back({xa.first, xb.first, c, xa.second * xb.second});
-        } else if (natural) {
-          sum[{xa.first, xb.first, c}] += xa.second * xb.second;
         } else {
-          for (auto& xc : XCt[c]) sum[{xa.first, xb.first, xc.first}] += xa.second * xb.second * xc.second;
+          for (auto& xc : XCt[c]) out->push_back({xa.first, xb.first, xc.first, xa.second * xb.second * xc.second});
         }
         if (++count > kMaxTriples) return false;
       }
@@ -1430,8 +1441,16 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
   }
   if (tree) {
     if (work > 4.0 * useful) return false;
-    for (auto& t : sum)
-      if (std::fabs(t.second) > 1e-13) out->push_back({t.first[0], t.first[1], t.first[2], t.second});
+    // products met through several intermediate labels, summed
+    auto key3 = [](const BlkTriple& t) { return std::array<int64_t, 3>{t.a, t.b, t.c}; };
+    std::stable_sort(out->begin(), out->end(), [&](const BlkTriple& x, const BlkTriple& y) { return key3(x) < key3(y); });
+    size_t n = 0;
+    for (size_t i = 0; i < out->size();) {
+      BlkTriple t = (*out)[i];
+      for (++i; i < out->size() && key3((*out)[i]) == key3(t); ++i) t.coef += (*out)[i].coef;
+      if (std::fabs(t.coef) > 1e-13) (*out)[n++] = t;
+    }
+    out->resize(n);
   }
   return true;
 }
@@ -1597,28 +1616,39 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
     std::vector<BlkTriple> triples;
     if (block_triples(Am, Bm, Cn, MA, MB, na, nc, XA, XB, XCt, natural, &triples)) {
       // all three phases or none: the matrix form shares its gathers between them
-      const double share = 1.0 / std::max(nbatch, 1);
-      double blk_us = 0.0, mat_us = 0.0;
-      bool ok = true;
-      for (int ph = 0; ph < 3 && ok; ++ph) {
-        std::vector<std::array<int64_t, 4>> mnk;  // the phase's GEMMs in matrix form, with their kernel kinds
+      const double share = 1.0 / std::max(nbatch, 1), win = nbatch > 1 ? 0.5 : 1.0;
+      std::vector<std::array<int64_t, 4>> mnk[3];  // the phases' GEMMs in matrix form, with their kernel kinds
+      double blk_us = 0.0, mat_us = 0.0, fma = 0.0;
+      for (int ph = 0; ph < 3; ++ph) {
         for (auto& g : gs)
-          mnk.push_back(ph == 0 ? std::array<int64_t, 4>{g.m, g.n, g.k, g.kind[0]}
-                                : ph == 1 ? std::array<int64_t, 4>{g.m, g.k, g.n, g.kind[1]}
-                                          : std::array<int64_t, 4>{g.k, g.n, g.m, g.kind[2]});
+          mnk[ph].push_back(ph == 0 ? std::array<int64_t, 4>{g.m, g.n, g.k, g.kind[0]}
+                                    : ph == 1 ? std::array<int64_t, 4>{g.m, g.k, g.n, g.kind[1]}
+                                              : std::array<int64_t, 4>{g.k, g.n, g.m, g.kind[2]});
+        mat_us += matrix_form_us(f64, mnk[ph], share);
+      }
+      for (auto& t : triples) {
+        double f = 1.0;
+        for (int l = 0; l < A.rank; ++l) f *= A.dim(t.a, l);
+        for (int l : freeB) f *= B.dim(t.b, l);
+        fma += f;
+      }
+      // work lists only where the arithmetic alone does not decide it: those of a
+      // rejected contraction took half of the planning time of a large one
+      bool ok = 3.0 * block_floor_us(f64, fma) < mat_us * win;
+      for (int ph = 0; ph < 3 && ok; ++ph) {
         double us = 0.0;
         ok = plan_block_phase(*P, ph, A, B, C, triples, freeA, freeB, pairsA, pairsB, share, &us);
         blk_us += us;
-        mat_us += matrix_form_us(f64, mnk, share);
+        ok = ok && blk_us < mat_us * win;
         P->blk_flops[ph] = P->flops_fwd;
         for (size_t i = 0; i < gs.size(); ++i)
           if (su2 || gs[i].k > tp.direct_max || gs[i].n > tp.direct_max)  // tiny sectors are no GEMMs
-            P->blk_mnk.push_back({(int)mnk[i][0], (int)mnk[i][1], (int)mnk[i][2]});
+            P->blk_mnk.push_back({(int)mnk[ph][i][0], (int)mnk[ph][i][1], (int)mnk[ph][i][2]});
       }
       // in a batch the matrix form's launches run for the other problems anyway:
       // taking some problems out of them pays only where the blocks win clearly
       // (128 two-site problems: 2.35 ms in matrix form, 2.47 ms at a factor of 1)
-      P->blocks = ok && blk_us < mat_us * (nbatch > 1 ? 0.5 : 1.0);
+      P->blocks = ok;
       if (!P->blocks) drop_blocks(*P);
     }
   }

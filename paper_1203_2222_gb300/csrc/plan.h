@@ -191,6 +191,8 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
                       const std::vector<BlkTriple>& triples, const std::vector<int>& freeA,
                       const std::vector<int>& freeB, const std::vector<int>& pairsA, const std::vector<int>& pairsB,
                       double share, double* model_us);
+// No phase with this many multiply-adds is modelled faster than this.
+double block_floor_us(bool f64, double fma);
 void drop_blocks(Plan& P);  // takes the lists of every phase out again
 void validate_blocks(const Plan& P);
 double blk_tile_cost(bool f64, const BlkTile& t);  // modelled clocks of a tile (launch order)
