@@ -632,6 +632,7 @@ __device__ int jacobi_sweeps_gram(float* W, float* V, int R, int C, int bw, int 
   // warps 0 .. GW-1 rotate the Gram matrix, GW .. GW+QW-1 Q
   constexpr int GW = (BW * BW + 31) / 32, QW = (BW * QP / 4 + 31) / 32;
   static_assert(GW + QW <= NW, "threads of a set");
+  static_assert(QP % 4 == 0 && (N * QP) % 4 == 0, "Qt's rows and what follows start on 16 bytes (as does N * gram_pitch)");
   const int tid = threadIdx.x, warp = tid >> 5;
   const int gx = tid / BW, gy = tid % BW;
   const int qx = tid < 32 * GW ? BW : (tid - 32 * GW) / (QP / 4), qy = tid < 32 * GW ? 0 : (tid - 32 * GW) % (QP / 4);
@@ -979,7 +980,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   __shared__ double wsum[(kThreads32 / 32)];
   __shared__ double fpart;  // this CTA's part of the squared Frobenius norm
   __shared__ float lred[(kThreads32 / 32) + 1], lsh[2 * kLanczos + 1];
-  extern __shared__ double sm_pair[];  // the sweeps by column blocks: a block pair of W and V
+  // the sweeps by column blocks: a block pair of W and V (16-byte vectors in jacobi_sweeps_gram)
+  extern __shared__ __align__(16) double sm_pair[];
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
   const int bi = blockIdx.x / kSvdCluster;
@@ -1409,7 +1411,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
                      int* __restrict__ err) {
   __shared__ unsigned long long nrot;
   __shared__ SweepCtl ctl;
-  extern __shared__ double sm_pair[];  // the sweeps by column blocks: a block pair of W and V
+  // the sweeps by column blocks: a block pair of W and V (16-byte vectors in jacobi_sweeps_gram)
+  extern __shared__ __align__(16) double sm_pair[];
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
   const int bi = blockIdx.x / kSvdCluster;
