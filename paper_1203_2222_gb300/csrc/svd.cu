@@ -182,15 +182,31 @@ __device__ __forceinline__ T warp_sum(T v) {
 template <typename T>
 struct JacobiArith;
 
+// Approximate root of x (of 0 for x < 0, where a rotated Gram matrix's diagonal can end up).
+__device__ __forceinline__ float sqrt_approx(float x) {
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(x) : "f"(fmaxf(x, 0.0f)));
+  return x;
+}
+// tan(theta) of a pair in FP32, d = bb - a and h = 2 g: 1 / (zeta + sign(zeta)
+// sqrt(zeta^2 + 1)), zeta = d / h.  Only ratios are squared: the squares of d and
+// h underflow for columns below 1e-10 of max |A| (equal ones, d = 0, then made
+// t = h / 0).  h is normal (kMinCoupling).
+__device__ __forceinline__ float tangent(float d, float h) {
+  const float zeta = __fdividef(d, h), z = fabsf(zeta);
+  return copysignf(__fdividef(1.0f, z + sqrt_approx(fmaf(z, z, 1.0f))), zeta);  // 0 where z^2 is infinite
+}
+constexpr float kMinCoupling = FLT_MIN;  // |w_p.w_q| below this is underflow, not an angle
+
 template <>
 struct JacobiArith<float> {
   // the FP32 sweeps only choose a starting point: approximate roots and quotients
-  static __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+  // |w_p| |w_q| (the product of the squared norms underflows before they do; with
+  // approximate roots here the pair loop spills twice as much: 7% at D = 96)
+  static __device__ __forceinline__ float norms(float a, float bb) { return sqrtf(a) * sqrtf(bb); }
   static __device__ __forceinline__ bool angle(float a, float bb, float g, float sab, float tol, float& c,
                                                float& s) {
-    if (!(fabsf(g) > tol * sab)) return false;
-    const float d = bb - a, h = 2.0f * g;  // t = sign(d) h / (|d| + sqrt(d^2 + h^2))
-    const float t = __fdividef(copysignf(1.0f, d) * h, fabsf(d) + root(fmaf(d, d, h * h)));
+    if (!(fabsf(g) > tol * sab && fabsf(g) > kMinCoupling)) return false;
+    const float t = tangent(bb - a, 2.0f * g);
     c = rsqrtf(fmaf(t, t, 1.0f));
     s = c * t;
     return true;
@@ -199,7 +215,7 @@ struct JacobiArith<float> {
 
 template <>
 struct JacobiArith<double> {
-  static __device__ __forceinline__ double root(double x) { return sqrt(x); }
+  static __device__ __forceinline__ double norms(double a, double bb) { return sqrt(a * bb); }
   // The angle itself needs only FP32 accuracy: an inexact angle is still an
   // exact rotation (c^2 + s^2 = 1 to FP64 precision), it just leaves the
   // pair slightly non-orthogonal for the next sweep.  So t = sign(d) h /
@@ -271,7 +287,7 @@ __device__ __forceinline__ int rotate_pair(T* wp, T* wq, T* vp, T* vq, T* na, T*
 #pragma unroll
   for (int u = 0; u < NR; ++u) g = fma(xw[u], yw[u], g);
   g = warp_sum(g);
-  const T sab = sqrt(a * bb);
+  const T sab = JacobiArith<T>::norms(a, bb);
   T c, s;
   if (!JacobiArith<T>::angle(a, bb, g, sab, tol, c, s)) return 0;
 #pragma unroll
@@ -307,7 +323,7 @@ __device__ __noinline__ int rotate_pair_stream(T* wp, T* wq, T* vp, T* vq, int R
   a = warp_sum(a);
   bb = warp_sum(bb);
   g = warp_sum(g);
-  const T sab = sqrt(a * bb);
+  const T sab = JacobiArith<T>::norms(a, bb);
   T c, s;
   if (!JacobiArith<T>::angle(a, bb, g, sab, tol, c, s)) return 0;
   for (int i = lane; i < R; i += 32) {
@@ -435,7 +451,7 @@ __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* n
   }
   g = warp_sum(g);
   const T a = *na, bb = *nb;
-  const T sab = JacobiArith<T>::root(a * bb);
+  const T sab = JacobiArith<T>::norms(a, bb);
   T c, sn;
   if (!JacobiArith<T>::angle(a, bb, g, sab, tol, c, sn)) return 0;
 #pragma unroll
@@ -615,9 +631,6 @@ __host__ __device__ inline int64_t gram_floats(int R, int C, int bw) {
   const int64_t n = 2 * bw, qp = (n + 3) / 4 * 4;
   return n * gram_pitch(R) + n * qp + 2 * n * (n + 1) + n * C;
 }
-__device__ __forceinline__ float sqrt_approx(float x) {  // of x >= 0, no branch
-  return x * rsqrtf(fmaxf(x, FLT_MIN));
-}
 template <int BW>
 __device__ int jacobi_sweeps_gram(float* W, float* V, int R, int C, int bw, int max_sweeps, float tol,
                                   cg::cluster_group& cluster, SweepCtl* ctl, int* flag0, int crank, int lane,
@@ -721,11 +734,10 @@ __device__ int jacobi_sweeps_gram(float* W, float* V, int R, int C, int bw, int 
             }
           };
           // no branches: a warp's threads look at different pairs, a thread at two
-          auto angle = [&](int p, int q, float& c, float& s) {  // 0: no rotation, 1, or 2: a large one
-            const float a = G[p * GP + p], b = G[q * GP + q], g = G[p * GP + q];
-            const float sab = sqrt_approx(a * b), d = b - a, h = 2.0f * g;
-            const float t = __fdividef(copysignf(1.0f, d) * h, fabsf(d) + sqrt_approx(fmaf(d, d, h * h)));
-            const bool on = fabsf(g) > tol * sab;
+          auto angle = [&](int i, int j, float& c, float& s) {  // 0: no rotation, 1, or 2: a large one
+            const float a = G[i * GP + i], b = G[j * GP + j], g = G[i * GP + j];
+            const float sab = sqrt_approx(a) * sqrt_approx(b), t = tangent(b - a, 2.0f * g);
+            const bool on = fabsf(g) > fmaxf(tol * sab, kMinCoupling);
             c = on ? rsqrtf(fmaf(t, t, 1.0f)) : 1.0f;
             s = on ? c * t : 0.0f;
             return on ? (fabsf(g) > big_tol * sab ? 2 : 1) : 0;

@@ -1,0 +1,50 @@
+"""Blockwise SVD and eigendecomposition (csrc/svd.cu) of blocks whose columns
+or whose values lie far from 1: the angles of the FP32 sweeps, the norms and
+the levels of the refinement keep their ratios at every scale."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1203_2222_gb300 as P
+from paper_1203_2222_gb300 import synthetic
+
+pytestmark = pytest.mark.gpu
+
+
+def _mat(n, m, seed):
+    return synthetic.normal(seed, n * m).reshape(n, m)
+
+
+def _svd(M):
+    """(u, s, w) of one block on the GPU."""
+    n, m = M.shape
+    k = min(n, m)
+    S = P.Structure(P.U1, [([0], [n], 1), ([0], [m], -1)])
+    U, s, V = P.svd(P.SymTensor(S, torch.as_tensor(np.ascontiguousarray(M).reshape(-1)).cuda()), 1)
+    torch.cuda.synchronize()
+    P.device_status()
+    return U.data.cpu().numpy().reshape(n, k), s.cpu().numpy(), V.data.cpu().numpy().reshape(k, m)
+
+
+def _pairs_of_tiny_columns(n, e):
+    """One entry 1; the other columns random, e times as large, and two of them equal."""
+    M = np.zeros((n, n))
+    M[0, 0] = 1.0
+    M[1:, 1:] = e * _mat(n - 1, n - 1, 77)
+    M[1:, 2] = M[1:, 1]
+    return M
+
+
+# e^2 is still a normal FP32 number for the first three, e^4 for the first one
+# only; n: the sweeps by pairs and through Gram matrices
+@pytest.mark.parametrize("e", [1e-8, 1e-11, 1e-13, 1e-18])
+@pytest.mark.parametrize("n", [3, 40, 70])
+def test_svd_with_equal_tiny_columns(n, e):
+    M = _pairs_of_tiny_columns(n, e)
+    u, s, w = _svd(M)
+    ref = np.linalg.svd(M, compute_uv=False)
+    # the values next to 1 to FP64 accuracy of e: the columns' own scale
+    assert abs(s[0] - 1.0) <= 1e-14
+    assert np.max(np.abs(s[1:] - ref[1:])) <= 1e-12 * e * np.sqrt(n)
+    assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
+    assert np.max(np.abs((u * s) @ w - M)[1:, 1:]) <= 1e-12 * e * np.sqrt(n)
