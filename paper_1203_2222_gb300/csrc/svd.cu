@@ -986,8 +986,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
     svd_jacobi_kernel(const SvdBlock* __restrict__ blocks, const SvdPiece* __restrict__ pieces,
                       const double* __restrict__ T, double* __restrict__ work, SvdState* __restrict__ state,
                       int* __restrict__ sweeps, long long* __restrict__ rotations) {
-  __shared__ unsigned long long nrot;
-  __shared__ unsigned long long amax;
+  __shared__ unsigned long long nrot;  // rotations of this CTA
+  __shared__ unsigned long long wmax[kThreads32 / 32], amax;  // the largest |A| of its warps, of this CTA
   __shared__ SweepCtl ctl;
   __shared__ double wsum[(kThreads32 / 32)];
   __shared__ double fpart;  // this CTA's part of the squared Frobenius norm
@@ -1009,11 +1009,11 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   constexpr int kCT = kSvdCluster * kThreads32;
   if (tid == 0) {
     nrot = 0;
-    amax = 0;
     ctl.flag[0] = ctl.flag[1] = 0;
     ctl.any = 0;
+    if (crank == 0) rotations[2 * b.slot] = rotations[2 * b.slot + 1] = 0;
   }
-  cluster.sync();  // shared state initialised before any remote access
+  cluster.sync();  // shared state initialised before any remote access, the counts before they are added to
 
   // A (m >= n: M_x, else M_x^T) in FP64, column-major, and max |A|
   for (int64_t i = ct; i < RC; i += kCT) __stcg(A + i, 0.0);
@@ -1069,9 +1069,21 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   f2 = 0.0;  // the same sum, in the same order, in every thread
   for (int r = 0; r < kSvdCluster; ++r) f2 += *cluster.map_shared_rank(&fpart, r);
   const double shift = b.eig ? sqrt(f2) : 0.0;  // eig: sigma
-  if (mx) atomicMax(cluster.map_shared_rank(&amax, 0), mx);
+  // the largest |A| of all CTAs, read from each of them (64-bit atomics on
+  // another CTA's shared memory lost the larger value now and then: a block
+  // with one large entry was then scaled out of FP32's range)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) wmax[tid >> 5] = mx;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < kThreads32 / 32; ++w) mx = max(mx, wmax[w]);
+    amax = mx;
+  }
   cluster.sync();
-  const double amx = __longlong_as_double((long long)*cluster.map_shared_rank(&amax, 0));
+  mx = 0;
+  for (int r = 0; r < kSvdCluster; ++r) mx = max(mx, *cluster.map_shared_rank(&amax, r));
+  const double amx = __longlong_as_double((long long)mx);
   // scale sa = 2^-e with 2^e <= max |A| < 2^(e+1); 1 for a zero or non-finite block
   const int ex = (__double2hiint(amx) >> 20) & 0x7ff;
   const bool scaled = ex > 0 && ex < 2046;
@@ -1120,14 +1132,13 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
       sw32 = jacobi_sweeps<float, kThreads32>(W32, V32, nrm32, R, C, kMaxSweeps32, tol32, cluster, &ctl, flag0, crank, cw, lane,
                                   gsweep, rot32, conv32, kBigRotation32);
   }
-  if (b.bw ? rot32 != 0 : lane == 0 && rot32) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot32);
+  if (b.bw ? rot32 != 0 : lane == 0 && rot32) atomicAdd(&nrot, rot32);
   for (int64_t i = ct; i < CC; i += kCT) __stcg(ws.V + i, (double)__ldcg(V32 + i));
-  cluster.sync();  // the rotation counts have arrived at rank 0
+  cluster.sync();  // no CTA leaves while its shared memory is read
+  if (tid == 0 && nrot) atomicAdd(reinterpret_cast<unsigned long long*>(rotations + 2 * b.slot + 1), nrot);
   if (crank == 0 && tid == 0) {
     sweeps[2 * b.slot + 1] = sw32;
-    rotations[2 * b.slot + 1] = (long long)nrot;
     sweeps[2 * b.slot] = 0;
-    rotations[2 * b.slot] = 0;
     SvdState& st = state[bi];
     st.sa = sa;
     st.unsa = unsa;
@@ -1499,7 +1510,7 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
       sw64 = jacobi_sweeps<double, kSvdThreads>(W, V, nrm, R, C, kMaxSweeps, tol64, cluster, &ctl, flag0, crank, cw, lane, gsweep,
                                    rot64, conv, kBigRotation);
   }
-  if (lane == 0 && rot64) atomicAdd(cluster.map_shared_rank(&nrot, 0), rot64);
+  if (lane == 0 && rot64) atomicAdd(&nrot, rot64);
 
   // undo the scaling (a power of two: exact) and take the column norms
   for (int j = cw; j < C; j += kCW) {
@@ -1513,11 +1524,11 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     a = warp_sum(a);
     if (lane == 0) __stcg(nrm + j, sqrt(a) - shift);
   }
-  cluster.sync();  // the rotation counts have arrived at rank 0
+  cluster.sync();  // no CTA leaves while its shared memory is read
+  if (tid == 0 && nrot) atomicAdd(reinterpret_cast<unsigned long long*>(rotations + 2 * b.slot), nrot);
   if (crank == 0 && tid == 0) {
     if (!conv) atomicExch(err, SYM_ERR_NUMERIC);
     sweeps[2 * b.slot] = sw64;
-    rotations[2 * b.slot] = (long long)nrot;
   }
 }
 

@@ -48,3 +48,17 @@ def test_svd_with_equal_tiny_columns(n, e):
     assert np.max(np.abs(s[1:] - ref[1:])) <= 1e-12 * e * np.sqrt(n)
     assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
     assert np.max(np.abs((u * s) @ w - M)[1:, 1:]) <= 1e-12 * e * np.sqrt(n)
+
+
+@pytest.mark.parametrize("n", [39, 40, 41, 70])
+def test_svd_with_one_entry_far_above_the_others(n):
+    # scaled by any entry but the largest, the block is out of FP32's range (several
+    # runs: which CTA of the cluster finds the largest entry last is not fixed)
+    e = 1e-60
+    for seed in range(8):
+        M = e * _mat(n, n, seed)
+        M[seed % n, (3 * seed) % n] = 1.0
+        u, s, w = _svd(M)
+        assert abs(s[0] - 1.0) <= 1e-14 and np.all(np.abs(s[1:]) <= 1e-14)
+        assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
+        assert np.linalg.norm((u * s) @ w - M) <= 1e-14
