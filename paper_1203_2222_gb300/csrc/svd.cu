@@ -121,8 +121,7 @@ constexpr int kMaxRefine = 5;
 // What the kernels of one call hand on per block (blocks in launch order).
 struct SvdState {
   double sa, unsa;  // power-of-two scale of A, and its inverse
-  double shift;     // eig: sigma (the block's Frobenius norm)
-  double norm2;     // squared Frobenius norm of sa A
+  double norm;      // Frobenius norm of sa A (eig: sa sigma)
   unsigned xmax[kMaxRefine];  // bits of the largest squared column norm of a step's correction X (FP32)
   int nulls[kMaxRefine];      // SVD: a step left pairs of columns at the rounding level alone
   int done;         // refinement step after which the block counts as converged (0: not, -1: given up)
@@ -973,47 +972,26 @@ __device__ float lanczos_shift(const float* W, int C, float* v, float* vp, float
   return *cluster.map_shared_rank(sh + 2 * kLanczos, 0);
 }
 
-// One cluster of kSvdCluster CTAs per block: the pairs of a round are spread
-// over the cluster's warps and the rounds are separated by cluster barriers
-// (their release / acquire order the workspace writes; the workspace is read
-// and written at L2, bypassing L1, so no SM keeps a stale copy).
-//
-// Mixed precision.  GB300 runs FP32 at many times its FP64 rate, so the
-// sweeps that do most of the work run in FP32 on A scaled by a power of two
-// (max |A| in [1/2, 1): no FP32 overflow or underflow of the bulk).  Their V
-// is only the starting point: the refinement below takes it to FP64.
-__global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32, 2)
-    svd_jacobi_kernel(const SvdBlock* __restrict__ blocks, const SvdPiece* __restrict__ pieces,
-                      const double* __restrict__ T, double* __restrict__ work, SvdState* __restrict__ state,
-                      int* __restrict__ sweeps, long long* __restrict__ rotations) {
-  __shared__ unsigned long long nrot;  // rotations of this CTA
-  __shared__ unsigned long long wmax[kThreads32 / 32], amax;  // the largest |A| of its warps, of this CTA
-  __shared__ SweepCtl ctl;
-  __shared__ double wsum[(kThreads32 / 32)];
+// A block for the sweeps: A from the tensor's blocks (eig: its symmetric part), sa A
+// and I in FP32 (eig: sa A plus the shift), and the block's state.  A function of
+// its own: inlined, its values cost the sweeps registers (6% at D = 96).
+__device__ __noinline__ void load_block(const SvdBlock* __restrict__ block, const SvdPiece* __restrict__ pieces,
+                                        const double* __restrict__ T, double* __restrict__ work,
+                                        SvdState* __restrict__ state) {
+  __shared__ unsigned long long wmax[kThreads32 / 32], amax;  // the largest |A| of the warps, of this CTA
+  __shared__ double wsum[kThreads32 / 32];
   __shared__ double fpart;  // this CTA's part of the squared Frobenius norm
   __shared__ float lred[(kThreads32 / 32) + 1], lsh[2 * kLanczos + 1];
-  // the sweeps by column blocks: a block pair of W and V (16-byte vectors in jacobi_sweeps_gram)
-  extern __shared__ __align__(16) double sm_pair[];
   cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank();
-  const int bi = blockIdx.x / kSvdCluster;
-  const SvdBlock b = blocks[bi];
+  constexpr int kCT = kSvdCluster * kThreads32;
+  const int crank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31;
+  const int ct = crank * kThreads32 + tid, cw = ct >> 5;  // thread, warp of the cluster
+  const SvdBlock& b = *block;
   const int R = b.R, C = b.C;
   const int64_t RC = (int64_t)R * C, CC = (int64_t)C * C;
   const SvdWork ws(work + b.w, R, C);
   double* A = ws.A;
   float *W32 = ws.W32, *V32 = ws.V32;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int ct = crank * kThreads32 + tid;       // thread of the cluster
-  const int cw = crank * (kThreads32 / 32) + (tid >> 5);  // warp of the cluster
-  constexpr int kCT = kSvdCluster * kThreads32;
-  if (tid == 0) {
-    nrot = 0;
-    ctl.flag[0] = ctl.flag[1] = 0;
-    ctl.any = 0;
-    if (crank == 0) rotations[2 * b.slot] = rotations[2 * b.slot + 1] = 0;
-  }
-  cluster.sync();  // shared state initialised before any remote access, the counts before they are added to
 
   // A (m >= n: M_x, else M_x^T) in FP64, column-major, and max |A|
   for (int64_t i = ct; i < RC; i += kCT) __stcg(A + i, 0.0);
@@ -1031,44 +1009,22 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
     }
   }
   cluster.sync();  // the whole block is in A
-  // eig: the symmetric part, in place (the thread of (r, c), r < c, writes
-  // both halves); the squared Frobenius norm
-  double f2 = 0.0;
+  // eig: the symmetric part, in place (the thread of (r, c), r < c, writes both halves)
   if (b.eig) {
     mx = 0;
     for (int64_t e = ct; e < RC; e += kCT) {
       const int r = (int)(e % R), c = (int)(e / R);
-      double v = 0.0;
+      if (r > c) continue;
+      double v = __ldcg(A + e);
       if (r < c) {
         const int64_t t = c + (int64_t)r * R;
-        v = 0.5 * (__ldcg(A + e) + __ldcg(A + t));
+        v = 0.5 * (v + __ldcg(A + t));
         __stcg(A + e, v);
         __stcg(A + t, v);
-        f2 = fma(2.0 * v, v, f2);
-      } else if (r == c) {
-        v = __ldcg(A + e);
-        f2 = fma(v, v, f2);
       }
       mx = max(mx, (unsigned long long)__double_as_longlong(fabs(v)));
     }
-  } else {
-    for (int64_t e = ct; e < RC; e += kCT) {
-      const double v = __ldcg(A + e);
-      f2 = fma(v, v, f2);
-    }
   }
-  f2 = warp_sum(f2);
-  if (lane == 0) wsum[tid >> 5] = f2;
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (kThreads32 / 32); ++w) t += wsum[w];
-    fpart = t;
-  }
-  cluster.sync();  // every CTA's part and the symmetric part are written
-  f2 = 0.0;  // the same sum, in the same order, in every thread
-  for (int r = 0; r < kSvdCluster; ++r) f2 += *cluster.map_shared_rank(&fpart, r);
-  const double shift = b.eig ? sqrt(f2) : 0.0;  // eig: sigma
   // the largest |A| of all CTAs, read from each of them (64-bit atomics on
   // another CTA's shared memory lost the larger value now and then: a block
   // with one large entry was then scaled out of FP32's range)
@@ -1090,16 +1046,84 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   const double sa = scaled ? __hiloint2double((2046 - ex) << 20, 0) : 1.0;
   const double unsa = scaled ? __hiloint2double(ex << 20, 0) : 1.0;  // 1 / sa
 
-  for (int64_t i = ct; i < RC; i += kCT) __stcg(W32 + i, (float)(sa * __ldcg(A + i)));
+  // sa A in FP32, and its squared Frobenius norm in FP64: of the scaled values,
+  // whose squares neither overflow nor underflow, at any scale of the block
+  double f2 = 0.0;
+  for (int64_t i = ct; i < RC; i += kCT) {
+    const double v = sa * __ldcg(A + i);
+    f2 = fma(v, v, f2);
+    __stcg(W32 + i, (float)v);
+  }
   for (int64_t i = ct; i < CC; i += kCT) __stcg(V32 + i, (i % (C + 1) == 0) ? 1.0f : 0.0f);
-  cluster.sync();
+  f2 = warp_sum(f2);
+  if (lane == 0) wsum[tid >> 5] = f2;
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < (kThreads32 / 32); ++w) t += wsum[w];
+    fpart = t;
+  }
+  cluster.sync();  // every CTA's part, and W32, are written
+  f2 = 0.0;  // the same sum, in the same order, in every thread
+  for (int r = 0; r < kSvdCluster; ++r) f2 += *cluster.map_shared_rank(&fpart, r);
+  const double norm = sqrt(f2);  // of sa A
   if (b.eig) {  // the FP32 sweeps run on B + a shift; A keeps B
     const double s = C >= 4 ? (double)lanczos_shift(W32, C, ws.F0, ws.F0 + C, ws.F0 + 2 * C, cluster, lred, lsh, crank, cw, lane)
-                            : sa * shift;
+                            : norm;
     for (int j = ct; j < C; j += kCT)
       __stcg(W32 + j + (int64_t)j * R, (float)(sa * __ldcg(A + j + (int64_t)j * R) + s));
     cluster.sync();
   }
+  if (crank == 0 && tid == 0) {
+    SvdState& st = *state;
+    st.sa = sa;
+    st.unsa = unsa;
+    st.norm = norm;
+    st.done = 0;
+    for (int i = 0; i < kMaxRefine; ++i) {
+      st.xmax[i] = 0;
+      st.nulls[i] = 0;
+    }
+  }
+}
+
+// One cluster of kSvdCluster CTAs per block: the pairs of a round are spread
+// over the cluster's warps and the rounds are separated by cluster barriers
+// (their release / acquire order the workspace writes; the workspace is read
+// and written at L2, bypassing L1, so no SM keeps a stale copy).
+//
+// Mixed precision.  GB300 runs FP32 at many times its FP64 rate, so the
+// sweeps that do most of the work run in FP32 on A scaled by a power of two
+// (max |A| in [1/2, 1): no FP32 overflow or underflow of the bulk).  Their V
+// is only the starting point: the refinement below takes it to FP64.
+__global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32, 2)
+    svd_jacobi_kernel(const SvdBlock* __restrict__ blocks, const SvdPiece* __restrict__ pieces,
+                      const double* __restrict__ T, double* __restrict__ work, SvdState* __restrict__ state,
+                      int* __restrict__ sweeps, long long* __restrict__ rotations) {
+  __shared__ unsigned long long nrot;  // rotations of this CTA
+  __shared__ SweepCtl ctl;
+  // the sweeps by column blocks: a block pair of W and V (16-byte vectors in jacobi_sweeps_gram)
+  extern __shared__ __align__(16) double sm_pair[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int crank = (int)cluster.block_rank();
+  const int bi = blockIdx.x / kSvdCluster;
+  const SvdBlock b = blocks[bi];
+  const int R = b.R, C = b.C;
+  const int64_t CC = (int64_t)C * C;
+  const SvdWork ws(work + b.w, R, C);
+  float *W32 = ws.W32, *V32 = ws.V32;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ct = crank * kThreads32 + tid;       // thread of the cluster
+  const int cw = crank * (kThreads32 / 32) + (tid >> 5);  // warp of the cluster
+  constexpr int kCT = kSvdCluster * kThreads32;
+  if (tid == 0) {
+    nrot = 0;
+    ctl.flag[0] = ctl.flag[1] = 0;
+    ctl.any = 0;
+    if (crank == 0) rotations[2 * b.slot] = rotations[2 * b.slot + 1] = 0;
+  }
+  cluster.sync();  // shared state initialised before any remote access, the counts before they are added to
+  load_block(blocks + bi, pieces, T, work, state + bi);
 
   int* flag0 = cluster.map_shared_rank(ctl.flag, 0);
   unsigned long long rot32 = 0;
@@ -1139,16 +1163,6 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kThreads32
   if (crank == 0 && tid == 0) {
     sweeps[2 * b.slot + 1] = sw32;
     sweeps[2 * b.slot] = 0;
-    SvdState& st = state[bi];
-    st.sa = sa;
-    st.unsa = unsa;
-    st.shift = shift;
-    st.norm2 = sa * sa * f2;
-    st.done = 0;
-    for (int i = 0; i < kMaxRefine; ++i) {
-      st.xmax[i] = 0;
-      st.nulls[i] = 0;
-    }
   }
 }
 
@@ -1304,11 +1318,11 @@ __global__ void __launch_bounds__(256)
   const SvdWork ws(work + b.w, b.R, b.C);
   const int C = b.C, q = bq.y;
   const double aq = ws.G[q + (int64_t)q * C], eqq = ws.E[q + (int64_t)q * C] - 1.0;
-  const double tol = b.eig ? 4.0 * DBL_EPSILON * st.sa * st.shift : sqrt((double)b.R) * DBL_EPSILON;
+  const double tol = b.eig ? 4.0 * DBL_EPSILON * st.norm : sqrt((double)b.R) * DBL_EPSILON;
   const float sq = sqrtf((float)aq);
   // a null space's off-diagonal elements: of W^T W they are squares of the
   // error of V times the squared norm, of V^T B V times the norm
-  const double null_level = (step == 0 ? 1e-10 : step == 1 ? 1e-18 : 1e-27) * (b.eig ? sqrt(st.norm2) : st.norm2);
+  const double null_level = (step == 0 ? 1e-10 : step == 1 ? 1e-18 : 1e-27) * st.norm * (b.eig ? 1.0 : st.norm);
   const double near = step == 0 ? 1e-6 : step == 1 ? 1e-11 : 0.0;
   bool skipped = false;
   float n2 = 0.0f, diag = 0.0f;
@@ -1333,7 +1347,7 @@ __global__ void __launch_bounds__(256)
       }
       const double big = fmax(aq, ap);
       if ((fabs(g) <= null_level && (fabsf(t) > 0.05f || (b.eig ? fabs(d) : big) <= null_level)) ||
-          m <= near * (b.eig ? sqrt(st.norm2) : big)) {
+          m <= near * (b.eig ? st.norm : big)) {
         skipped = true;
       } else {
         const float c = rsqrtf(fmaf(t, t, 1.0f));
@@ -1442,7 +1456,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
   const int done = state[bi].done;  // the same for the whole cluster
   const SvdBlock b = blocks[bi];
   if (refined(state[bi], b)) return;
-  const double sa = state[bi].sa, unsa = state[bi].unsa, shift = state[bi].shift;
+  const double sa = state[bi].sa, unsa = state[bi].unsa;
+  const double shift = b.eig ? state[bi].norm : 0.0;  // sa sigma
   const int R = b.R, C = b.C;
   const int64_t CC = (int64_t)C * C;
   const SvdWork ws(work + b.w, R, C);
@@ -1466,8 +1481,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     // two Newton-Schulz steps through the G buffer, the first one's product in
     // W's buffer (free until W = A V)
     for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, (double)__ldcg(ws.V32 + i));
-    if (b.eig)
-      for (int j = ct; j < C; j += kCT) __stcg(A + j + (int64_t)j * R, __ldcg(A + j + (int64_t)j * R) + shift);
+    if (b.eig)  // sa (B + sigma I)
+      for (int64_t i = ct; i < CC; i += kCT) __stcg(A + i, sa * __ldcg(A + i) + (i % (C + 1) == 0 ? shift : 0.0));
     cluster.sync();
     newton_schulz_factor(V, C, G, cw, lane);
     cluster.sync();
@@ -1477,7 +1492,7 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     cluster.sync();
     gemm_cols(W, C, C, G, V, 1.0, cw, lane);
     cluster.sync();
-    gemm_cols(A, R, C, V, W, sa, cw, lane);  // W = (sa A) V
+    gemm_cols(A, R, C, V, W, b.eig ? 1.0 : sa, cw, lane);  // W = (sa A) V
     cluster.sync();
   }
 
@@ -1512,17 +1527,18 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
   }
   if (lane == 0 && rot64) atomicAdd(&nrot, rot64);
 
-  // undo the scaling (a power of two: exact) and take the column norms
+  // take the column norms (of the scaled columns: their squares stay in range)
+  // and undo the scaling (a power of two: exact)
   for (int j = cw; j < C; j += kCW) {
     double* wj = W + (int64_t)j * R;
     double a = 0.0;
     for (int i = lane; i < R; i += 32) {
-      const double x = unsa * __ldcg(wj + i);
-      __stcg(wj + i, x);
+      const double x = __ldcg(wj + i);
+      __stcg(wj + i, unsa * x);
       a = fma(x, x, a);
     }
     a = warp_sum(a);
-    if (lane == 0) __stcg(nrm + j, sqrt(a) - shift);
+    if (lane == 0) __stcg(nrm + j, unsa * (sqrt(a) - shift));
   }
   cluster.sync();  // no CTA leaves while its shared memory is read
   if (tid == 0 && nrot) atomicAdd(reinterpret_cast<unsigned long long*>(rotations + 2 * b.slot), nrot);
@@ -1532,7 +1548,7 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
   }
 }
 
-// Refined blocks: W (the last step's W2, scaling undone) and its column norms,
+// Refined blocks: W (the last step's W2, scaling undone) and its column norms (as in svd_sweep_kernel),
 // and V, to their places; a warp per column.
 __global__ void __launch_bounds__(256)
     svd_place_kernel(const SvdBlock* __restrict__ blocks, const int2* __restrict__ cols, int ncols,
@@ -1548,12 +1564,12 @@ __global__ void __launch_bounds__(256)
   if (!b.eig) {
     double a = 0.0;
     for (int i = lane; i < R; i += 32) {
-      const double x = st.unsa * ws.W2[i + (int64_t)j * R];
-      ws.W[i + (int64_t)j * R] = x;
+      const double x = ws.W2[i + (int64_t)j * R];
+      ws.W[i + (int64_t)j * R] = st.unsa * x;
       a = fma(x, x, a);
     }
     a = warp_sum(a);
-    if (lane == 0) ws.nrm[j] = sqrt(a);
+    if (lane == 0) ws.nrm[j] = st.unsa * sqrt(a);
   }
   if (st.done & 1)
     for (int i = lane; i < C; i += 32) ws.V[i + (int64_t)j * C] = ws.V2[i + (int64_t)j * C];

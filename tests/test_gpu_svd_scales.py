@@ -62,3 +62,34 @@ def test_svd_with_one_entry_far_above_the_others(n):
         assert abs(s[0] - 1.0) <= 1e-14 and np.all(np.abs(s[1:]) <= 1e-14)
         assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
         assert np.linalg.norm((u * s) @ w - M) <= 1e-14
+
+
+def _eig(M):
+    n = M.shape[0]
+    S = P.Structure(P.U1, [([0], [n], 1), ([0], [n], -1)])
+    U, lam, _ = P.eig(P.SymTensor(S, torch.as_tensor(np.ascontiguousarray(M).reshape(-1)).cuda()), 1)
+    torch.cuda.synchronize()
+    P.device_status()
+    return U.data.cpu().numpy().reshape(n, n), lam.cpu().numpy()
+
+
+# squares of the values over- and underflow beyond 1e+-154; the same block scaled by a
+# power of two has the same factors, and values that differ by that power alone
+@pytest.mark.parametrize("power", [-1000, -660, -531, -520, -512, 512, 531, 660, 1000])
+@pytest.mark.parametrize("n", [2, 40, 70])
+def test_values_whose_squares_leave_the_range(n, power):
+    M = _mat(n, n + 1, 18)
+    u, s, w = _svd(M)
+    u2, s2, w2 = _svd(np.ldexp(M, power))
+    np.testing.assert_array_equal(np.ldexp(s2, -power), s)
+    np.testing.assert_array_equal(u2, u)
+    np.testing.assert_array_equal(w2, w)
+    B = _mat(n, n, 10)
+    B = 0.5 * (B + B.T)
+    q, lam = _eig(B)
+    q2, lam2 = _eig(np.ldexp(B, power))
+    np.testing.assert_array_equal(np.ldexp(lam2, -power), lam)
+    np.testing.assert_array_equal(q2, q)
+    ref = np.linalg.eigvalsh(B)
+    assert np.linalg.norm(B @ q - q * lam) <= 1e-12 * np.sqrt(n) * np.max(np.abs(ref))
+    assert np.max(np.abs(np.sort(lam) - ref)) <= 1e-12 * np.max(np.abs(ref))
