@@ -118,6 +118,9 @@ struct SvdBlock {
 
 // FP64 refinement steps after the FP32 sweeps before a block goes on to FP64 sweeps
 constexpr int kMaxRefine = 5;
+// squared norm of a column of sa A V below which an SVD block goes to the FP64
+// sweeps: its angles to the large columns are out of FP32's reach
+constexpr double kMinNorm2 = 1e-36;
 // What the kernels of one call hand on per block (blocks in launch order).
 struct SvdState {
   double sa, unsa;  // power-of-two scale of A, and its inverse
@@ -235,9 +238,9 @@ struct JacobiArith<double> {
       tf = copysignf(1.0f, df) * hf / (fabsf(df) + sqrtf(fmaf(df, df, hf * hf)));
     }
     double t;
-    if (tf != 0.0f && isfinite(tf)) {
+    if (fabsf(tf) >= FLT_MIN && isfinite(tf)) {
       t = (double)tf;
-    } else {  // out of FP32's reach: the angle in FP64
+    } else {  // out of FP32's reach (a subnormal tf has few digits: no sweep would end): the angle in FP64
       const double zeta = d / h;
       t = fabs(zeta) > 1e150 ? 0.5 / zeta : copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
     }
@@ -1368,6 +1371,10 @@ __global__ void __launch_bounds__(256)
     ws.X[q + (int64_t)q * C] = x;
     n2 = fmaf(x, x, n2);
     if (skipped && step < 2) n2 = fmaxf(n2, 1e-15f);  // not the last step
+    // a column of an SVD block this far below the others: X and W X, in FP32, no
+    // longer carry its corrections.  One-sided sweeps find such values (of graded
+    // columns) to full relative accuracy
+    if (!b.eig && aq > 0.0 && aq < kMinNorm2) n2 = 1.0f;
     atomicMax(&st.xmax[step], __float_as_uint(n2));  // n2 >= 0 orders as its bits, a NaN above all
     if (b.eig) ws.nrm[q] = st.unsa * (aq / (1.0 + eqq));  // lambda: the Rayleigh quotient
   }

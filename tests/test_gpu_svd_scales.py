@@ -93,3 +93,19 @@ def test_values_whose_squares_leave_the_range(n, power):
     ref = np.linalg.eigvalsh(B)
     assert np.linalg.norm(B @ q - q * lam) <= 1e-12 * np.sqrt(n) * np.max(np.abs(ref))
     assert np.max(np.abs(np.sort(lam) - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("e", [1e-16, 1e-20, 1e-25, 1e-45, 1e-60])
+@pytest.mark.parametrize("n", [5, 40, 70])
+def test_svd_with_one_tiny_column(n, e):
+    M = _mat(n, n, 21)
+    M[:, n - 1] *= e
+    u, s, w = _svd(M)
+    # the value of the tiny column: what the other columns do not span of it
+    Q, _ = np.linalg.qr(M[:, :n - 1])
+    x = M[:, n - 1] / e
+    x -= Q @ (Q.T @ x)
+    x -= Q @ (Q.T @ x)
+    assert abs(s[-1] / e - np.linalg.norm(x)) <= 1e-12 * np.linalg.norm(M) / np.min(s[:-1])
+    assert np.max(np.abs(u.T @ u - np.eye(n))) <= 1e-12
+    assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
