@@ -1443,6 +1443,35 @@ __global__ void __launch_bounds__(kTileThreads)
     }
 }
 
+// Columns of W at the rounding level of the block, |w| <= R eps |A|, can be exact
+// multiples of one another (a block with equal rows): rotations then shrink them
+// by eps a sweep without an end.  Sets such columns to 0 and returns whether the
+// others are orthogonal.
+__device__ bool drop_null_columns(double* W, int R, int C, double norm, cg::cluster_group& cluster, int* bad, int cw,
+                                  int lane) {
+  constexpr int kCW = kSvdCluster * (kSvdThreads / 32);
+  const double level = (double)R * DBL_EPSILON * norm;
+  auto dot = [&](int p, int q) {
+    double g = 0.0;
+    for (int i = lane; i < R; i += 32) g = fma(__ldcg(W + (int64_t)p * R + i), __ldcg(W + (int64_t)q * R + i), g);
+    return warp_sum(g);
+  };
+  for (int j = cw; j < C; j += kCW)
+    if (dot(j, j) <= level * level)
+      for (int i = lane; i < R; i += 32) __stcg(W + (int64_t)j * R + i, 0.0);
+  cluster.sync();
+  int b = 0;
+  for (int p = cw; p < C; p += kCW) {
+    const double a = dot(p, p);
+    for (int q = p + 1; q < C && a > 0.0; ++q) b |= !(fabs(dot(p, q)) <= 1e-13 * sqrt(a) * sqrt(dot(q, q)));
+  }
+  b = __syncthreads_or(b);
+  if (threadIdx.x == 0) *bad = b;
+  cluster.sync();
+  for (int r = 0; r < kSvdCluster; ++r) b |= *cluster.map_shared_rank(bad, r);
+  return !b;
+}
+
 // Blocks the refinement did not finish.  Where it converged but left columns
 // at the rounding level (SVD), FP64 sweeps on its W and V, which mostly find
 // nothing to rotate.  Else the FP32 V made orthogonal in FP64 by two
@@ -1455,6 +1484,7 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
                      int* __restrict__ err) {
   __shared__ unsigned long long nrot;
   __shared__ SweepCtl ctl;
+  __shared__ int bad;
   // the sweeps by column blocks: a block pair of W and V (16-byte vectors in jacobi_sweeps_gram)
   extern __shared__ __align__(16) double sm_pair[];
   cg::cluster_group cluster = cg::this_cluster();
@@ -1533,6 +1563,7 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
                                    rot64, conv, kBigRotation);
   }
   if (lane == 0 && rot64) atomicAdd(&nrot, rot64);
+  if (!conv && !b.eig) conv = drop_null_columns(W, R, C, state[bi].norm, cluster, &bad, cw, lane);
 
   // take the column norms (of the scaled columns: their squares stay in range)
   // and undo the scaling (a power of two: exact)

@@ -109,3 +109,20 @@ def test_svd_with_one_tiny_column(n, e):
     assert abs(s[-1] / e - np.linalg.norm(x)) <= 1e-12 * np.linalg.norm(M) / np.min(s[:-1])
     assert np.max(np.abs(u.T @ u - np.eye(n))) <= 1e-12
     assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
+
+
+@pytest.mark.parametrize("e", [1.0, 1e-8, 1e-11, 1e-13, 1e-18])
+@pytest.mark.parametrize("n", [5, 40, 70])
+def test_svd_with_equal_rows(n, e):
+    # one entry 1, all others in the rest equal: every column of A V that belongs to a
+    # zero value is rounding, and an exact multiple of every other
+    M = np.zeros((n, n))
+    M[0, 0] = 1.0
+    M[1:, 1:] = e
+    u, s, w = _svd(M)
+    ref = sorted([1.0, e * (n - 1)], reverse=True)
+    assert np.max(np.abs(s[:2] / ref - 1.0)) <= 1e-14
+    assert np.all(np.abs(s[2:]) <= n * 2.3e-16 * ref[0])
+    assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
+    assert np.max(np.abs(u[:, :2].T @ u[:, :2] - np.eye(2))) <= 1e-12
+    assert np.max(np.abs((u * s) @ w - M)[1:, 1:]) <= 1e-14 * e * n
