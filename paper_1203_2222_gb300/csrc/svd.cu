@@ -87,13 +87,21 @@ constexpr int kSvdSmem32Max = 112 * 1024;
 constexpr int kSvdSmem64Max = 100 * 1024;
 constexpr int kMaxSweeps = 64;    // FP64 sweeps before a block counts as not converged
 constexpr int kMaxSweeps32 = 40;  // FP32 sweeps (their result only seeds the FP64 ones)
-// An FP64 sweep whose rotations all had |w_p.w_q| <= kBigRotation |w_p| |w_q|
-// ends the sweeps: what it leaves is of order kBigRotation^2 from the pairs'
-// coupling plus the rotation's own residual (the angle is formed to FP32
-// accuracy, about 6e-8 of kBigRotation), both near the FP64 rounding level,
-// so a further sweep would find nothing to rotate.
+// An FP64 sweep ends the sweeps if all its rotations had a coupling |w_p.w_q| <=
+// kBigRotation |w_p| |w_q|, and either none an angle above kBigAngle or none a
+// coupling above rounding (16 times the threshold of a rotation).  What it leaves
+// is the product of the angles and the couplings, plus the rotations' own residual (the angle
+// is formed to FP32 accuracy, about 6e-8 of the coupling): near the FP64
+// rounding level, so a further sweep would find nothing to rotate.  The angles
+// count on their own: in a cluster of values that are close on the columns'
+// scale -- the small eigenvalues of a density matrix, next to the shift -- they
+// are of order 1 down to rounding, and carry the couplings of other pairs along.
+// With the first condition alone eigenvectors of decaying values (k^-4 to k^-8) had
+// residuals |B v - lambda v| of 1e-9 |B|; with all it takes 3 to 6 more sweeps
+// there and none on values that are apart.
 constexpr double kBigRotation = 1e-8;
-// The FP32 sweeps stop on the same rule at 1e-4: what they leave (1e-8) is
+constexpr double kBigAngle = 1e-6;
+// The FP32 sweeps stop on the coupling alone, at 1e-4: what they leave (1e-8) is
 // below FP32's own rounding of the pair products.
 constexpr float kBigRotation32 = 1e-4f;
 
@@ -254,6 +262,32 @@ struct JacobiArith<double> {
   }
 };
 
+// What a rotation says about convergence (bits; or'ed over a sweep): kRotated, kBig
+// (another sweep has to follow), and in FP64 kAngle, kCoupling (another one if the
+// sweep has seen both).
+constexpr int kRotated = 1, kBig = 2, kAngle = 4, kCoupling = 8;
+template <typename T>
+__device__ __forceinline__ int rotated(T g, T sab, T sn, T tol, T big) {
+  int r = kRotated;
+  if (fabs(g) > big * sab) r |= kBig;
+  if constexpr (sizeof(T) == 8) {
+    if (fabs(sn) > kBigAngle) r |= kAngle;
+    if (fabs(g) > T(16) * tol * sab) r |= kCoupling;
+  }
+  return r;
+}
+// what the CTA's threads have seen
+template <typename T>
+__device__ __forceinline__ int seen_by_all(int seen) {
+  int f = (__syncthreads_or(seen & kRotated) ? kRotated : 0) | (__syncthreads_or(seen & kBig) ? kBig : 0);
+  if constexpr (sizeof(T) == 8)
+    f |= (__syncthreads_or(seen & kAngle) ? kAngle : 0) | (__syncthreads_or(seen & kCoupling) ? kCoupling : 0);
+  return f;
+}
+__device__ __forceinline__ bool sweeps_done(int seen) {
+  return !(seen & kBig) && (seen & (kAngle | kCoupling)) != (kAngle | kCoupling);
+}
+
 // Rotate one column pair (p, q) of W (length R) and V (length C) if needed.
 // NR rows per lane held in registers (R <= 32 NR); V's columns are loaded
 // with W's, so a pair costs one round trip to L2.
@@ -309,7 +343,7 @@ __device__ __forceinline__ int rotate_pair(T* wp, T* wq, T* vp, T* vq, T* na, T*
     __stcg(na, fma(cc, a, fma(ss, bb, -cs2g)));
     __stcg(nb, fma(ss, a, fma(cc, bb, cs2g)));
   }
-  return fabs(g) > big * sab ? 2 : 1;
+  return rotated(g, sab, s, tol, big);
 }
 
 // Any R: the columns streamed twice (products, then the rotation).
@@ -338,7 +372,7 @@ __device__ __noinline__ int rotate_pair_stream(T* wp, T* wq, T* vp, T* vq, int R
     __stcg(vp + i, c * x - s * y);
     __stcg(vq + i, s * x + c * y);
   }
-  return fabs(g) > big * sab ? 2 : 1;
+  return rotated(g, sab, s, tol, big);
 }
 
 // Per-cluster state of the sweeps (shared memory of every CTA; rank 0's
@@ -365,7 +399,7 @@ __device__ int jacobi_sweeps(T* W, T* V, T* nrm2, int R, int C, int max_sweeps, 
   while (!conv && sweeps < max_sweeps) {
     ++sweeps;
     const int gs = ++gsweep;  // sweeps so far over both precisions (same in every thread): picks the flag
-    int did = 0, big = 0;
+    int seen = 0;
     if (nrm2 && nr) {  // the squared column norms, exact at the sweep's start, carried by the rotations
       for (int j = cw; j < C; j += kCW) {
         const T* wj = W + (int64_t)j * R;
@@ -406,17 +440,14 @@ __device__ int jacobi_sweeps(T* W, T* V, T* nrm2, int R, int C, int max_sweeps, 
           case 12: rot = rotate_pair<T, 12>(wp, wq, vp, vq, na, nb, R, C, lane, tol, big_tol); break;
           default: rot = rotate_pair_stream<T>(wp, wq, vp, vq, R, C, lane, tol, big_tol); break;
         }
-        if (rot) {
-          did = 1;
-          big |= rot == 2;
-          ++myrot;
-        }
+        seen |= rot;
+        myrot += rot != 0;
       }
       cluster.sync();  // the next round's pairs read columns this round wrote
     }
     // did any warp of the cluster rotate?  flags alternate between sweeps, so
     // the one read now is never the one being cleared for the next sweep
-    const int f = (__syncthreads_or(did) ? 1 : 0) | (__syncthreads_or(big) ? 2 : 0);
+    const int f = seen_by_all<T>(seen);
     if (f && threadIdx.x == 0) atomicOr(flag0 + (gs & 1), f);
     cluster.sync();
     if (threadIdx.x == 0) {
@@ -424,9 +455,7 @@ __device__ int jacobi_sweeps(T* W, T* V, T* nrm2, int R, int C, int max_sweeps, 
       if (crank == 0) ctl->flag[(gs + 1) & 1] = 0;
     }
     __syncthreads();
-    // converged: nothing rotated by more than big_tol relative -- what
-    // remains is then of order big_tol^2
-    conv = !(ctl->any & 2);
+    conv = sweeps_done(ctl->any);
     __syncthreads();  // any and gsweep are rewritten by the next sweep
   }
   return sweeps;
@@ -437,8 +466,8 @@ __device__ int jacobi_sweeps(T* W, T* V, T* nrm2, int R, int C, int max_sweeps, 
 // from rotation to rotation (recomputed at every sweep's start), so a pair
 // costs one dot product (w_p . w_q), not three; the rotation updates them
 // exactly as it rotates the columns: |w_p'|^2 = c^2 a - 2 c s g + s^2 b,
-// |w_q'|^2 = s^2 a + 2 c s g + c^2 b.  Returns 0 (no rotation), 1, or 2 (a
-// rotation larger than big relative to the pair's norms).
+// |w_q'|^2 = s^2 a + 2 c s g + c^2 b.  Returns 0 (no rotation)
+// or what `rotated` says of it.
 template <typename T, int NR>
 __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* na, T* nb, int R, int C, int lane,
                                                 T tol, T big) {
@@ -475,7 +504,7 @@ __device__ __forceinline__ int rotate_pair_smem(T* wp, T* wq, T* vp, T* vq, T* n
     *na = fma(cc, a, fma(ss, bb, -cs2g));
     *nb = fma(ss, a, fma(cc, bb, cs2g));
   }
-  return fabs(g) > big * sab ? 2 : 1;
+  return rotated(g, sab, sn, tol, big);
 }
 
 // FP64 sweeps by column blocks: the C columns form kColBlocks blocks of bw
@@ -527,7 +556,7 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
   while (!conv && sweeps < max_sweeps) {
     ++sweeps;
     const int gs = ++gsweep;
-    int did = 0, big = 0;
+    int seen = 0;
     for (int j = cw; j < C; j += kCW) {  // the squared column norms, exact at the sweep's start
       const T* wj = W + (int64_t)j * R;
       T a = 0;
@@ -541,11 +570,8 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
     cluster.sync();
     auto rot = [&](T* wp, T* wq, T* vp, T* vq, T* na, T* nb) {
       const int r = rotate_pair_smem<T, NR>(wp, wq, vp, vq, na, nb, R, C, lane, tol, big_tol);
-      if (r) {
-        did = 1;
-        big |= r == 2;
-        ++myrot;
-      }
+      seen |= r;
+      myrot += r != 0;
     };
     for (int r = 0; r < kColBlocks - 1; ++r) {
       const int k = crank;
@@ -594,7 +620,7 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
       copy_out<NT>(nrm2 + q0, Nq, nq);
       cluster.sync();  // the next round reads columns this round wrote, on other CTAs
     }
-    const int f = (__syncthreads_or(did) ? 1 : 0) | (__syncthreads_or(big) ? 2 : 0);
+    const int f = seen_by_all<T>(seen);
     if (f && threadIdx.x == 0) atomicOr(flag0 + (gs & 1), f);
     cluster.sync();
     if (threadIdx.x == 0) {
@@ -602,7 +628,7 @@ __device__ int jacobi_sweeps_blocked(T* W, T* V, T* nrm2, int R, int C, int bw, 
       if (crank == 0) ctl->flag[(gs + 1) & 1] = 0;
     }
     __syncthreads();
-    conv = !(ctl->any & 2);
+    conv = sweeps_done(ctl->any);
     __syncthreads();
   }
   return sweeps;

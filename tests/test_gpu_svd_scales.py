@@ -126,3 +126,34 @@ def test_svd_with_equal_rows(n, e):
     assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
     assert np.max(np.abs(u[:, :2].T @ u[:, :2] - np.eye(2))) <= 1e-12
     assert np.max(np.abs((u * s) @ w - M)[1:, 1:]) <= 1e-14 * e * n
+
+
+def _orth(n, seed):
+    return np.linalg.qr(_mat(n, n, seed))[0]
+
+
+DECAYS = {f"1e-{d}": lambda n, d=d: np.logspace(0, -d, n) for d in (4, 6, 8, 10, 14, 20)}
+DECAYS.update({f"k^-{p}": lambda n, p=p: np.arange(1.0, n + 1.0) ** -p for p in (4, 6, 8)})
+DECAYS["signs"] = lambda n: np.logspace(0, -9, n) * (-1.0) ** np.arange(n)
+DECAYS["gaps of 1e-9"] = lambda n: 1.0 + 1e-9 * np.arange(n)
+DECAYS["gaps of 1e-11"] = lambda n: 1.0 + 1e-11 * np.arange(n)
+
+
+@pytest.mark.parametrize("name", sorted(DECAYS))
+@pytest.mark.parametrize("n", [40, 70, 128])
+def test_close_and_decaying_values(n, name):
+    v = DECAYS[name](n)
+    Q = _orth(n, 7)
+    B = (Q * v) @ Q.T
+    B = 0.5 * (B + B.T)
+    q, lam = _eig(B)
+    assert np.linalg.norm(B @ q - q * lam) <= 1e-12 * np.sqrt(n)
+    assert np.max(np.abs(np.sort(lam) - np.linalg.eigvalsh(B))) <= 1e-12
+    assert np.max(np.abs(q.T @ q - np.eye(n))) <= 1e-12
+    M = (_orth(n, 5) * v) @ _orth(n, 6)
+    u, s, w = _svd(M)
+    assert np.linalg.norm((u * s) @ w - M) <= 1e-12 * np.sqrt(n)
+    assert np.max(np.abs(s - np.linalg.svd(M, compute_uv=False))) <= 1e-12
+    assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
+    live = s > 1e-10 * s[0]
+    assert np.max(np.abs(u[:, live].T @ u[:, live] - np.eye(live.sum()))) <= 1e-12
