@@ -293,7 +293,8 @@ __device__ __forceinline__ void block_tile(const BlkTile& tl, const BlkSeg* sseg
       if (cf) {
         const T c = cf[k];
 #pragma unroll
-        for (int j = 0; j < RN; ++j) bv[j] *= c;
+        for (int j = 0; j < RN; ++j)
+          if (TX * j < nlive) bv[j] *= c;  // as costly as a multiply-add: only what is used
       }
 #pragma unroll
       for (int i = 0; i < RM; ++i)

@@ -64,15 +64,17 @@ bool pack(const Dims& x, int32_t* sizes, uint32_t* mag, int* shf, int32_t* ostr)
 // Modelled cost of a tile in SM clocks at full occupancy (throughput) and
 // alone (latency), from the kernel's own counts: FP32 128 multiply-adds a
 // clock at about half rate for the 8 x 4 microtile and less for the smaller
-// ones, FP64 two a clock over the live part of the tile; a slab's round trip
+// ones, FP64 two operations a clock, multiply-adds and the products with the
+// coefficients alike, over the live part of the tile; a slab's round trip
 // about 700 clocks; 2500 clocks of set-up and stores, shared by the CTAs of an SM.
 // kModelScale: measured over modelled time, 1.5 to 1.6 on the contractions of
-// the U(1) and SU(2) x U(1) MPS step (D = 2048, 1024) and of the MERA patch.
-constexpr double kModelScale = 1.55;
+// the U(1) and SU(2) x U(1) MPS step (D = 2048, 1024) and of the MERA patch;
+// FP64 0.9 to 1.2 (those steps, D = 128 to 1500, and SU(2) recoupling contractions).
+constexpr double kModelScale = 1.55, kModelScale64 = 1.1;
 struct Cost {
   double thr, lat;
 };
-Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k) {
+Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k, bool coef) {
   const int TM = blk_rows(f64, shape), TN = blk_cols(f64, shape);
   const double slabs = std::ceil((double)k / blk_slab(f64, shape));
   if (shape == BLK_DOT) {
@@ -81,11 +83,12 @@ Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k) {
   }
   if (f64) {
     const int64_t gm = shape == BLK_TALL ? 64 : 8, gn = shape == BLK_TALL ? 2 : 16;
-    const double lm = (double)std::min<int64_t>(TM, (m + gm - 1) / gm * gm), ln = (double)std::min<int64_t>(TN, (n + gn - 1) / gn * gn);
-    const double fma = lm * ln * (double)k / 2.0 * 1.1;
+    const double lm = (double)(std::min<int64_t>(TM, m + gm - 1) / gm), ln = (double)(std::min<int64_t>(TN, n + gn - 1) / gn);
+    const double fma = 64.0 * (lm * ln + (coef ? ln : 0.0)) * (double)k * 1.1;  // four warps' operations, 16 clocks each
     return {fma + 500.0, fma + slabs * 700.0 + 2500.0};
   }
-  const double fma = (double)TM * TN * (double)k / 128.0 / (shape == BLK_BIG ? 0.6 : shape == BLK_MID ? 0.5 : shape == BLK_SMALL ? 0.35 : 0.16);
+  const double fma = (coef ? 1.25 : 1.0) * (double)TM * TN * (double)k / 128.0 /
+                     (shape == BLK_BIG ? 0.6 : shape == BLK_MID ? 0.5 : shape == BLK_SMALL ? 0.35 : 0.16);
   return {fma + slabs * 60.0 + 500.0, std::max(fma, slabs * 700.0) + 2500.0};
 }
 
@@ -94,12 +97,14 @@ Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k) {
 // The best rates tile_cost knows: 76.8 multiply-adds a clock of an SM in FP32
 // (BLK_BIG), below 2 in FP64; whole tiles and latencies only add to that.
 double block_floor_us(bool f64, double fma) {
-  return kModelScale * fma / (f64 ? 2.0 : 76.8) / 152.0 / 1900.0;
+  return (f64 ? kModelScale64 : kModelScale) * fma / (f64 ? 2.0 : 76.8) / 152.0 / 1900.0;
 }
 
 double blk_tile_cost(bool f64, const BlkTile& t) {
   const int64_t ks = blk_slab(f64, t.shape);
-  return tile_cost(f64, t.shape, t.ob.m - t.r0, t.ob.n - t.c0, std::min<int64_t>(t.ob.ktot, t.s1 * ks) - t.s0 * ks).lat;
+  return tile_cost(f64, t.shape, t.ob.m - t.r0, t.ob.n - t.c0, std::min<int64_t>(t.ob.ktot, t.s1 * ks) - t.s0 * ks,
+                   (t.ob.flags & kBlkCoef) != 0)
+      .lat;
 }
 
 bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, const Tensor& C,
@@ -154,6 +159,7 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
   const int seg_base = (int)P.bsegs.size(), out_base = (int)P.bouts.size();
   struct Choice {
     int64_t m, n, k;
+    bool coef;
   };
   std::vector<Choice> sizes;
   int64_t so[kMaxDim], sp[kMaxDim], sq[kMaxDim];
@@ -244,7 +250,7 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
       segs.push_back(g);
     }
     outs.push_back(b);
-    sizes.push_back({b.m, b.n, k0});
+    sizes.push_back({b.m, b.n, k0, (b.flags & kBlkCoef) != 0});
   }
   // tile shapes: the cheapest per block, or only the small ones when the
   // launch would otherwise end on a few long tiles
@@ -263,11 +269,11 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
       // interior tiles, the right and bottom edges, the corner
       const int64_t fm = c.m / TM, fn = c.n / TN, em = c.m % TM, en = c.n % TN;
       double t = 0.0;
-      if (fm && fn) t += (double)(fm * fn) * tile_cost(f64, sh, TM, TN, c.k).thr;
-      if (fm && en) t += (double)fm * tile_cost(f64, sh, TM, en, c.k).thr;
-      if (em && fn) t += (double)fn * tile_cost(f64, sh, em, TN, c.k).thr;
-      if (em && en) t += tile_cost(f64, sh, em, en, c.k).thr;
-      if (t < cost) {
+      if (fm && fn) t += (double)(fm * fn) * tile_cost(f64, sh, TM, TN, c.k, c.coef).thr;
+      if (fm && en) t += (double)fm * tile_cost(f64, sh, TM, en, c.k, c.coef).thr;
+      if (em && fn) t += (double)fn * tile_cost(f64, sh, em, TN, c.k, c.coef).thr;
+      if (em && en) t += tile_cost(f64, sh, em, en, c.k, c.coef).thr;
+      if (t < cost || (t == cost && sh <= BLK_SMALL)) {  // equal for a block within one tile in FP64: the fewer loads
         cost = t;
         pick = sh;
       }
@@ -276,25 +282,43 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
   };
   for (int mode = 0; mode < 2; ++mode) {
     double thr = 0.0, lat = 0.0;
+    std::vector<std::pair<double, double>> units;  // (throughput clocks, tiles)
     for (auto& c : sizes) {
       const int sh = shape_of(c, mode);
       const int64_t TM = blk_rows(f64, sh), TN = blk_cols(f64, sh);
       const double full = (double)(c.m / TM) * (double)(c.n / TN);
-      const Cost f = tile_cost(f64, sh, TM, TN, c.k), e = tile_cost(f64, sh, std::min(c.m, TM), std::min(c.n, TN), c.k);
+      const Cost f = tile_cost(f64, sh, TM, TN, c.k, c.coef), e = tile_cost(f64, sh, std::min(c.m, TM), std::min(c.n, TN), c.k, c.coef);
       const double all = (double)((c.m + TM - 1) / TM) * (double)((c.n + TN - 1) / TN);
       thr += f.thr * full + (all - full) * e.thr;
       lat = std::max(lat, (full > 0 ? f : e).lat);
+      if (f64) units.push_back({f.thr, full}), units.push_back({e.thr, all - full});
     }
     const double cut = std::max(thr / nsm, 6000.0);
+    // the clocks of the busiest SM: tiles go out longest first, one to each SM in
+    // turn.  In FP64, where a few hundred tiles fill the pipe, that is up to
+    // twice the average (an SU(2) recoupling contraction with 172 tiles took 240 us)
+    double busy = thr / nsm;
+    if (f64) {
+      for (auto& u : units)
+        if (u.first > 2.0 * cut) u = {cut, u.second * u.first / cut};  // cut along its reduction
+      std::sort(units.begin(), units.end(), [](auto& a, auto& b) { return a.first > b.first; });
+      double next = 0.0, seen = 0.0, first = 0.0;
+      for (auto& u : units)
+        for (seen += u.second; next < seen; next += nsm) first += u.first;
+      busy = std::max(busy, first);
+    }
     lat = std::min(lat, 2.0 * cut) * share;  // longer tiles are cut along their reductions
-    const double us = kModelScale * (std::max(thr / nsm, lat) + 0.3 * std::min(thr / nsm, lat)) / 1900.0 + 3.0 * share;
+    auto model = [&](double t) {
+      return (f64 ? kModelScale64 : kModelScale) * (std::max(t, lat) + 0.3 * std::min(t, lat)) / 1900.0 + 3.0 * share;
+    };
+    const double us = model(thr / nsm);
     if (best_mode < 0 || us < best) {
       best = us;
       best_mode = mode;
       target = cut;
+      *model_us = model(busy);
     }
   }
-  *model_us = best;
   struct Unit {
     double cost;
     BlkTile t;
@@ -315,7 +339,7 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
         t.c0 = q;
         t.shape = sh;
         // a tile much longer than the launch's share of an SM is cut along its reduction
-        const double lat = tile_cost(f64, sh, c.m - r, c.n - q, c.k).lat;
+        const double lat = tile_cost(f64, sh, c.m - r, c.n - q, c.k, c.coef).lat;
         int parts = 1;
         if (lat > 2.0 * target) parts = (int)std::min({std::ceil(lat / target), std::max(1.0, slabs / 4.0), 512.0});
         if (slots + parts > kMaxSlots) parts = 1;
