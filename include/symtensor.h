@@ -174,6 +174,19 @@ int sym_plan_execute(sym_plan plan, const void* in, void* out, void* stream);
  *   side) skip the matrix form: their product is taken directly on A's and
  *   C's blocks with B's sector matrix as coefficients (one streaming pass;
  *   the gradient of B is an atomic reduction into dB).
+ *   A contraction of small and medium sectors runs on the blocks throughout
+ *   instead, one launch forward and one backward with no matrix form: a grouped
+ *   GEMM on the CUDA cores (FP32 with FP32 accumulation, or FP64) that takes each product of
+ *   blocks where it lies, with the recoupling sums multiplied out.  The planner
+ *   takes the form that a model of both finds faster, if every parameter of
+ *   sym_tune that chooses among kernels has the value the library ships (and
+ *   tensors stay below 2^31 elements); any other value of tc_min_mn, tc_min_k,
+ *   tc_max_k, direct_max, direct_mixed or tc_all, from sym_tune_set or the
+ *   environment, selects the matrix form.  Where the blocks win by the launches and the host
+ *   time alone, the plan keeps both forms (with the scratch of both), and calls whose stream is
+ *   being captured run in matrix form: replays pay no host time.  The two
+ *   forms agree to rounding (FP32: split-BF16 on the tensor cores against FP32
+ *   multiply-adds), not to the bit.
  * sym_contract: C = contract(A, B) on device buffers.
  * sym_contract_backward: dA, dB = gradient of <dC, C> with respect to A's
  *   and B's blocks (adjoint on the same sector tables); dA or dB may be NULL
@@ -322,8 +335,9 @@ int sym_su2_gamma(int rank, const int* spins, const int* tree_in, const int* per
                   int* labels_in, int* labels_out);
 
 /* ------------------------------------------ contraction without allocation ---
- * sym_contract_noalloc: C = contract(A, B) exactly as sym_contract_plan +
- *   sym_contract with tree_c = NULL would compute it, for callers that cannot
+ * sym_contract_noalloc: C = contract(A, B) as sym_contract_plan + sym_contract
+ *   with tree_c = NULL compute it in matrix form (a plan that runs on the blocks
+ *   agrees with it to rounding, not to the bit), for callers that cannot
  *   call cudaMalloc (code that must not enter the CUDA allocator, or that runs
  *   next to a framework owning all device memory).  It allocates no device
  *   memory: its work lists and operand scratch live in one file-scope

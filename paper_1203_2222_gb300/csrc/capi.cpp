@@ -379,8 +379,11 @@ int sym_plan_launches(sym_plan plan, int* launches) {
 int sym_plan_profile(sym_plan plan, int enable) {
   return guard([&] {
     need(plan && plan->p, "plan is NULL");
-    if (enable) plan->p->clear_profile();
-    plan->p->profiling = enable != 0;
+    for (sym::Plan* p : {plan->p.get(), plan->p->captured.get()}) {
+      if (!p) continue;
+      if (enable) p->clear_profile();
+      p->profiling = enable != 0;
+    }
     return SYM_OK;
   });
 }
@@ -400,13 +403,20 @@ int sym_plan_profile_read(sym_plan plan, int phase, int* launches, double* total
   return guard([&] {
     need(plan && plan->p, "plan is NULL");
     need(phase >= 0 && phase < sym::PH_COUNT, "bad phase");
-    sym::PhaseProfile& pp = plan->p->prof[phase];
-    double ms = 0.0;
-    for (auto& e : pp.events) ms += launch_ms(e);
-    if (launches) *launches = pp.launches;
+    int n = 0;
+    double ms = 0.0, by = 0.0, fl = 0.0;
+    for (const sym::Plan* p : {plan->p.get(), plan->p->captured.get()}) {  // launches of either form
+      if (!p) continue;
+      const sym::PhaseProfile& pp = p->prof[phase];
+      for (auto& e : pp.events) ms += launch_ms(e);
+      n += pp.launches;
+      by += pp.bytes;
+      fl += pp.flops;
+    }
+    if (launches) *launches = n;
     if (total_ms) *total_ms = ms;
-    if (bytes) *bytes = pp.bytes;
-    if (flops) *flops = pp.flops;
+    if (bytes) *bytes = by;
+    if (flops) *flops = fl;
     return SYM_OK;
   });
 }
@@ -418,14 +428,17 @@ int sym_plan_profile_kernel(sym_plan plan, int kernel, int* launches, double* to
     need(kernel >= 0 && kernel < SYM_KERNEL_COUNT, "bad kernel");
     int n = 0;
     double ms = 0.0, by = 0.0, fl = 0.0;
-    for (const sym::PhaseProfile& pp : plan->p->prof)
-      for (const auto& e : pp.events)
-        if (e.kernel == kernel) {
-          ++n;
-          ms += launch_ms(e);
-          by += e.bytes;
-          fl += e.flops;
-        }
+    for (const sym::Plan* p : {plan->p.get(), plan->p->captured.get()}) {
+      if (!p) continue;
+      for (const sym::PhaseProfile& pp : p->prof)
+        for (const auto& e : pp.events)
+          if (e.kernel == kernel) {
+            ++n;
+            ms += launch_ms(e);
+            by += e.bytes;
+            fl += e.flops;
+          }
+    }
     if (launches) *launches = n;
     if (total_ms) *total_ms = ms;
     if (bytes) *bytes = by;

@@ -1459,6 +1459,7 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
 // form at 3 TB/s, the GEMM kernels, and per phase 40 us for its three to six
 // launches and their side streams (15 us on the device, 25 us more on the host,
 // which is what bounds a chain of small contractions).
+constexpr double kPhaseUs = 40.0;
 double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, double share) {
   const double es = f64 ? 8.0 : 4.0;
   double bytes = 0.0, tc = 0.0, tclat = 0.0, simt = 0.0;
@@ -1475,7 +1476,24 @@ double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, 
       simt += 2.0 * m * n * k;
     }
   }
-  return 40.0 * share + bytes / 3.0e6 + std::max(tc, tclat * share) + simt / (f64 ? 0.4e6 : 10e6);
+  return kPhaseUs * share + bytes / 3.0e6 + std::max(tc, tclat * share) + simt / (f64 ? 0.4e6 : 10e6);
+}
+
+// Whether a contraction that runs on the blocks when it is called keeps its
+// matrix form for calls under stream capture, whose replays pay no host time:
+// modelled device times of forward and both gradients (blk, mat: the two models
+// above over the three phases), in FP32.  In a replay the launches of the
+// matrix form take 25 us for all three phases, and the kernels of thin or short
+// sectors, where those are most of the work, 90 us more; the block kernel 1.3
+// times its model.  Fitted to 70
+// contractions of U(1), fermion-parity, SU(2) x U(1) chains and of rank-4 pairs, forward and
+// gradients replayed (us, blocks / matrix form): L.A of a U(1) chain D = 384 17 / 32, 1024
+// 42 / 41, 1700 81 / 43, 2500 209 / 68; its SU(2) x U(1) MPO step D = 1024 68 /
+// 155.  The blocks have to win by a tenth, about what the two models miss.  In FP64
+// they took 0.11 to 1.0 of the time of the matrix form wherever they are chosen.
+bool matrix_form_captured(bool f64, double blk, double mat, bool thin) {
+  const double m = mat - 3.0 * kPhaseUs + 25.0 + (thin ? 90.0 : 0.0), b = 1.3 * blk - 5.0;
+  return !f64 && b > 0.9 * m;
 }
 
 }  // namespace
@@ -1650,6 +1668,15 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
       // (128 two-site problems: 2.35 ms in matrix form, 2.47 ms at a factor of 1)
       P->blocks = ok;
       if (!P->blocks) drop_blocks(*P);
+      double work = 0.0, thin = 0.0;
+      for (int ph = 0; ph < 3; ++ph)
+        for (auto& g : mnk[ph]) {
+          const double f = (double)g[0] * (double)g[1] * (double)g[2];
+          work += f;
+          if (g[3] >= 3) thin += f;
+        }
+      if (P->blocks && device && nbatch == 1 && matrix_form_captured(f64, blk_us, mat_us, thin > 0.5 * work))
+        P->captured = plan_contract(A, B, pairsA, pairsB, C, precision, device, /*blocks=*/false);
     }
   }
 
@@ -2787,8 +2814,25 @@ int exec_transform(Plan& p, const void* in, void* out, void* stream) {
   return run_box(p, p.xform, ptrs, stream, PH_XFORM);
 }
 
+static bool capturing(void* stream) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &st) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside a capture: this call is not part of it
+    return false;
+  }
+  return st == cudaStreamCaptureStatusActive;
+}
+
 int exec_contract(Plan& p, const void* A, const void* B, void* C, void* stream) {
   if (p.dry) fail(SYM_ERR_UNSUPPORTED, "plan was built with SYM_PLAN_DRYRUN=1 and cannot run");
+  if (p.captured) {
+    if (capturing(stream)) {
+      const int rc = exec_contract(*p.captured, A, B, C, stream);
+      p.last_launches = p.captured->last_launches;
+      return rc;
+    }
+    p.captured->fwd_a = p.captured->fwd_b = nullptr;  // a backward captured after this one gathers its operands itself
+  }
   p.last_launches = 0;
   BoxPtrs d{};
   d.src[0] = A;
@@ -2814,6 +2858,11 @@ int exec_contract(Plan& p, const void* A, const void* B, void* C, void* stream) 
 int exec_contract_backward(Plan& p, const void* A, const void* B, const void* dC, void* dA, void* dB,
                            void* stream) {
   if (p.dry) fail(SYM_ERR_UNSUPPORTED, "plan was built with SYM_PLAN_DRYRUN=1 and cannot run");
+  if (p.captured && capturing(stream)) {
+    const int rc = exec_contract_backward(*p.captured, A, B, dC, dA, dB, stream);
+    p.last_launches = p.captured->last_launches;
+    return rc;
+  }
   p.last_launches = 0;
   if (!dA && !dB) return SYM_OK;
   BoxPtrs d{};

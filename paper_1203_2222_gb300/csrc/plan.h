@@ -78,6 +78,9 @@ struct Plan {
   double blk_bytes[3] = {0.0, 0.0, 0.0};  // algorithmic bytes of a phase (its two operands and its result once)
   double blk_flops[3] = {0.0, 0.0, 0.0};  // useful flops of a phase
   std::vector<std::array<int, 3>> blk_mnk;  // the phases' sectors (statistics)
+  // the same contraction in matrix form, for calls whose stream is being
+  // captured: set where the blocks win by the launches alone (see plan_contract)
+  std::unique_ptr<Plan> captured;
 
   // GEMM work lists.  Kinds: 0 = tcgen05 split-BF16 x3, 1 = CUDA-core 64x64,
   // 2 = CUDA-core 256x16, 3 = CUDA-core thin (m, n <= 8), 4 = CUDA-core
