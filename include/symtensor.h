@@ -238,6 +238,16 @@ int sym_plan_destroy(sym_plan plan);
  * (m, n, k, kernel) with kernel 0 = tcgen05 split-BF16, 1 = CUDA cores. */
 int sym_plan_gemm_shapes(sym_plan plan, int* nsec, int* mnk);
 
+/* How a contraction that runs on the blocks is cut up (all 0 for one in matrix
+ * form; any pointer may be NULL): tiles of each of the kernel's
+ * SYM_BLOCK_SHAPES shapes over the three phases (large, medium, small, tall,
+ * dot), output tiles whose reduction is cut into parts, the most pairs of
+ * blocks that one tile sums, and the bytes in which the parts are added up (at
+ * most 64 MiB, of all problems of a batch together).                       */
+#define SYM_BLOCK_SHAPES 5
+int sym_plan_block_info(sym_plan plan, int* tiles, int* cut, int* segments,
+                        int64_t* workspace);
+
 /* Per-phase device timing of a plan's own launches.  sym_plan_profile(p, 1)
  * clears and starts recording a CUDA event pair around every launch (on the
  * launch stream); 0 stops.  sym_plan_profile_read synchronizes on the

@@ -90,6 +90,7 @@ _SIGS = {
     "sym_plan_profile_kernel": ([_P, _I, _IP, _DP, _DP, _DP], _I),
     "sym_plan_destroy": ([_P], _I),
     "sym_plan_gemm_shapes": ([_P, _IP, _IP], _I),
+    "sym_plan_block_info": ([_P, _IP, _IP, _IP, _LP], _I),
     "sym_device_status": ([], _I),
     "sym_wait_probe": ([_I, _I], _I),
     "sym_su2_F": ([_I, _I, _I, _I, _I, _I, _DP], _I),

@@ -171,7 +171,7 @@ __device__ __forceinline__ bool join_parts(const BlkTile& tl, T (&v)[N], T* __re
                                            int* flag) {
   const int part = tl.part & 0xffff, nparts = tl.part >> 16;
   if (nparts <= 1) return true;
-  T* slot = ws + (int64_t)(tl.ws + part) * kBlkSlot + threadIdx.x;
+  T* slot = ws + (int64_t)(tl.ws + part * N) * kThreads + threadIdx.x;
 #pragma unroll
   for (int i = 0; i < N; ++i) __stcg(slot + i * kThreads, v[i]);
   __threadfence();
@@ -183,7 +183,7 @@ __device__ __forceinline__ bool join_parts(const BlkTile& tl, T (&v)[N], T* __re
 #pragma unroll
   for (int i = 0; i < N; ++i) v[i] = T(0);
   for (int q = 0; q < nparts; ++q) {
-    const T* s = ws + (int64_t)(tl.ws + q) * kBlkSlot + threadIdx.x;
+    const T* s = ws + (int64_t)(tl.ws + q * N) * kThreads + threadIdx.x;
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] += __ldcg(s + i * kThreads);
   }
@@ -196,7 +196,6 @@ __device__ __forceinline__ void block_tile(const BlkTile& tl, const BlkSeg* sseg
                                            const BoxPtrs& ptrs, void* smem, T* __restrict__ ws,
                                            int* __restrict__ counters, int* flag) {
   static_assert((TM / RM) * (TN / RN) == kThreads, "one microtile per thread");
-  static_assert(TM * TN <= kBlkSlot, "a part's tile fits its workspace slot");
   Smem<T, TM, TN, KS>& sm = *static_cast<Smem<T, TM, TN, KS>*>(smem);
   constexpr int TX = TN / RN, TY = TM / RM;
   constexpr bool kVec = sizeof(T) == 4;  // consecutive rows and columns per thread (else strided)

@@ -12,8 +12,6 @@ namespace sym {
 
 namespace {
 
-constexpr int kMaxSlots = 4096;  // workspace slots of the cut tiles of one phase (64 MB in FP64)
-
 void strides_of(const Tensor& T, int64_t s, int64_t* st) {
   int64_t acc = 1;
   for (int l = T.rank - 1; l >= 0; --l) {
@@ -293,6 +291,9 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
       lat = std::max(lat, (full > 0 ? f : e).lat);
       if (f64) units.push_back({f.thr, full}), units.push_back({e.thr, all - full});
     }
+    // an SM's share of this phase; in a batch too, where the largest problem's tiles
+    // end the launch (eight two-site problems of 256 <= D <= 1024: 721 us, 747 with the
+    // share of eight such problems)
     const double cut = std::max(thr / nsm, 6000.0);
     // the clocks of the busiest SM: tiles go out longest first, one to each SM in
     // turn.  In FP64, where a few hundred tiles fill the pipe, that is up to
@@ -325,7 +326,12 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
     int out;
   };
   std::vector<Unit> tiles;
-  int slots = 0, counters = 0;
+  // dA's and dB's parts lie side by side (one launch), the forward's in the same place
+  const int64_t first_unit = phase == 2 ? P.blk_end : 0;
+  const int64_t unit_bytes = kBlkThreads * (f64 ? 8 : 4);
+  const int64_t max_units = (int64_t)((double)(kBlkWorkspace / 2) * share) / unit_bytes;
+  int64_t units = 0;
+  int counters = 0;
   for (size_t i = 0; i < sizes.size(); ++i) {
     const Choice& c = sizes[i];
     const int sh = shape_of(c, best_mode);
@@ -342,14 +348,14 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
         const double lat = tile_cost(f64, sh, c.m - r, c.n - q, c.k, c.coef).lat;
         int parts = 1;
         if (lat > 2.0 * target) parts = (int)std::min({std::ceil(lat / target), std::max(1.0, slabs / 4.0), 512.0});
-        if (slots + parts > kMaxSlots) parts = 1;
+        if (units + (int64_t)parts * blk_values(f64, sh) > max_units) parts = 1;
         const int per = parts > 1 ? (slabs + parts - 1) / parts : slabs;
         parts = per > 0 ? (slabs + per - 1) / per : 1;
         for (int p = 0; p < parts; ++p) {
           t.s0 = p * per;
           t.s1 = std::min(slabs, (p + 1) * per);
           t.part = p | (parts << 16);
-          t.ws = P.blk_slots + slots;
+          t.ws = (int)(first_unit + units);
           t.cnt = P.blk_counters + counters;
           // the segments that meet [s0, s1)
           const BlkSeg* sg = segs.data() + (outs[i].seg0 - seg_base);
@@ -361,7 +367,7 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
           tiles.push_back({blk_tile_cost(f64, t), t, out_base + (int)i});
         }
         if (parts > 1) {
-          slots += parts;
+          units += (int64_t)parts * blk_values(f64, sh);
           ++counters;
         }
       }
@@ -376,7 +382,8 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
     P.btiles.push_back(t.t);
     P.btile_out.push_back(t.out);
   }
-  P.blk_slots += slots;
+  P.blk_end = first_unit + units;
+  P.blk_units = std::max(P.blk_units, P.blk_end);
   P.blk_counters += counters;
   P.blk_bytes[phase] = (f64 ? 8.0 : 4.0) * ((double)A.numel() + (double)B.numel() + (double)C.numel());
   return true;
@@ -388,7 +395,8 @@ void drop_blocks(Plan& P) {
   P.btiles.clear();
   P.btile_out.clear();
   P.blk_mnk.clear();
-  P.blk_slots = P.blk_counters = 0;
+  P.blk_units = P.blk_end = 0;
+  P.blk_counters = 0;
   P.blocks = false;
   for (int ph = 0; ph < 3; ++ph) {
     P.blk_range[ph] = Range{};
@@ -476,7 +484,8 @@ void validate_blocks(const Plan& P) {
       bad("tile range");
     if (t.shape == BLK_DOT && (b.m > 8 || b.n > 8)) bad("output too wide for a dot");
     if (nparts == 1 ? (t.s0 != 0 || t.s1 != slabs)
-                    : (t.ws < 0 || t.ws + nparts > P.blk_slots || t.cnt < 0 || t.cnt >= P.blk_counters))
+                    : (t.ws < 0 || t.ws + (int64_t)nparts * blk_values(P.f64(), t.shape) > P.blk_units || t.cnt < 0 ||
+                       t.cnt >= P.blk_counters))
       bad("tile parts");
   }
 }

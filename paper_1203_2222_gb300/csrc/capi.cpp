@@ -471,6 +471,24 @@ int sym_tune_epoch(int* epoch) {
   });
 }
 
+int sym_plan_block_info(sym_plan plan, int* tiles, int* cut, int* segments, int64_t* workspace) {
+  return guard([&] {
+    need(plan && plan->p, "plan is NULL");
+    const sym::Plan& p = *plan->p;
+    int shapes[sym::BLK_SHAPES] = {}, ncut = 0, nseg = 0;
+    for (const sym::BlkTile& t : p.btiles) {
+      ++shapes[t.shape];
+      ncut += (t.part >> 16) > 1 && (t.part & 0xffff) == 0;
+      nseg = std::max(nseg, t.ob.nseg);
+    }
+    if (tiles) std::copy(shapes, shapes + sym::BLK_SHAPES, tiles);
+    if (cut) *cut = ncut;
+    if (segments) *segments = nseg;
+    if (workspace) *workspace = p.blk_units * sym::kBlkThreads * (p.f64() ? 8 : 4);
+    return SYM_OK;
+  });
+}
+
 int sym_plan_gemm_shapes(sym_plan plan, int* nsec, int* mnk) {
   return guard([&] {
     need(plan && plan->p && nsec, "NULL argument");

@@ -225,11 +225,14 @@ SYM_HD constexpr int blk_cols(bool f64, int shape) {
 SYM_HD constexpr int blk_slab(bool f64, int shape) {
   return shape <= BLK_MID ? 16 : shape == BLK_SMALL ? (f64 ? 16 : 32) : shape == BLK_TALL ? 8 : kBlkThreads;
 }
+// Elements a thread keeps of a tile (BLK_DOT: threads 0 .. 63 one each).
+SYM_HD constexpr int blk_values(bool f64, int shape) {
+  return shape == BLK_DOT ? 1 : blk_rows(f64, shape) * blk_cols(f64, shape) / kBlkThreads;
+}
 // One unit of work: a tile of an output block, over slabs [s0, s1) of its
-// reduction.  A tile cut into nparts > 1 parts adds them up in workspace slots
-// ws .. ws + nparts - 1 (kBlkSlot elements each): the part that arrives last
+// reduction.  A tile cut into nparts > 1 parts adds them up in the workspace,
+// part p at ws + p blk_values (in units of kBlkThreads elements): the part that arrives last
 // (counter cnt) sums them in order, writes the tile and clears the counter.
-constexpr int kBlkSlot = 4096;
 struct BlkTile {
   BlkOut ob;      // with the segments of [s0, s1) only
   int32_t r0, c0;

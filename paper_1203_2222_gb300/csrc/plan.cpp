@@ -802,8 +802,8 @@ void Plan::upload(bool device) {
   d_btiles = static_cast<BlkTile*>(up(btiles.data(), btiles.size() * sizeof(BlkTile)));
   if (kind == CONTRACT) {
     const size_t es = f64() ? sizeof(double) : sizeof(float);
-    if (blk_slots > 0) {
-      blk_ws = arena.alloc((size_t)blk_slots * kBlkSlot * es, false);
+    if (blk_units > 0) {
+      blk_ws = arena.alloc((size_t)blk_units * kBlkThreads * es, false);
       d_blk_cnt = static_cast<int*>(arena.alloc((size_t)blk_counters * sizeof(int), true));
     }
     if (img_elems > 0) {  // hi and lo planes; the TMA loads fill past-the-edge boxes with zeros
@@ -1379,7 +1379,7 @@ bool default_kernel_choice(const sym_tune& t) {
 // Every product of blocks a contraction sums, with its coefficient (swap
 // signs; SU(2): the recoupling sums on both operands and on the result
 // multiplied out).  False when there are too many for the work lists, or when
-// multiplying the recoupling sums out more than doubles the arithmetic.
+// multiplying the recoupling sums out takes more than four times the arithmetic.
 constexpr int64_t kMaxTriples = 200000;
 bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const MatForm& MA, const MatForm& MB, int na,
                    int nc, const std::vector<TermList>& XA, const std::vector<TermList>& XB,
@@ -2519,11 +2519,11 @@ std::unique_ptr<Plan> merge_contract_plans(std::vector<std::unique_ptr<Plan>>& p
       }
       M->blk_mnk.insert(M->blk_mnk.end(), p.blk_mnk.begin(), p.blk_mnk.end());
     }
-    std::vector<int> slot0(n), cnt0(n);
+    std::vector<int> unit0(n), cnt0(n);
     for (int i = 0; i < n; ++i) {
-      slot0[i] = M->blk_slots;
+      unit0[i] = (int)M->blk_units;
       cnt0[i] = M->blk_counters;
-      M->blk_slots += ps[i]->blk_slots;
+      M->blk_units += ps[i]->blk_units;
       M->blk_counters += ps[i]->blk_counters;
     }
     for (int ph = 0; ph < 3; ++ph) {
@@ -2544,7 +2544,7 @@ std::unique_ptr<Plan> merge_contract_plans(std::vector<std::unique_ptr<Plan>>& p
           b.ob = M->bouts[out];
           b.ob.seg0 = own.seg0 + seg0[i];
           b.ob.nseg = own.nseg;
-          b.ws += slot0[i];
+          b.ws += unit0[i];
           b.cnt += cnt0[i];
           v.push_back({blk_tile_cost(f64, b), b, out});
         }

@@ -73,7 +73,10 @@ struct Plan {
   std::vector<BlkSeg> bsegs;
   std::vector<BlkTile> btiles;
   std::vector<int> btile_out;  // output block of every tile (host checks)
-  int blk_slots = 0, blk_counters = 0;  // workspace of the cut tiles
+  // workspace of the cut tiles: units of kBlkThreads elements, shared by the forward and the
+  // backward launch (which do not overlap), and counters (of their own)
+  int64_t blk_units = 0, blk_end = 0;  // blk_end: of the phases planned so far in the current launch
+  int blk_counters = 0;
   Range blk_range[3];
   double blk_bytes[3] = {0.0, 0.0, 0.0};  // algorithmic bytes of a phase (its two operands and its result once)
   double blk_flops[3] = {0.0, 0.0, 0.0};  // useful flops of a phase
@@ -190,6 +193,7 @@ struct BlkTriple {
 // takes or an offset leaves 32 bits.  free / pairs: leg numbers as in
 // plan_contract; share: the part of a launch's fixed costs and latency this
 // plan bears (1, or 1/n in a batch of n).  *model_us: the phase's modelled time.
+constexpr int64_t kBlkWorkspace = 64 << 20;  // bytes of a plan's cut tiles at most, of all problems of a batch plan together
 bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, const Tensor& C,
                       const std::vector<BlkTriple>& triples, const std::vector<int>& freeA,
                       const std::vector<int>& freeB, const std::vector<int>& pairsA, const std::vector<int>& pairsB,

@@ -127,6 +127,13 @@ class Plan:
         L.check(L.lib.sym_plan_gemm_shapes(self._h, _byref(n), buf))
         return [tuple(buf[4 * i:4 * i + 4]) for i in range(n.value)]
 
+    def block_info(self):
+        """How a contraction on the blocks is cut up (include/symtensor.h, sym_plan_block_info)."""
+        tiles, cut, seg, ws = (ctypes.c_int * 5)(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int64()
+        L.check(L.lib.sym_plan_block_info(self._h, tiles, _byref(cut), _byref(seg), _byref(ws)))
+        return {"tiles": dict(zip(("large", "medium", "small", "tall", "dot"), tiles)), "cut": cut.value,
+                "segments": seg.value, "workspace": ws.value}
+
     def profile(self, enable=True):
         """Start (clear) or stop recording device time of this plan's launches."""
         L.check(L.lib.sym_plan_profile(self._h, 1 if enable else 0))
