@@ -685,39 +685,46 @@ void Plan::encode_maps(const void* img_base) {
 // fuse and split of 470 MB 246 -> 237 us.  Only launches of flat items: with
 // recoupling sums (SU(2), FP64: 237 -> 263 us) the order of the sectors is the
 // better one, where items that share their sources are neighbours.  And only
-// stretches of at most kMaxSorted items: beyond 200 items a warp the shares are
+// stretches of at most kMaxSorted items: beyond 30 items a warp the shares are
 // even anyway (the full-size SU(2) recoupling contraction with gradients, 21.5
 // million items: 90.0 ms in the order of the sectors, 90.6 sorted), and sorting
-// them took 2.0 of 9.8 s of planning.
-constexpr int kMaxSorted = 1 << 20;
+// them would take a good part of the planning.
+constexpr int kMaxSorted = 1 << 18;
 void Plan::sort_items() {
   std::vector<int> cut = {0, (int)items.size()};  // items between two cuts are in the same launches
   for (const Range* r : {&xform, &fwd_gather, &fwd_scatter, &bwd_gather_a, &bwd_gather_b, &bwd_scatter_a, &bwd_scatter_b})
     if (r->count > 0) cut.insert(cut.end(), {r->first, r->first + r->count});
   std::sort(cut.begin(), cut.end());
-  std::vector<std::pair<int, int>> ord;  // (class, item) of one stretch
-  std::vector<BoxItem> sorted;
-  std::vector<double> bytes;
+  std::vector<uint8_t> cls;  // size class of every item of a stretch, and
+  std::vector<int> to;       // where the item goes
   for (size_t k = 0; k + 1 < cut.size(); ++k) {
-    const int i0 = cut[k], i1 = cut[k + 1];
-    if (i1 - i0 > kMaxSorted) continue;
-    if (!std::all_of(items.begin() + i0, items.begin() + i1, [](const BoxItem& i) { return i.sel & kSelFlat; })) continue;
-    ord.clear();
-    ord.reserve(i1 - i0);
-    for (int i = i0; i < i1; ++i) ord.push_back({std::ilogb((double)items[i].count * std::max(1, items[i].nterm)), i});
-    auto larger = [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first > y.first; };
-    if (std::is_sorted(ord.begin(), ord.end(), larger)) continue;
-    std::stable_sort(ord.begin(), ord.end(), larger);
-    sorted.clear();
-    bytes.clear();
-    sorted.reserve(ord.size());
-    bytes.reserve(ord.size());
-    for (auto& o : ord) {
-      sorted.push_back(items[o.second]);
-      bytes.push_back(item_bytes_prefix[o.second + 1]);
+    const int i0 = cut[k], n = cut[k + 1] - i0;
+    if (n > kMaxSorted) continue;
+    if (!std::all_of(items.begin() + i0, items.begin() + i0 + n, [](const BoxItem& i) { return i.sel & kSelFlat; })) continue;
+    int at[65] = {};
+    bool sorted = true;
+    cls.resize(n);
+    for (int i = 0; i < n; ++i) {
+      uint64_t size = (uint64_t)items[i0 + i].count * std::max(1, items[i0 + i].nterm);
+      int c = 0;
+      while (size >>= 1) ++c;
+      cls[i] = (uint8_t)(63 - c);  // largest first
+      sorted = sorted && (i == 0 || cls[i - 1] <= cls[i]);
+      ++at[cls[i] + 1];
     }
-    std::copy(sorted.begin(), sorted.end(), items.begin() + i0);
-    std::copy(bytes.begin(), bytes.end(), item_bytes_prefix.begin() + i0 + 1);
+    if (sorted) continue;
+    for (int c = 0; c < 64; ++c) at[c + 1] += at[c];
+    to.resize(n);
+    for (int i = 0; i < n; ++i) to[i] = at[cls[i]]++;
+    // cycle by cycle in place: a copy of the items would be most of the time
+    double* const bytes = item_bytes_prefix.data() + i0 + 1;
+    for (int i = 0; i < n; ++i)
+      while (to[i] != i) {
+        const int j = to[i];
+        std::swap(items[i0 + i], items[i0 + j]);
+        std::swap(bytes[i], bytes[j]);
+        std::swap(to[i], to[j]);
+      }
   }
 }
 
@@ -1631,19 +1638,23 @@ std::unique_ptr<Plan> plan_contract(const Tensor& A, const Tensor& B, const std:
                             return g.k <= tp.direct_max && g.n <= tp.direct_max;
                           });
   if (blocks && !all_direct && default_kernel_choice(tp)) {
+    // all three phases or none: the matrix form shares its gathers between them
+    const double share = 1.0 / std::max(nbatch, 1), win = nbatch > 1 ? 0.5 : 1.0;
+    std::vector<std::array<int64_t, 4>> mnk[3];  // the phases' GEMMs in matrix form, with their kernel kinds
+    double blk_us = 0.0, mat_us = 0.0, fma = 0.0;
+    for (int ph = 0; ph < 3; ++ph) {
+      for (auto& g : gs)
+        mnk[ph].push_back(ph == 0 ? std::array<int64_t, 4>{g.m, g.n, g.k, g.kind[0]}
+                                  : ph == 1 ? std::array<int64_t, 4>{g.m, g.k, g.n, g.kind[1]}
+                                            : std::array<int64_t, 4>{g.k, g.n, g.m, g.kind[2]});
+      mat_us += matrix_form_us(f64, mnk[ph], share);
+    }
     std::vector<BlkTriple> triples;
-    if (block_triples(Am, Bm, Cn, MA, MB, na, nc, XA, XB, XCt, natural, &triples)) {
-      // all three phases or none: the matrix form shares its gathers between them
-      const double share = 1.0 / std::max(nbatch, 1), win = nbatch > 1 ? 0.5 : 1.0;
-      std::vector<std::array<int64_t, 4>> mnk[3];  // the phases' GEMMs in matrix form, with their kernel kinds
-      double blk_us = 0.0, mat_us = 0.0, fma = 0.0;
-      for (int ph = 0; ph < 3; ++ph) {
-        for (auto& g : gs)
-          mnk[ph].push_back(ph == 0 ? std::array<int64_t, 4>{g.m, g.n, g.k, g.kind[0]}
-                                    : ph == 1 ? std::array<int64_t, 4>{g.m, g.k, g.n, g.kind[1]}
-                                              : std::array<int64_t, 4>{g.k, g.n, g.m, g.kind[2]});
-        mat_us += matrix_form_us(f64, mnk[ph], share);
-      }
+    // the blocks take at least the matrix form's multiply-adds: the products are
+    // only listed where those alone do not decide it (58 of 266 ms of planning an
+    // SU(2) contraction of dmax = 16)
+    if (3.0 * block_floor_us(f64, 0.5 * P->flops_fwd) < mat_us * win &&
+        block_triples(Am, Bm, Cn, MA, MB, na, nc, XA, XB, XCt, natural, &triples)) {
       for (auto& t : triples) {
         double f = 1.0;
         for (int l = 0; l < A.rank; ++l) f *= A.dim(t.a, l);
