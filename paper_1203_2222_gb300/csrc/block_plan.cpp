@@ -85,7 +85,7 @@ Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k, bool coef) 
     const double fma = 64.0 * (lm * ln + (coef ? ln : 0.0)) * (double)k * 1.1;  // four warps' operations, 16 clocks each
     return {fma + 500.0, fma + slabs * 700.0 + 2500.0};
   }
-  const double fma = (coef ? 1.25 : 1.0) * (double)TM * TN * (double)k / 128.0 /
+  const double fma = (coef && shape != BLK_TALL ? 1.25 : 1.0) * (double)TM * TN * (double)k / 128.0 /
                      (shape == BLK_BIG ? 0.6 : shape == BLK_MID ? 0.5 : shape == BLK_SMALL ? 0.35 : 0.16);
   return {fma + slabs * 60.0 + 500.0, std::max(fma, slabs * 700.0) + 2500.0};
 }
@@ -279,7 +279,7 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
     return pick;
   };
   for (int mode = 0; mode < 2; ++mode) {
-    double thr = 0.0, lat = 0.0;
+    double thr = 0.0, lat = 0.0, count = 0.0;
     std::vector<std::pair<double, double>> units;  // (throughput clocks, tiles)
     for (auto& c : sizes) {
       const int sh = shape_of(c, mode);
@@ -289,24 +289,28 @@ bool plan_block_phase(Plan& P, int phase, const Tensor& A, const Tensor& B, cons
       const double all = (double)((c.m + TM - 1) / TM) * (double)((c.n + TN - 1) / TN);
       thr += f.thr * full + (all - full) * e.thr;
       lat = std::max(lat, (full > 0 ? f : e).lat);
-      if (f64) units.push_back({f.thr, full}), units.push_back({e.thr, all - full});
+      units.push_back({f.thr, full});
+      units.push_back({e.thr, all - full});
+      count += all;
     }
     // an SM's share of this phase; in a batch too, where the largest problem's tiles
     // end the launch (eight two-site problems of 256 <= D <= 1024: 721 us, 747 with the
     // share of eight such problems)
     const double cut = std::max(thr / nsm, 6000.0);
     // the clocks of the busiest SM: tiles go out longest first, one to each SM in
-    // turn.  In FP64, where a few hundred tiles fill the pipe, that is up to
-    // twice the average (an SU(2) recoupling contraction with 172 tiles took 240 us)
+    // turn.  With few tiles -- in FP64, where a few hundred fill the pipe, with
+    // more -- that is up to twice the average (an SU(2) recoupling contraction
+    // with 172 tiles took 240 us; three sectors of 512 x 512 x 512 in FP32, 192
+    // tiles, 65 us a phase where the tensor cores take 25)
     double busy = thr / nsm;
-    if (f64) {
+    if (share == 1.0 && (f64 || count < 2.0 * nsm)) {
       for (auto& u : units)
         if (u.first > 2.0 * cut) u = {cut, u.second * u.first / cut};  // cut along its reduction
       std::sort(units.begin(), units.end(), [](auto& a, auto& b) { return a.first > b.first; });
       double next = 0.0, seen = 0.0, first = 0.0;
       for (auto& u : units)
         for (seen += u.second; next < seen; next += nsm) first += u.first;
-      busy = std::max(busy, first);
+      if (f64 || first > 24000.0) busy = std::max(busy, first);  // shorter tiles in FP32: the latency covers it
     }
     lat = std::min(lat, 2.0 * cut) * share;  // longer tiles are cut along their reductions
     auto model = [&](double t) {

@@ -1463,13 +1463,17 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
 }
 
 // Modelled time of one phase in matrix form: the moves in and out of matrix
-// form at 3 TB/s, the GEMM kernels, and per phase 40 us for its three to six
-// launches and their side streams (15 us on the device, 25 us more on the host,
-// which is what bounds a chain of small contractions).
-constexpr double kPhaseUs = 40.0;
+// form at 3 TB/s, the GEMM kernels, and per phase 30 us for its three to six
+// launches and their side streams (15 us on the device, 15 us more on the host
+// than one launch of the block kernel, which is what bounds a chain of small
+// contractions).  FP64: whole tiles of 64 x 64 (256 x 16) at two multiply-adds a clock
+// of an SM, 90% of them, or the longest tile, its reduction cut in two, if there are
+// too few to fill the chip (three sectors of 512 x 512 x 512: 818 us measured, 775
+// modelled, on the blocks 1196).
+constexpr double kPhaseUs = 30.0;
 double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, double share) {
   const double es = f64 ? 8.0 : 4.0;
-  double bytes = 0.0, tc = 0.0, tclat = 0.0, simt = 0.0;
+  double bytes = 0.0, tc = 0.0, tclat = 0.0, simt = 0.0, tiles = 0.0, longest = 0.0;
   for (auto& s : mnk) {
     const double m = (double)s[0], n = (double)s[1], k = (double)s[2];
     bytes += 2.0 * es * (m * k + k * n + m * n);
@@ -1479,11 +1483,21 @@ double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, 
       tclat = std::max(tclat, t);
     } else if (s[3] >= 3) {
       bytes += es * (m * k + k * n + m * n);
+    } else if (f64) {
+      const double out = s[3] == 1 ? std::ceil(m / 64.0) * std::ceil(n / 64.0) : std::ceil(m / 256.0) * std::ceil(n / 16.0);
+      tiles += out;
+      simt += out * 2048.0 * k;  // clocks of an SM: 4096 multiply-adds a tile and step of the reduction
+      longest = std::max(longest, k);
     } else {
       simt += 2.0 * m * n * k;
     }
   }
-  return kPhaseUs * share + bytes / 3.0e6 + std::max(tc, tclat * share) + simt / (f64 ? 0.4e6 : 10e6);
+  double cuda = simt / 10e6;
+  if (f64) {
+    const double split = std::max(1.0, std::min(304.0 / std::max(tiles, 1.0), 2.0));  // deeper cuts gain little more
+    cuda = std::max(simt / 152.0 / 0.9, 2048.0 * longest / split * share) / 1900.0;
+  }
+  return kPhaseUs * share + bytes / 3.0e6 + std::max(tc, tclat * share) + cuda;
 }
 
 // Whether a contraction that runs on the blocks when it is called keeps its

@@ -1,0 +1,44 @@
+"""Which form the planner takes for contractions whose times differ clearly
+(planner on the host; times in us on one GB300, forward and both gradients,
+on the blocks / in matrix form)."""
+import json
+import os
+import subprocess
+import sys
+
+from tests.conftest import ROOT
+
+SCRIPT = r'''
+import json
+import paper_1203_2222_gb300 as P
+from paper_1203_2222_gb300 import synthetic
+
+def on_blocks(g, la, lb, pa, pb, prec):
+    p = P.contract_plan(P.Structure(g, la), P.Structure(g, lb), pa, pb, prec)
+    return sum(p.block_info()["tiles"].values()) > 0
+
+def product(d, prec):
+    legs = [([0, 2, 4], [d] * 3, 1), ([0, 2, 4], [d] * 3, -1)]
+    return on_blocks(P.SU2, legs, legs, [1], [0], prec)
+
+def recouple(d, j):
+    r = synthetic.su2_recouple(dmax=d, jmax2=j)
+    return on_blocks(P.SU2, r["A"], r["B"], r["pairsA"], r["pairsB"], P.FP64)
+
+print(json.dumps({"f64": {d: product(d, P.FP64) for d in (128, 512, 1024)},
+                  "f32": {d: product(d, P.BF16X3) for d in (128, 512, 1024)},
+                  "recouple": {f"{d} {j}": recouple(d, j) for d, j in ((2, 4), (3, 3), (2, 7), (4, 6), (6, 6))}}))
+'''
+
+
+def test_form_of_clear_cases():
+    env = dict(os.environ, SYM_PLAN_DRYRUN="1", PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", SCRIPT], env=env, capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 0, r.stderr
+    d = json.loads(r.stdout)
+    # three sectors of d x d x d: FP64 193 / 318, 3000 / 2266, 19390 / 16460; FP32 (forward alone)
+    # 27 / 31, 65 / 32 and the tensor cores far ahead
+    assert d["f64"] == {"128": True, "512": False, "1024": False}
+    assert d["f32"] == {"128": True, "512": False, "1024": False}
+    # SU(2) recoupling: 190 / 235, 173 / 225; 412, 600 and 1000 in matrix form
+    assert d["recouple"] == {"2 4": True, "3 3": True, "2 7": False, "4 6": False, "6 6": False}

@@ -29,7 +29,7 @@ def _rel(x, ref):
 
 
 # few sectors large enough for the tensor cores: the blocks win by the launches alone
-@pytest.mark.parametrize("D,qmax", [(600, 3), (1000, 5)])
+@pytest.mark.parametrize("D,qmax", [(400, 3), (600, 3)])
 def test_captured_and_plain_calls_mixed(D, qmax):
     w, SL, SA, plan = _chain(D, qmax)
     oL, oA = (([ou1.Leg(*l) for l in w[n]], 0, synthetic.normal(i, S.numel))
@@ -78,7 +78,7 @@ def test_captured_and_plain_calls_mixed(D, qmax):
 
 
 def test_the_captured_form_is_the_matrix_form():
-    _, SL, SA, plan = _chain(1000, 5)
+    _, SL, SA, plan = _chain(600, 3)
     a, b = torch.randn(SL.numel, device="cuda"), torch.randn(SA.numel, device="cuda")
     replay(lambda: P.contract(P.SymTensor(SL, a), P.SymTensor(SA, b), [2], [0]).data)  # warm
     plan.profile(True)
