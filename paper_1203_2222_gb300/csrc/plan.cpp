@@ -1463,14 +1463,15 @@ bool block_triples(const Tensor& Am, const Tensor& Bm, const Tensor& Cn, const M
 }
 
 // Modelled time of one phase in matrix form: the moves in and out of matrix
-// form at 3 TB/s, the GEMM kernels, and per phase 30 us for its three to six
-// launches and their side streams (15 us on the device, 15 us more on the host
-// than one launch of the block kernel, which is what bounds a chain of small
-// contractions).  FP64: whole tiles of 64 x 64 (256 x 16) at two multiply-adds a clock
+// form at 3 TB/s, the GEMM kernels, and per phase 40 us for its three to six
+// launches and their side streams (15 us on the device, 25 us more on the host,
+// which is what bounds a chain of small contractions; 30 us sent FP32
+// contractions to the matrix form that took 161 us on the blocks and 222 in matrix
+// form, a MERA pass 1598 and 1842).  FP64: whole tiles of 64 x 64 (256 x 16) at two multiply-adds a clock
 // of an SM, 90% of them, or the longest tile, its reduction cut in two, if there are
 // too few to fill the chip (three sectors of 512 x 512 x 512: 818 us measured, 775
 // modelled, on the blocks 1196).
-constexpr double kPhaseUs = 30.0;
+constexpr double kPhaseUs = 40.0;
 double matrix_form_us(bool f64, const std::vector<std::array<int64_t, 4>>& mnk, double share) {
   const double es = f64 ? 8.0 : 4.0;
   double bytes = 0.0, tc = 0.0, tclat = 0.0, simt = 0.0, tiles = 0.0, longest = 0.0;
