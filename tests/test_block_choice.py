@@ -45,3 +45,26 @@ def test_form_of_clear_cases():
     assert d["recouple"] == {"2 4": True, "3 3": True, "2 7": False, "4 6": False, "6 6": False}
     # FP32: 162 / 222, 167 / 230
     assert d["recouple32"] == {"4 5": True, "7 4": True}
+
+
+
+CUT = r'''
+import json
+import paper_1203_2222_gb300 as P
+from paper_1203_2222_gb300 import synthetic
+
+# (L A) W by R of the fermion-parity step: four blocks of 80 x 80 by a reduction of 400, three of
+# them with signs
+r = synthetic.z2f_mps_heff(D=160)
+S = {n: P.Structure(P.Z2F, r[n]) for n in "LAWR"}
+T = P.contract_plan(S["L"], S["A"], [2], [0], P.FP64).out
+T = P.contract_plan(T, S["W"], *map(list, r["steps"][0]), P.FP64).out
+print(json.dumps(P.contract_plan(T, S["R"], *map(list, r["steps"][1]), P.FP64).block_info()))
+'''
+
+
+def test_tiles_of_one_size_are_cut_alike():
+    env = dict(os.environ, SYM_PLAN_DRYRUN="1", PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", CUT], env=env, capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 0, r.stderr
+    assert json.loads(r.stdout)["cut"] in (0, 100)
