@@ -407,7 +407,7 @@ int sym_wait_probe(int limit_us, int word);
  * column-label tuples likewise, and every tensor block is the row-major
  * sub-matrix at its tuples' first row and column.  Every M_x is decomposed
  * independently, M_x = U_x diag(S_x) V_x, in FP64 (one-sided Jacobi, one
- * cluster of 8 CTAs per block).  U(1) and fermion-parity tensors of rank
+ * cluster of 16 CTAs per block, and refinement).  U(1) and fermion-parity tensors of rank
  * >= 2 with 1 <= nrow < rank; SU(2) tensors of rank 2 (nrow = 1; the block
  * of spin x = 2j is M_x; SYM_ERR_UNSUPPORTED for higher ranks).  SU(2)
  * values and factors follow the block normalisation of the contraction
@@ -419,13 +419,14 @@ int sym_wait_probe(int limit_us, int word);
  * sym_svd_plan: plan the decomposition of tensors with T's structure:
  *   nblocks = number of diagonal blocks (labels x with rows and columns),
  *   nsv = sum over blocks of min(m_x, n_x) (the length of S).  The plan owns
- *   a workspace of about (3.5 max(m,n) + 6 min(m,n)) min(m,n) doubles per
+ *   a workspace of about (2.5 max(m,n) + 5 min(m,n)) min(m,n) doubles per
  *   block.
  * sym_svd_blocks: per block, ascending x: x, m_x, n_x (arrays of nblocks
  *   ints; any may be NULL).
  * sym_svd_execute: decompose the FP64 blocks `T` (device, T's layout).
  *   Jacobi sweeps in FP32 choose the starting point, which FP64 Newton
- *   steps (or, for blocks of less than full rank, FP64 sweeps) take to FP64
+ *   steps (or, for blocks of less than full rank or with values that decay
+ *   past about seven decades, FP64 sweeps, several times slower) take to FP64
  *   accuracy, so the result is an FP64 SVD.
  *   S (device, nsv doubles, caller-owned) receives every block's singular
  *   values in descending order, blocks in ascending x; the singular vectors

@@ -14,28 +14,30 @@
 //   not orthogonal to within sqrt(R) ulp is rotated so that they are, and the
 //   same rotation is applied to V (V = I at the start).  Blocks with at least
 //   64 columns take the pairs by column blocks, a block pair in a CTA's shared
-//   memory (jacobi_sweeps_blocked), others a warp per pair with a cluster
-//   barrier between rounds.  V is the starting point of
+//   memory through its Gram matrix (jacobi_sweeps_gram), others a warp per pair
+//   with a cluster barrier between rounds.  V is the starting point of
 // svd_av_kernel, svd_gram_kernel, svd_correction_kernel, svd_update_kernel:
 //   up to kMaxRefine Newton steps in FP64 (below), each a few products over all
 //   blocks that spread over every SM.  A V = W then has orthogonal columns: S =
 //   their norms, U = W / S.
 // svd_sweep_kernel: FP64 Jacobi sweeps for the blocks that the refinement did
-//   not finish (rank-deficient blocks, clusters).  They are bounded
-//   (kMaxSweeps); a block that has not converged by then sets the device error
-//   word to SYM_ERR_NUMERIC.
+//   not finish: values that decay past what the FP32 sweeps separate (seven decades
+//   of singular values, four to five of eigenvalues), rank-deficient blocks of an SVD,
+//   clusters.  They are bounded (kMaxSweeps); a block that has not converged by
+//   then sets the device error word to SYM_ERR_NUMERIC.
 // svd_place_kernel, svd_rank_kernel: norms, and the columns ranked by norm
 //   (descending, ties by index) into S and a permutation.
 // svd_factor_kernel: one CTA per block writes the kept singular vectors into
 //   the blocks of U (row legs, bond) and V (bond, column legs), optionally
 //   scaled by S.
 //
-// Measured (GB300, two-site tensor D = 2048: 41 blocks up to 272 x 272):
-// execute and factors 19.3 -> 6.6 ms; the two-site density matrix (42 blocks)
-// 25.6 -> 8.0 ms.  Before, two FP64 sweeps (eig: four) in serial rounds on each
-// block's own cluster took 14 ms (20 ms); the refinement takes 2.6 ms, bound
+// Measured (GB300, two-site tensor D = 2048: 41 blocks up to 272 x 272, normal
+// entries): execute and factors 19.3 -> 6.6 ms; the two-site density matrix (42
+// blocks) 25.6 -> 8.0 ms.  Before, two FP64 sweeps (eig: four) in serial rounds on
+// each block's own cluster took 14 ms (20 ms); the refinement takes 2.6 ms, bound
 // by FP64 (two multiply-adds a clock of an SM; 70% of it), the FP32 sweeps 3.8
-// to 4.7 ms, bound by the latencies of a round.
+// to 4.7 ms, bound by the latencies of a round.  Where all blocks end in FP64 sweeps,
+// the sweeps are what they were: geometric values to 1e-8 61 -> 62 ms.
 //
 // The same kernels give the blockwise eigendecomposition of a symmetric
 // tensor seen as a square matrix (Ch. 5, Eq. spectral, by blocks as the
@@ -144,11 +146,11 @@ struct SvdTile {
 
 // The parts of a block's workspace.
 struct SvdWork {
-  double *W, *V, *nrm, *Ss, *A, *G, *E, *W2, *V2;
+  double *W, *V, *nrm, *Ss, *A, *G, *E;
   float *W32, *V32, *X, *F0, *F1;
   __host__ __device__ static int64_t elems(int64_t R, int64_t C) {
     const int64_t rc = R * C, cc = C * C;
-    return 3 * rc + 4 * cc + 2 * C + (rc + 4 * cc + 1) / 2 + 1;
+    return 2 * rc + 3 * cc + 2 * C + (rc + 4 * cc + 1) / 2 + 1;
   }
   __device__ SvdWork(double* w, int64_t R, int64_t C) {
     const int64_t rc = R * C, cc = C * C;
@@ -159,9 +161,7 @@ struct SvdWork {
     A = Ss + C;
     G = A + rc;
     E = G + cc;
-    W2 = E + cc;
-    V2 = W2 + rc;
-    W32 = reinterpret_cast<float*>(V2 + cc);
+    W32 = reinterpret_cast<float*>(E + cc);
     V32 = W32 + rc;
     X = V32 + cc;
     F0 = X + cc;
@@ -1291,7 +1291,6 @@ __device__ __forceinline__ void tile_f64(const double* __restrict__ p, int64_t l
       if (ty + 8 * i < ml && tx + 16 * j < nl) store(i0 + ty + 8 * i, j0 + tx + 16 * j, acc[i][j]);
 }
 
-__device__ __forceinline__ double* refine_v(const SvdWork& ws, int step) { return step & 1 ? ws.V2 : ws.V; }
 __device__ __forceinline__ float* refine_f(const SvdWork& ws, int step) {
   return step == 0 ? ws.V32 : step & 1 ? ws.F0 : ws.F1;
 }
@@ -1307,7 +1306,7 @@ __global__ void __launch_bounds__(kTileThreads)
   const double sa = state[t.block].sa;
   const int R = b.R;
   const bool eig = b.eig != 0;
-  tile_f64<false>(ws.A, R, R, refine_v(ws, step), b.C, b.C, b.C, t.i0, t.j0, [&](int i, int j, double v) {
+  tile_f64<false>(ws.A, R, R, ws.V, b.C, b.C, b.C, t.i0, t.j0, [&](int i, int j, double v) {
     ws.W[i + (int64_t)j * R] = sa * v;
     if (!eig) ws.W32[i + (int64_t)j * R] = (float)(sa * v);
   });
@@ -1321,7 +1320,7 @@ __global__ void __launch_bounds__(kTileThreads)
   if (state[t.block].done) return;
   const SvdBlock& b = blocks[t.block];
   const SvdWork ws(work + b.w, b.R, b.C);
-  const double* V = refine_v(ws, step);
+  const double* V = ws.V;
   const int C = b.C;
   double* out = t.kind ? ws.E : ws.G;
   auto store = [&](int i, int j, double v) { out[i + (int64_t)j * C] = v; };
@@ -1426,7 +1425,8 @@ __device__ __forceinline__ bool refined(const SvdState& st, const SvdBlock& b) {
   return st.done > 0 && (b.eig || !st.nulls[st.done - 1]);
 }
 
-// V' = V + V X (kind 0), and on a block's last step W2 = W + W X (kind 1)
+// V' = V + V X (kind 0), and on a block's last step W' = W + W X (kind 1): in place,
+// since the products read the FP32 copies
 __global__ void __launch_bounds__(kTileThreads)
     svd_update_kernel(const SvdBlock* __restrict__ blocks, const SvdTile* __restrict__ tiles, double* __restrict__ work,
                       SvdState* __restrict__ state, int step) {
@@ -1443,9 +1443,8 @@ __global__ void __launch_bounds__(kTileThreads)
   if (lost || (t.kind && (!last || b.eig))) return;
   const SvdWork ws(work + b.w, b.R, b.C);
   const int C = b.C, m = t.kind ? b.R : C;
-  const double* src = t.kind ? ws.W : refine_v(ws, step);
+  double* out = t.kind ? ws.W : ws.V;
   const float* srcf = t.kind ? ws.W32 : refine_f(ws, step);
-  double* dst = t.kind ? ws.W2 : refine_v(ws, step + 1);
   float* dstf = t.kind ? nullptr : refine_f(ws, step + 1);
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int ml = min(kTile, m - t.i0), nl = min(kTile, C - t.j0);
@@ -1474,8 +1473,8 @@ __global__ void __launch_bounds__(kTileThreads)
       const int r = ty + 8 * i, c = tx + 16 * j;
       if (r >= ml || c >= nl) continue;
       const int64_t at = t.i0 + r + (int64_t)(t.j0 + c) * m;
-      const double v = src[at] + (double)acc[i][j];
-      dst[at] = v;
+      const double v = out[at] + (double)acc[i][j];
+      out[at] = v;
       if (dstf) dstf[at] = (float)v;
     }
 }
@@ -1546,12 +1545,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
     ctl.flag[0] = ctl.flag[1] = 0;
     ctl.any = 0;
   }
-  if (done > 0) {  // the refined V (in V2 after an odd number of steps) and W
-    if (done & 1)
-      for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, __ldcg(ws.V2 + i));
-    for (int64_t i = ct; i < (int64_t)R * C; i += kCT) __stcg(W + i, __ldcg(ws.W2 + i));
-    cluster.sync();
-  } else {
+  cluster.sync();  // shared state initialised before any remote access
+  if (done <= 0) {  // else the refined V and W are in place
     // two Newton-Schulz steps through the G buffer, the first one's product in
     // W's buffer (free until W = A V)
     for (int64_t i = ct; i < CC; i += kCT) __stcg(V + i, (double)__ldcg(ws.V32 + i));
@@ -1623,8 +1618,8 @@ __global__ void __cluster_dims__(kSvdCluster, 1, 1) __launch_bounds__(kSvdThread
   }
 }
 
-// Refined blocks: W (the last step's W2, scaling undone) and its column norms (as in svd_sweep_kernel),
-// and V, to their places; a warp per column.
+// Refined blocks: the scaling of W undone, and its column norms (as in
+// svd_sweep_kernel); a warp per column.
 __global__ void __launch_bounds__(256)
     svd_place_kernel(const SvdBlock* __restrict__ blocks, const int2* __restrict__ cols, int ncols,
                      double* __restrict__ work, const SvdState* __restrict__ state, int* __restrict__ sweeps) {
@@ -1639,15 +1634,13 @@ __global__ void __launch_bounds__(256)
   if (!b.eig) {
     double a = 0.0;
     for (int i = lane; i < R; i += 32) {
-      const double x = ws.W2[i + (int64_t)j * R];
+      const double x = ws.W[i + (int64_t)j * R];
       ws.W[i + (int64_t)j * R] = st.unsa * x;
       a = fma(x, x, a);
     }
     a = warp_sum(a);
     if (lane == 0) ws.nrm[j] = st.unsa * sqrt(a);
   }
-  if (st.done & 1)
-    for (int i = lane; i < C; i += 32) ws.V[i + (int64_t)j * C] = ws.V2[i + (int64_t)j * C];
   if (j == 0 && lane == 0) sweeps[2 * b.slot] = st.done;
 }
 
@@ -1807,7 +1800,7 @@ struct SvdPlan {
   bool dry = false;
   bool bonded = false;
 
-  std::vector<SvdTile> tiles[3];  // refinement products: W; the two Gram matrices; V' and W2
+  std::vector<SvdTile> tiles[3];  // refinement products: W; the two Gram matrices; V' and W'
   std::vector<int2> columns;      // (block, column)
 
   DeviceArena arena;

@@ -157,3 +157,15 @@ def test_close_and_decaying_values(n, name):
     assert np.max(np.abs(w @ w.T - np.eye(n))) <= 1e-12
     live = s > 1e-10 * s[0]
     assert np.max(np.abs(u[:, live].T @ u[:, live] - np.eye(live.sum()))) <= 1e-12
+
+
+def test_workspace_is_bounded():
+    """7.5 n^2 doubles a square block: V and W are refined where they are."""
+    n = 3000
+    S = P.Structure(P.U1, [([0], [n], 1), ([0], [n], -1)])
+    P.svd_plan(P.Structure(P.U1, [([0], [8], 1), ([0], [8], -1)]), 1)  # whatever a first plan sets up
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    plan = P.svd_plan(S, 1)
+    assert free - torch.cuda.mem_get_info()[0] <= 8.4 * n * n * 8
+    del plan
