@@ -497,25 +497,19 @@ WORKLOADS = {"u1_mps_heff": MPSWorkload, "su2_recouple": SU2Workload, "u1_two_si
 # the captured launches, applied to the full launch's algorithmic bytes.
 TRAFFIC = {
     "u1_mps_heff": {  # profiles/traffic_u1_mps_heff.md
-        "gemm_tc": {"bytes_per_launch": 13768640, "sha": "e8b8ba59c26dc3b8"},
+        "gemm_tc": {"bytes_per_launch": 13768640, "sha": "c2195c1e91557657"},
         "box_flat": {"bytes_per_launch": 5856928, "sha": "b2745455cd736886"},
         "box": {"bytes_per_launch": 13080064, "sha": "b2745455cd736886"},
         "direct": {"bytes_per_launch": 11909291, "sha": "a481e530fd08e2e9"},
     },
     "su2_recouple": {  # profiles/gemm_tc_su2_recouple.md (full size, forward and backward launches)
-        "gemm_tc": {"bytes_per_launch": 61145753344, "sha": "e8b8ba59c26dc3b8"},
+        "gemm_tc": {"bytes_per_launch": 61145753344, "sha": "c2195c1e91557657"},
     },
     "u1_two_site_batch": {  # profiles/direct_u1_two_site_batch.md (128 of the 512 problems)
         "direct": {"ratio": 0.96, "sha": "a481e530fd08e2e9"},
     },
-    "u1_two_site_svd": {  # profiles/svd_u1_two_site_svd.md (full size, mean of 11 launches)
-        "svd_jacobi": {"bytes_per_launch": 9013271, "sha": "96f8106d63b42dfd"},
-    },
-    "u1_two_site_eig": {  # profiles/eig_u1_two_site_eig.md (full size, mean of 11 launches)
-        "svd_jacobi": {"bytes_per_launch": 8889972, "sha": "96f8106d63b42dfd"},
-    },
     "z2f_mps_heff": {  # profiles/traffic_z2f_mps_heff_and_mera.md (full size, mean of 62 step launches)
-        "gemm_tc": {"bytes_per_launch": 196322104, "sha": "e8b8ba59c26dc3b8"},
+        "gemm_tc": {"bytes_per_launch": 196322104, "sha": "c2195c1e91557657"},
     },
     "u1_mera_grad": {  # profiles/traffic_z2f_mps_heff_and_mera.md (full size, mean of 663 launches)
         "box_flat": {"bytes_per_launch": 2139167, "sha": "b2745455cd736886"},
@@ -523,11 +517,10 @@ TRAFFIC = {
 }
 KERNEL_SOURCES = {
     "box": ["box.cu", "kernels.h", "pdl.h"], "box_flat": ["box.cu", "kernels.h", "pdl.h"],
-    "gemm_tc": ["gemm_tc.cu", "kernels.h", "pdl.h"],
+    "gemm_tc": ["gemm_tc.cu", "pdl.h"],  # of kernels.h only the layout of its work items
     "gemm_tile": ["gemm_simt.cu", "kernels.h", "pdl.h"], "gemm_wide": ["gemm_simt.cu", "kernels.h", "pdl.h"],
     "gemm_thin": ["gemm_simt.cu", "kernels.h", "pdl.h"], "gemm_rows": ["gemm_simt.cu", "kernels.h", "pdl.h"],
     "direct": ["direct.cu", "kernels.h", "pdl.h"], "block": ["block.cu", "kernels.h", "pdl.h"],
-    "svd_jacobi": ["svd.cu"],
 }
 
 
@@ -1057,8 +1050,12 @@ def run_svd(args, rank, world):
     ms_per_step = ms / args.steps
     value = whole_job_rate(1.0, args.steps, world, ms)
 
-    # per-kernel device times (the same launches, timed one by one)
-    kms = {"svd_jacobi": 0.0, "svd_factor": 0.0}
+    # device times of the step's two parts (the same launches): execute (the
+    # FP32 sweeps, the FP64 refinement and sweeps, the ranking) and the factors
+    execute = ("svd_jacobi_kernel; 5 x svd_av, svd_gram, svd_correction, svd_update_kernel; "
+               "svd_sweep, svd_place, svd_rank_kernel")
+    kms = {"svd_execute": 0.0, "svd_factor": 0.0}
+    symbols = {"svd_execute": (execute, 24), "svd_factor": ("svd_factor_kernel", 1)}  # kernels, launches a step
     for _ in range(args.steps):
         flush.fill_(1.0)
         e0, e1, e2 = (torch.cuda.Event(enable_timing=True) for _ in range(3))
@@ -1068,22 +1065,22 @@ def run_svd(args, rank, world):
         plan.factors(absorb)
         e2.record(stream)
         torch.cuda.synchronize()
-        kms["svd_jacobi"] += e0.elapsed_time(e1)
+        kms["svd_execute"] += e0.elapsed_time(e1)
         kms["svd_factor"] += e1.elapsed_time(e2)
     f64, f32 = plan.flops()
     sweeps64, _ = plan.stats()
     sweeps32, _ = plan.stats(fp32=True)
-    kernels = {k: {"symbol": k + "_kernel", "launches": args.steps, "ms": round(v, 4),
+    kernels = {k: {"symbol": symbols[k][0], "launches": symbols[k][1] * args.steps, "ms": round(v, 4),
                    "share": round(v / max(sum(kms.values()), 1e-12), 4)} for k, v in kms.items()}
-    jac_s = kms["svd_jacobi"] * 1e-3 / args.steps
+    exec_s = kms["svd_execute"] * 1e-3 / args.steps
     mhz = clk.get("sm_mhz") or 2070.0
     peak64 = 152 * FP64_FLOPS_PER_SM_CLK * mhz * 1e6 / 1e12
     peak32 = 152 * FP32_FLOPS_PER_SM_CLK * mhz * 1e6 / 1e12
-    roof = {"bound": "alu", "kernel": "svd_jacobi", "symbol": "svd_jacobi_kernel",
-            "achieved": round(f64 / jac_s / 1e12, 5), "peak": round(peak64, 4), "unit": "TFLOP/s",
-            "frac": round(f64 / jac_s / 1e12 / peak64, 4), "traffic": svd_traffic(args.workload),
-            "algorithmic_per_launch": f64, "fp32_flops_per_launch": f32,
-            "avg_launch_us": round(jac_s * 1e6, 2), "launches_timed": args.steps,
+    roof = {"bound": "alu", "kernel": "svd_execute", "symbol": execute,
+            "achieved": round(f64 / exec_s / 1e12, 5), "peak": round(peak64, 4), "unit": "TFLOP/s",
+            "frac": round(f64 / exec_s / 1e12 / peak64, 4), "traffic": None,
+            "algorithmic_per_execute": f64, "fp32_flops_per_execute": f32,
+            "avg_execute_us": round(exec_s * 1e6, 2), "launches_timed": 24 * args.steps,
             "peak_source": "FP64 ALU: 152 SMs x 4 flops/clk (1.25 TFLOP/s nominal at 2070 MHz) x sampled SM clock",
             "sweeps_fp64_max": max(sweeps64), "sweeps_fp32_max": max(sweeps32)}
     # the step's floor: FP64 flops at the FP64 peak plus FP32 flops at the FP32 peak
@@ -1143,11 +1140,6 @@ def run_svd(args, rank, world):
     vals_gpu = plan.execute(T.data).cpu().numpy()  # every block's values, for the oracle's comparison
     torch.cuda.synchronize()
     return out, (plan.labels, plan.m if is_eig else [min(a, b) for a, b in zip(plan.m, plan.n)], vals_gpu)
-
-
-def svd_traffic(workload="u1_two_site_svd"):
-    t = TRAFFIC[workload]["svd_jacobi"]
-    return t["bytes_per_launch"] if t["sha"] == kernel_source_sha("svd_jacobi") else None
 
 
 def _oracle_svd_step(w, To):
