@@ -65,6 +65,9 @@ bool pack(const Dims& x, int32_t* sizes, uint32_t* mag, int* shf, int32_t* ostr)
 // ones, FP64 two operations a clock, multiply-adds and the products with the
 // coefficients alike, over the live part of the tile; a slab's round trip
 // about 700 clocks; 2500 clocks of set-up and stores, shared by the CTAs of an SM.
+// FP32 products with coefficients count in the two large shapes, which multiply-adds
+// bound; the small one waits for its loads (with a quarter more there too, an SU(2)
+// recoupling contraction that takes 150 us on the blocks went to its matrix form, 209).
 // kModelScale: measured over modelled time, 1.5 to 1.6 on the contractions of
 // the U(1) and SU(2) x U(1) MPS step (D = 2048, 1024) and of the MERA patch;
 // FP64 0.9 to 1.2 (those steps, D = 128 to 1500, and SU(2) recoupling contractions).
@@ -85,7 +88,7 @@ Cost tile_cost(bool f64, int shape, int64_t m, int64_t n, int64_t k, bool coef) 
     const double fma = 64.0 * (lm * ln + (coef ? ln : 0.0)) * (double)k * 1.1;  // four warps' operations, 16 clocks each
     return {fma + 500.0, fma + slabs * 700.0 + 2500.0};
   }
-  const double fma = (coef && shape != BLK_TALL ? 1.25 : 1.0) * (double)TM * TN * (double)k / 128.0 /
+  const double fma = (coef && shape <= BLK_MID ? 1.25 : 1.0) * (double)TM * TN * (double)k / 128.0 /
                      (shape == BLK_BIG ? 0.6 : shape == BLK_MID ? 0.5 : shape == BLK_SMALL ? 0.35 : 0.16);
   return {fma + slabs * 60.0 + 500.0, std::max(fma, slabs * 700.0) + 2500.0};
 }

@@ -28,7 +28,7 @@ def recouple(d, j, prec=P.FP64):
 print(json.dumps({"f64": {d: product(d, P.FP64) for d in (128, 512, 1024)},
                   "f32": {d: product(d, P.BF16X3) for d in (128, 512, 1024)},
                   "recouple": {f"{d} {j}": recouple(d, j) for d, j in ((2, 4), (3, 3), (2, 7), (4, 6), (6, 6))},
-                  "recouple32": {f"{d} {j}": recouple(d, j, P.BF16X3) for d, j in ((4, 5), (7, 4))}}))
+                  "recouple32": {f"{d} {j}": recouple(d, j, P.BF16X3) for d, j in ((4, 5), (5, 5), (7, 4))}}))
 '''
 
 
@@ -43,8 +43,8 @@ def test_form_of_clear_cases():
     assert d["f32"] == {"128": True, "512": False, "1024": False}
     # SU(2) recoupling: 190 / 235, 173 / 225; 412, 600 and 1000 in matrix form
     assert d["recouple"] == {"2 4": True, "3 3": True, "2 7": False, "4 6": False, "6 6": False}
-    # FP32: 162 / 222, 167 / 230
-    assert d["recouple32"] == {"4 5": True, "7 4": True}
+    # FP32: 162 / 222, 150 / 209, 167 / 230
+    assert d["recouple32"] == {"4 5": True, "5 5": True, "7 4": True}
 
 
 
