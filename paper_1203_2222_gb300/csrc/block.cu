@@ -21,15 +21,17 @@
 // vector to keep the transposing writes apart); FP64 tiles stride their
 // microtile so that rows and columns past the block's edge are skipped whole
 // -- an FP64 multiply-add costs a warp 16 clocks.
-// Measured (GB300, eager, forward and gradients unless said; before: the
-// matrix form): two small rank-4 U(1) tensors 224 -> 161 us; U(1) MPS step D =
-// 2048 433 -> 325 us, 35 -> 8 launches (its four block launches take 40 to 84
-// us, bound by the shared-memory pipe: l1tex 75% busy, FP32 multiply-adds a
-// quarter of the instructions); SU(2) x U(1) MPS step 525 -> 307 us, 32 -> 6
-// launches; MERA patch 1.70 -> 1.46 ms, 98 -> 38; FP64 MPS apply D = 768 543 ->
-// 143 us (tiles small enough for 152 SMs).  64 threads with an 8 x 8 microtile
-// (12 warps an SM) took 104 us a launch instead of 67, a persistent CTA with
-// the next tile's descriptors prefetched 69.
+// Measured (GB300, the passes of perf/cases.py through the public API, launches
+// and host time included; before: the matrix form): two small rank-4 U(1) tensors
+// 263 -> 155 us; U(1) MPS step D = 2048 541 -> 366 us, 35 -> 8 launches; SU(2) x
+// U(1) MPS step 551 -> 309 us, 32 -> 6 launches; MERA patch 2.04 -> 1.42 ms, 98 ->
+// 38; FP64 MPS apply D = 768 543 -> 121 us (tiles small enough for 152 SMs).  The
+// U(1) step's block launches take 44 and 71 us forward, 116 and 82 backward, bound
+// by the shared-memory pipe (l1tex 75% busy, FP32 multiply-adds a quarter of the
+// instructions); the matrix form's launches take 31 and 30, 41 and 50 us on the
+// device, so a captured call takes those (plan.cpp).  64 threads with an 8 x 8
+// microtile (12 warps an SM) took 104 us a launch instead of 67, a persistent CTA
+// with the next tile's descriptors prefetched 69.
 // Outputs of at most 8 x 8 with a long reduction (the gradient of a small
 // operator, a scalar) take a thread per reduction step instead.
 #include <cuda_runtime.h>
